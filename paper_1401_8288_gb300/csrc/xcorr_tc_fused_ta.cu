@@ -123,7 +123,7 @@ struct TItem {
   const CUtensorMap* map;  // raw input
   int2* out;
   int64_t n_pairs;
-  int c, I, J, n_inputs, n_kt, accumulate;
+  int c, I, J, n_inputs, n_kt;
   int t_first;             // first sample of the item
   int ax, ay, bx, by;      // TMA coordinates (input or channel-input column, channel) of the row and column tiles
   bool diag, valid;
@@ -142,7 +142,6 @@ __device__ __forceinline__ TItem resolve(const TParams& p, const CUtensorMap* ma
     it.n_pairs = s->n_pairs;
     it.n_inputs = s->n_inputs;
     it.n_kt = s->n_kt;
-    it.accumulate = s->accumulate;
     it.c = static_cast<int>(w.y);
     it.I = static_cast<int>(w.z);
     it.J = static_cast<int>(w.w);
@@ -152,7 +151,6 @@ __device__ __forceinline__ TItem resolve(const TParams& p, const CUtensorMap* ma
     it.out = p.out;
     it.n_pairs = p.n_pairs;
     it.n_inputs = p.n_inputs;
-    it.accumulate = p.accumulate;
     int tile = item;
     it.n_kt = p.n_kt;
     it.t_first = p.t0;
@@ -196,7 +194,13 @@ __device__ __forceinline__ void prefetch_item_stage(const TItem& it, int s) {
 // of a phase-2 load) land in opposite halves of each eight-chunk group.
 __device__ __forceinline__ int staging_swizzle(int row) { return ((row & 1) << 2) | ((row >> 1) & 3); }
 
-template <int KT, int RAW, int DEC, bool BATCH, bool SMALL, bool PACK>
+// ADD: the launch adds into out with plain loads and stores (else it stores, or adds with atomics).  An
+// added pair costs a load that waits for L2 or HBM; issued one by one between the stores these made an
+// adding launch 7x slower than a storing one (1125 us against 154 us at 1024 inputs x 64 channels x 1024
+// samples).  With a chunk's sixteen loads in flight together the epilogue stays beside the next tile
+// pair's MMAs: 216 us for the same launch.  A kernel of its own, so that the storing launch carries none of the loads
+// registers (0.3 % at 512 inputs when it did).
+template <int KT, int RAW, int DEC, bool BATCH, bool SMALL, bool PACK, bool ADD>
 __global__ void __launch_bounds__(kThreads, 1)
     xcorr_tc_fused_ta_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ TParams p) {
   using G = TGeom<KT, RAW, DEC>;
@@ -521,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int2* out_c = it.out + (int64_t)c * it.n_pairs;
       const int row0 = I * kBlk + warp * 32;
       const int buf = g & 1;
-      if (!SMALL && it.accumulate) {
+      if (ADD && !SMALL) {
         // the sums this tile pair adds to, pulled into L2 while its MMAs run: each thread
         // prefetches the 128-byte lines of its own row's segment (pairs J*128 .. min(J*128 + 127, i))
         const int i = I * kBlk + r_own;
@@ -606,6 +610,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int4 s0 = *reinterpret_cast<const int4*>(cs + jc);  // (8P, 8Q) of columns jc, jc + 1
         const int4 s1 = *reinterpret_cast<const int4*>(cs + jc + 8);
         const int sp[4] = {s0.x, s0.z, s1.x, s1.z}, sq[4] = {s0.y, s0.w, s1.y, s1.w};
+        int2 old[4][4];  // the chunk's earlier sums
+        if (ADD) {
+#pragma unroll
+          for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int j = jc + 8 * (k >> 1) + (k & 1);
+              old[m][k] = row_out[m] != nullptr && j <= lastm[m] && j >= firstm[m] ? row_out[m][j - firstm[m]]
+                                                                                   : make_int2(0, 0);
+            }
+        } else {
+#pragma unroll
+          for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) old[m][k] = make_int2(0, 0);
+        }
         tmem_ld_wait();
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
@@ -633,13 +653,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 nr = __float2int_rn(__uint_as_float(xr) * 262144.0f);
                 ni = __float2int_rn(__uint_as_float(xi) * 262144.0f);
               }
-              v[e] = make_int2(nr + rcm[m].x - sp[2 * jj + e], -ni + rcm[m].y + sq[2 * jj + e]);
+              v[e] = make_int2(nr + rcm[m].x - sp[2 * jj + e] + old[m][2 * jj + e].x,
+                               -ni + rcm[m].y + sq[2 * jj + e] + old[m][2 * jj + e].y);
             }
             // (first is a multiple of 16 and j0 even: a pair of columns starts inside the row or before it)
             if (j0 > last || j0 < first) continue;
             int2* dst = row_out[m] + (j0 - first);
             const int nv = j0 + 1 <= last ? 2 : 1;
-            if (SMALL && p.atomic_out) {  // time-split items of one tile add into the same pairs
+            if (SMALL && !ADD && p.atomic_out) {  // time-split items of one tile add into the same pairs
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 if (e < nv) {
@@ -648,25 +669,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
               }
             } else if (nv == 2 && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-              int4 w = make_int4(v[0].x, v[0].y, v[1].x, v[1].y);
-              if (it.accumulate) {
-                const int4 o = *reinterpret_cast<const int4*>(dst);
-                w = make_int4(w.x + o.x, w.y + o.y, w.z + o.z, w.w + o.w);
-              }
-              *reinterpret_cast<int4*>(dst) = w;
+              *reinterpret_cast<int4*>(dst) = make_int4(v[0].x, v[0].y, v[1].x, v[1].y);
             } else {
 #pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                if (e < nv) {
-                  int2 w = v[e];
-                  if (it.accumulate) {
-                    const int2 o = dst[e];
-                    w.x += o.x;
-                    w.y += o.y;
-                  }
-                  dst[e] = w;
-                }
-              }
+              for (int e = 0; e < 2; ++e)
+                if (e < nv) dst[e] = v[e];
             }
           }
         }
@@ -685,10 +692,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-template <int KT, int RAW, int DEC, bool BATCH = false, bool SMALL = false, bool PACK = false>
-cudaError_t launch_ta(const CUtensorMap& raw_map, const TParams& p, int grid, cudaStream_t stream) {
+template <int KT, int RAW, int DEC, bool BATCH, bool SMALL, bool PACK, bool ADD>
+cudaError_t launch_ta_kernel(const CUtensorMap& raw_map, const TParams& p, int grid, cudaStream_t stream) {
   using G = TGeom<KT, RAW, DEC>;
-  auto kern = xcorr_tc_fused_ta_kernel<KT, RAW, DEC, BATCH, SMALL, PACK>;
+  auto kern = xcorr_tc_fused_ta_kernel<KT, RAW, DEC, BATCH, SMALL, PACK, ADD>;
   static int attr_device = -1;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -700,6 +707,13 @@ cudaError_t launch_ta(const CUtensorMap& raw_map, const TParams& p, int grid, cu
   }
   kern<<<grid, kThreads, G::kSmem, stream>>>(raw_map, p);
   return cudaGetLastError();
+}
+
+template <int KT, int RAW, int DEC, bool BATCH = false, bool SMALL = false, bool PACK = false>
+cudaError_t launch_ta(const CUtensorMap& raw_map, const TParams& p, int grid, cudaStream_t stream) {
+  if (!BATCH && p.accumulate && !p.atomic_out)
+    return launch_ta_kernel<KT, RAW, DEC, false, SMALL, PACK, !BATCH>(raw_map, p, grid, stream);
+  return launch_ta_kernel<KT, RAW, DEC, BATCH, SMALL, PACK, false>(raw_map, p, grid, stream);
 }
 
 }  // namespace

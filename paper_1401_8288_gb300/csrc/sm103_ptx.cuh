@@ -344,6 +344,23 @@ __device__ __forceinline__ void mma_pair_f8f6f4_ta(uint32_t d_tmem, uint32_t a_t
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate));
 }
 
+// As mma_pair_f8f6f4_ta with A in shared memory: each CTA's 128 rows at the same offset.
+// ESIZE 1: kind::f8f6f4 operands, 2: kind::f16.
+template <int ESIZE>
+__device__ __forceinline__ void mma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                         uint32_t accumulate) {
+  if (ESIZE == 1)
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+  else
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+}
+
 // Arrive on `bar` in both CTAs (the same offset) once the pair's MMAs issued so far are complete.
 __device__ __forceinline__ void mma_pair_commit_both(uint64_t* bar) {
   asm volatile(

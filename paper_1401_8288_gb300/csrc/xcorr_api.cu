@@ -74,6 +74,8 @@ void release(xcorr_plan plan) {
   if (plan->planes) cudaFree(plan->planes);
   if (plan->exps) cudaFree(plan->exps);
   plan->exps = nullptr;
+  if (plan->ring_flags) cudaFree(plan->ring_flags);
+  plan->ring_flags = nullptr;
   if (plan->status) cudaFree(plan->status);
   if (plan->status_host) cudaFreeHost(plan->status_host);
   plan->acc = nullptr;
@@ -155,6 +157,28 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     e = xc::launch_xcorr_tc_fused_ci4(static_cast<const uint8_t*>(d_in), C, plan->tune_variant, n_time, C, N,
                                       static_cast<int2*>(target), !target_fresh, plan->status, plan->num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "fused X kernel launch");
+    if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
+    if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
+  } else if (plan->pair) {
+    // one launch on the caller's stream: unpack warps feed the CTA pairs through the ring
+    if (ev && ((e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventRecord(ev[2], s)) != cudaSuccess))
+      return cuda_fail(e, "profile event");
+    xc::PairLaunch L;
+    L.fmt = plan->cfg.fmt;
+    L.in = d_in;
+    L.n_time = n_time;
+    L.n_chan = C;
+    L.n_inputs = N;
+    L.accumulate = !target_fresh;
+    L.out = target;
+    L.status = plan->status;
+    L.ring = &plan->ring;
+    L.ring_mem = plan->planes;
+    L.flags = plan->ring_flags;
+    L.exps = plan->exps;
+    L.exp_windows = plan->exp_windows;
+    L.exp_pitch = plan->ni_pad;
+    if ((e = xc::launch_xcorr_tc_pair(L, s)) != cudaSuccess) return cuda_fail(e, "CTA-pair X kernel launch");
     if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
     if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
   } else if (plan->engine == XCORR_ENGINE_TENSOR) {
@@ -318,13 +342,26 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   const int elem_bytes = c.fmt == XCORR_IN_CI4 ? 1 : 2;
   const int ppc = c.fmt == XCORR_IN_CF32 ? 6 : 2;
   const size_t acc_bytes = (size_t)c.n_channels * (size_t)n_pairs * 8;
-  const size_t planes_bytes = engine == XCORR_ENGINE_TENSOR ? (size_t)c.n_channels * ppc *
-                                                                  (size_t)c.max_time_per_exec * ni_pad * elem_bytes
-                                                            : 0;
+  // three or more 128-input tiles run on CTA pairs from a small ring of planes; smaller problems
+  // stage all their planes
+  const bool pair = engine == XCORR_ENGINE_TENSOR && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles;
+  size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !pair ? (size_t)c.n_channels * ppc *
+                                                                     (size_t)c.max_time_per_exec * ni_pad * elem_bytes
+                                                               : 0;
   const int exp_windows = (c.max_time_per_exec + xc::kTcWindowBF16 - 1) / xc::kTcWindowBF16;
-  const size_t exps_bytes =
-      (engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CF32) ? (size_t)c.n_channels * exp_windows * ni_pad * 2 : 0;
-  const size_t dev_bytes = acc_bytes + planes_bytes + exps_bytes + 256;
+  // (+ 256: the drain reads a tile's 128 column exponents past the last row's ni_pad)
+  const size_t exps_bytes = (engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CF32)
+                                ? (size_t)c.n_channels * exp_windows * ni_pad * 2 + 256
+                                : 0;
+  xc::PairRing ring;
+  if (pair) {
+    const size_t other = acc_bytes + exps_bytes + 256;
+    const size_t room = c.hbm_budget_bytes > other ? c.hbm_budget_bytes - other : 1;
+    e = xc::pair_ring_layout(c.fmt, n_inputs, c.n_channels, c.max_time_per_exec, c.hbm_budget_bytes ? room : 0, &ring);
+    if (e != cudaSuccess) return cuda_fail(e, "ring layout");
+    planes_bytes = ring.bytes;
+  }
+  const size_t dev_bytes = acc_bytes + planes_bytes + ring.flag_bytes + exps_bytes + 256;
   if (c.hbm_budget_bytes && dev_bytes > c.hbm_budget_bytes)
     return fail(XCORR_ERR_BUDGET, "plan needs " + std::to_string(dev_bytes) + " device bytes, budget is " +
                                       std::to_string(c.hbm_budget_bytes));
@@ -344,6 +381,8 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   plan->device_bytes = dev_bytes;
   plan->elem_bytes = elem_bytes;
   plan->planes_per_chan = ppc;
+  plan->pair = pair;
+  plan->ring = ring;
   plan->window_samples = c.fmt == XCORR_IN_CI4 ? xc::kTcWindowCI4 : xc::kTcWindowBF16;
   plan->exp_windows = exp_windows;
   // 4-bit input starts on the fused kernel with the A operand in tensor memory (the fastest
@@ -357,6 +396,7 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   if ((e = cudaMalloc(&plan->acc, acc_bytes)) != cudaSuccess ||
       (planes_bytes && (e = cudaMalloc(&plan->planes, planes_bytes)) != cudaSuccess) ||
       (exps_bytes && (e = cudaMalloc(&plan->exps, exps_bytes)) != cudaSuccess) ||
+      (pair && (e = cudaMalloc(&plan->ring_flags, ring.flag_bytes)) != cudaSuccess) ||
       (e = cudaMalloc(&plan->status, 256)) != cudaSuccess ||
       (e = cudaMallocHost(&plan->status_host, sizeof(int))) != cudaSuccess) {
     release(plan);
@@ -377,6 +417,15 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
       release(plan);
       delete plan;
       return cuda_fail(e, "stream or event creation");
+    }
+  }
+  if (pair) {
+    // the planes' columns past n_inputs are read but never written: any finite number will do
+    if ((e = cudaMemset(plan->planes, 0, ring.bytes)) != cudaSuccess ||
+        (e = cudaMemset(plan->ring_flags, 0, ring.flag_bytes)) != cudaSuccess) {
+      release(plan);
+      delete plan;
+      return cuda_fail(e, "ring initialisation");
     }
   }
   if (plan->exps && (e = cudaMemset(plan->exps, 0, exps_bytes)) != cudaSuccess) {
@@ -611,10 +660,11 @@ xcorr_status xcorr_plan_query(xcorr_plan plan, xcorr_plan_info* info) {
   const bool fused = plan->engine == XCORR_ENGINE_TENSOR && plan->cfg.fmt == XCORR_IN_CI4 && !plan->tune_unfused &&
                      plan->n_inputs % 16 == 0;
   info->kernels_per_execute = fused ? xc::fused_launches(plan->cfg.max_time_per_exec)
+                              : plan->pair                          ? 1
                               : plan->engine == XCORR_ENGINE_TENSOR ? 2 * tensor_groups(plan)
                                                                      : 1;
   info->tuning.stage_variant = plan->tune_variant;
-  info->tuning.groups = fused ? 1 : tensor_groups(plan);
+  info->tuning.groups = fused || plan->pair ? 1 : tensor_groups(plan);
   info->tuning.x_streams = plan->tune_x_streams;
   info->tuning.unfused = plan->tune_unfused;
   return XCORR_OK;
@@ -670,6 +720,7 @@ xcorr_status xcorr_autotune(xcorr_plan plan, const void* d_in, int n_time, void*
       for (int xs = 1; xs <= 2 && st == XCORR_OK; ++xs) {
         if (group_choices[gi] == 1 && xs == 2) continue;  // one group has one X launch
         if (uf == 0 && (gi > 0 || xs > 1)) continue;      // the fused kernel is one launch
+        if (uf == 1 && plan->pair && (v > 0 || gi > 0)) continue;  // so is the CTA-pair kernel, of one shape
         plan->tune_variant = v;
         plan->tune_groups = group_choices[gi];
         plan->tune_x_streams = xs;

@@ -64,6 +64,20 @@ enum ExecMode : int { MODE_STORE = 0, MODE_ADD = 1, MODE_ATOMIC = 2 };
 constexpr int kMaxGroups = 8;
 constexpr int kProfileEvents = 2 + 2 * kMaxGroups;  // per timed execute
 
+// The whole tensor path in one launch on CTA pairs (xcorr_tc_pair.cu), for three or more 128-input
+// tiles: samples unpacked once into a ring of operand planes, correlated from it.
+constexpr int kTcPairMinTiles = 3;
+constexpr size_t kRingBytes = size_t(48) << 20;  // of the 129 MB L2
+struct PairRing {
+  int clusters = 0;      // CTA pairs of a launch
+  int halves = 0;        // 64-input halves of a plane: two per tile
+  int chunk = 0;         // samples per slot
+  int batch_chans = 0;   // channel places of a batch (one entry per cluster) in the unpack order
+  int slots = 0;
+  int places = 0;        // flags of each kind
+  size_t slot_bytes = 0, bytes = 0, flag_bytes = 0;
+};
+
 }  // namespace xc
 
 struct xcorr_plan_s {
@@ -101,6 +115,11 @@ struct xcorr_plan_s {
   CUtensorMap tmap{};          // planes, for tmap_ntime / tmap_variant
   int tmap_ntime = -1;
   int tmap_variant = -1;
+
+  // CTA-pair path (pair): planes is its ring
+  bool pair = false;
+  xc::PairRing ring;
+  int* ring_flags = nullptr;
 
   // internal streams of the tensor path (forked from and joined to the caller's stream)
   cudaStream_t s_unpack = nullptr;
@@ -179,6 +198,23 @@ cudaError_t launch_xcorr_tc_fused_ta_batch(const TaSubDesc* subs, const uint4* i
 cudaError_t launch_xcorr_tc_batch(const void* subs, const uint4* items, int n_items, int variant, int* status,
                                   int num_sms, cudaStream_t stream);
 cudaError_t launch_xcorr_tc(const CUtensorMap* tmap, const TcLaunch& launch, cudaStream_t stream);
+
+// The ring for executes of up to max_time samples, within most_bytes (0: no limit) where possible.
+cudaError_t pair_ring_layout(int fmt, int n_inputs, int n_chan, int max_time, size_t most_bytes, PairRing* ring);
+struct PairLaunch {
+  int fmt = 0;
+  const void* in = nullptr;  // [t][c][i] samples, any alignment (float: 4 bytes)
+  int n_time = 0, n_chan = 0, n_inputs = 0;
+  bool accumulate = false;   // add into out (else store)
+  void* out = nullptr;       // int2 or float2 [C][P]
+  int* status = nullptr;
+  const PairRing* ring = nullptr;
+  void* ring_mem = nullptr;
+  int* flags = nullptr;      // ring->flag_bytes, zero before the first launch
+  int16_t* exps = nullptr;   // float input: window exponents [C][exp_windows][exp_pitch]
+  int exp_windows = 0, exp_pitch = 0;
+};
+cudaError_t launch_xcorr_tc_pair(const PairLaunch& launch, cudaStream_t stream);
 
 cudaError_t launch_xcorr_cuda_core(int fmt, const void* in, int n_time, int n_chan, int n_inputs,
                                    int2* acc, int mode, int ksplit, cudaStream_t stream);

@@ -9,12 +9,11 @@
 // the X kernel reads them as MN-major operands, so the tensor memory access
 // itself performs the transpose of the corner turn and this kernel is a pure
 // element-wise decode with 128-bit loads and stores.
-#include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
 #include <cstring>
 
-#include "ci4_decode.cuh"
+#include "unpack_device.cuh"
 #include "xcorr_internal.h"
 
 namespace xc {
@@ -296,53 +295,6 @@ __global__ void __launch_bounds__(256) unpack_ci8_bf16_elem(const int8_t* __rest
     dst[0] = static_cast<uint16_t>(bf16_bits(static_cast<float>(in[2 * s])));
     dst[comp_stride] = static_cast<uint16_t>(bf16_bits(static_cast<float>(in[2 * s + 1])));
   }
-}
-
-// Float input, one thread per (channel, window, input): find the window's
-// largest magnitude max < 2^(E+1), quantise each component to the integer
-// M = rint(x 2^(22-E)) (|M| < 2^23, error <= 2^-23 max), and write the
-// balanced base-256 digits of M = d0 2^16 + d1 2^8 + d2 (|d_p| <= 128, exact
-// BF16 values) to planes re_p = p and im_p = 3 + p.  E goes to exps.
-//
-// Edges.  The maximum is taken over the components' bit patterns with the
-// sign cleared: for non-negative floats they order as the values do, and the
-// patterns of infinities and NaNs lie above every finite one, so one integer
-// maximum also finds a non-finite sample.  Such a window gets E =
-// kExpNonFinite and zero digits; the X kernel's drain turns every block that
-// involves it into NaN.  A window whose maximum is subnormal gets that
-// maximum's own exponent (down to -149), so its samples keep 23-bit integers
-// like any other window's and no finite input is flushed.  2^(22-E) spans
-// 2^-105 .. 2^171, past the float range, so it is applied as two exact
-// power-of-two factors.
-__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
-
-__device__ __forceinline__ int window_exponent(uint32_t max_bits) {
-  if (max_bits >= 0x7F800000u) return kExpNonFinite;
-  if (max_bits >= 0x00800000u) return static_cast<int>(max_bits >> 23) - 127;  // normal
-  if (max_bits == 0u) return kExpMin;
-  return (31 - __clz(static_cast<int>(max_bits))) - 149;  // subnormal m 2^-149: floor(log2 m) - 149
-}
-
-// The two factors of 2^(22 - e), each in [2^-53, 2^86]; zero for a non-finite window.
-__device__ __forceinline__ void window_scale(int e, float& s1, float& s2) {
-  if (e == kExpNonFinite) {
-    s1 = s2 = 0.f;
-    return;
-  }
-  const int n = 22 - e, a = n >> 1;
-  s1 = pow2i(a);
-  s2 = pow2i(n - a);
-}
-
-__device__ __forceinline__ void digits_of(float x, float s1, float s2, uint16_t (&d)[3]) {
-  const int m = __float2int_rn((x * s1) * s2);
-  const int d2 = ((m + 128) & 255) - 128;
-  const int m1 = (m - d2) >> 8;
-  const int d1 = ((m1 + 128) & 255) - 128;
-  const int d0 = (m1 - d1) >> 8;
-  d[0] = __bfloat16_as_ushort(__float2bfloat16_rn(static_cast<float>(d0)));
-  d[1] = __bfloat16_as_ushort(__float2bfloat16_rn(static_cast<float>(d1)));
-  d[2] = __bfloat16_as_ushort(__float2bfloat16_rn(static_cast<float>(d2)));
 }
 
 // Any 4-byte aligned input: the components are read as single floats.

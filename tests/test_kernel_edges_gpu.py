@@ -32,3 +32,138 @@ def test_adding_launch_of_the_fused_kernel(torch, variant, n_sta, n_chan, n_time
         got = plan.dump().cpu().numpy()
         plan.sync()
     assert np.array_equal(got.astype(np.int64), oracle.correlate(oracle.FMT_CI4, x))
+
+
+# ------------------------------------------------ the CTA-pair kernel over its ring of planes ---
+# Three or more 128-input tiles: every tile count's grouping (an odd one leaves a CTA without a row
+# tile, transposed tile pairs), input counts that end inside a tile and inside 16, samples that end
+# inside a stage (64 / 32), a chunk (512 / 256 / 384) and an exact window, few and many channels.
+PAIR_SIZES = [(129, 1, 1), (130, 3, 65), (169, 5, 513), (192, 2, 385), (200, 3, 700), (256, 2, 1100), (320, 1, 130),
+              (331, 2, 96)]
+
+
+def draw(fmt, n_time, n_chan, n_sta, seed):
+    if fmt == "ci4":
+        return synth.uniform_ci4(n_time, n_chan, n_sta, seed=seed, lo=-8, hi=7)
+    if fmt == "ci8":
+        return synth.uniform_ci8(n_time, n_chan, n_sta, seed=seed)
+    return synth.gaussian_cf32(n_time, n_chan, n_sta, seed=seed)
+
+
+def placed(torch, x, offset):
+    """x on the device, its first byte `offset` bytes past a 16-byte boundary."""
+    flat = torch.from_numpy(np.ascontiguousarray(x)).view(torch.uint8).reshape(-1).cuda()
+    buf = torch.zeros(flat.numel() + 64, dtype=torch.uint8, device="cuda")
+    buf[offset:offset + flat.numel()] = flat
+    assert buf.data_ptr() % 16 == 0
+    return buf
+
+
+def check(fmt, got, x, n_in):
+    want = oracle.correlate({"ci4": oracle.FMT_CI4, "ci8": oracle.FMT_CI8, "cf32": oracle.FMT_CF32}[fmt], x)
+    if fmt != "cf32":
+        assert np.array_equal(got.astype(np.int64), want)
+        return
+    # the float path's tolerance: 1e-6 of sqrt(V_ii V_jj) per entry
+    i = np.arange(n_in)
+    autos = want[:, i * (i + 1) // 2 + i, 0]
+    ii, jj = np.tril_indices(n_in)
+    scale = np.sqrt(autos[:, ii] * autos[:, jj])
+    err = np.abs((got[..., 0] - want[..., 0]) + 1j * (got[..., 1] - want[..., 1]))
+    assert (err <= 1e-6 * scale).all()
+
+
+@pytest.mark.parametrize("fmt", ["ci4", "ci8", "cf32"])
+@pytest.mark.parametrize("n_sta,n_chan,n_time", PAIR_SIZES)
+def test_pair_ring_kernel(torch, fmt, n_sta, n_chan, n_time):
+    x = draw(fmt, n_time, n_chan, n_sta, seed=n_sta + n_time)
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor") as plan:
+        plan.set_tuning(0, 0, 1, 1)
+        out = torch.full((n_chan, plan.info["n_pairs"], 2), -1, device="cuda",
+                         dtype=torch.float32 if fmt == "cf32" else torch.int32)
+        plan.execute_dump(torch.from_numpy(x).cuda(), out)
+        plan.sync()
+    check(fmt, out.cpu().numpy(), x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("fmt,offset", [("ci4", 1), ("ci4", 6), ("ci8", 3), ("ci8", 2), ("cf32", 4), ("cf32", 8)])
+@pytest.mark.parametrize("n_sta", [160, 135, 129, 192])
+def test_pair_ring_kernel_reads_any_alignment(torch, fmt, offset, n_sta):
+    x = draw(fmt, 150, 3, n_sta, seed=offset)
+    buf = placed(torch, x, offset)
+    with xcorr.Plan(n_sta, 3, 150, fmt=fmt, engine="tensor") as plan:
+        xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, 150, torch.cuda.current_stream().cuda_stream)
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check(fmt, got, x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("fmt,n_chan,n_time", [("ci4", 200, 600), ("ci8", 130, 300), ("cf32", 60, 800)])
+def test_pair_ring_kernel_refills_its_ring(torch, fmt, n_chan, n_time):
+    """More chunks than ring slots, over three adding executes of different lengths."""
+    n_sta = 129
+    x = draw(fmt, 2 * n_time + 40, n_chan, n_sta, seed=11)
+    parts = [x[:n_time], x[n_time:n_time + 40], x[n_time + 40:]]
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor") as plan:
+        plan.set_tuning(0, 0, 1, 1)
+        for part in parts:
+            plan.execute(torch.from_numpy(np.ascontiguousarray(part)).cuda())
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check(fmt, got, x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("fmt", ["ci8", "cf32"])
+def test_pair_ring_kernel_in_graphs_and_on_two_streams(torch, fmt):
+    """A captured execute replays on new data; two plans on two streams do not wait for each other."""
+    n_sta, n_chan, n_time = 136, 4, 200
+    xs = [draw(fmt, n_time, n_chan, n_sta, seed=s) for s in (1, 2)]
+    xd = [torch.from_numpy(x).cuda() for x in xs]
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt) as plan, xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt) as other:
+        out = plan.execute_dump(xd[0])
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        buf = xd[0].clone()
+        with torch.cuda.graph(graph):
+            plan.execute_dump(buf, out)
+        for k in (1, 0):
+            buf.copy_(xd[k])
+            out.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            check(fmt, out.cpu().numpy(), xs[k], 2 * n_sta)
+        streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+        outs = [torch.zeros_like(out) for _ in range(2)]
+        torch.cuda.synchronize()
+        for _ in range(5):
+            for k, pl in enumerate((plan, other)):
+                pl.execute_dump(xd[k], outs[k], stream=streams[k])
+        torch.cuda.synchronize()
+        plan.sync()
+        other.sync()
+        for k in range(2):
+            check(fmt, outs[k].cpu().numpy(), xs[k], 2 * n_sta)
+
+
+def test_pair_ring_kernel_float_edges(torch):
+    """Windows past the drain's fast range (powers 2^90 apart), an all-zero input, one NaN."""
+    n_sta, n_chan, n_time = 130, 2, 500
+    x = synth.gaussian_cf32(n_time, n_chan, n_sta, seed=3)
+    x[:, :, 5] *= np.float32(2.0**50)
+    x[:, :, 9] *= np.float32(2.0**-40)
+    x[:, 1, 40, 1] = 0
+    clean = oracle.correlate(oracle.FMT_CF32, x)
+    x[450, 0, 100, 0, 1] = np.nan
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="cf32") as plan:
+        got = plan.execute_dump(torch.from_numpy(x).cuda()).cpu().numpy()
+        plan.sync()
+    n_in = 2 * n_sta
+    ii, jj = np.tril_indices(n_in)
+    bad = np.zeros((n_chan, ii.size), dtype=bool)
+    bad[0] = (ii == 200) | (jj == 200)
+    assert np.array_equal(np.isnan(got[..., 0]), bad) and np.array_equal(np.isnan(got[..., 1]), bad)
+    i = np.arange(n_in)
+    autos = clean[:, i * (i + 1) // 2 + i, 0]
+    scale = np.sqrt(autos[:, ii] * autos[:, jj])
+    err = np.abs((got[..., 0] - clean[..., 0]) + 1j * (got[..., 1] - clean[..., 1]))
+    assert (err[~bad] <= 1e-6 * scale[~bad]).all()

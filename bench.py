@@ -75,7 +75,9 @@ KERNEL_SOURCES = {
     "xcorr_tc_fused_ta_kernel": ("xcorr_tc_fused_ta.cu", "fused_common.cuh", "sm103_ptx.cuh", "xcorr_internal.h"),
     "xcorr_tc_fused_kernel": ("xcorr_tc_fused.cu", "fused_common.cuh", "sm103_ptx.cuh", "xcorr_internal.h"),
     "xcorr_tc_kernel": ("xcorr_tc.cu", "sm103_ptx.cuh", "xcorr_internal.h"),
-    "xcorr_tc_pair_kernel": ("xcorr_tc_pair.cu", "unpack_device.cuh", "ci4_decode.cuh", "fused_pairing.h",
+    "xcorr_tc_raw_pair_kernel": ("xcorr_tc_raw_pair.cu", "pair_common.cuh", "fused_pairing.h", "sm103_ptx.cuh",
+                                 "xcorr_internal.h"),
+    "xcorr_tc_pair_kernel": ("pair_common.cuh","xcorr_tc_pair.cu", "unpack_device.cuh", "ci4_decode.cuh", "fused_pairing.h",
                              "sm103_ptx.cuh", "xcorr_internal.h"),
 }
 FUSED_TA_VARIANTS = (4, 5, 6, 10)  # tuning stage_variants served by the tensor-memory-A fused kernel
@@ -604,8 +606,9 @@ def our_arm(args) -> int:
     fused_ta = fused and tuning["stage_variant"] in FUSED_TA_VARIANTS
     fused_pair = fused and tuning["stage_variant"] in FUSED_PAIR_VARIANTS
     x_kernel = (("xcorr_tc_fused_pair_kernel" if fused_pair else "xcorr_tc_fused_ta_kernel" if fused_ta
-                 else "xcorr_tc_fused_kernel") if fused else "xcorr_tc_pair_kernel" if n_sta > 128 else "xcorr_tc_kernel")
-    one_launch = fused or n_sta > 128  # else unpack + X per channel group
+                 else "xcorr_tc_fused_kernel") if fused else "xcorr_tc_raw_pair_kernel" if fmt == "ci8"
+                else "xcorr_tc_pair_kernel" if n_sta > 64 else "xcorr_tc_kernel")
+    one_launch = fused or fmt == "ci8" or n_sta > 64  # else unpack + X per channel group
     x_launches = launches_per_step if one_launch else launches_per_step // 2
     out_dtype = torch.float32 if fmt == "cf32" else torch.int32
     out = torch.empty((n_chan, n_pairs, 2), dtype=out_dtype, device=dev)
@@ -786,8 +789,9 @@ def our_arm(args) -> int:
                                       "correction, int32 out)") if fused else
                                      ("tcgen05 kind::f8f6f4 (E4M3 codes of 4-bit integers, exact "
                                       "FP32 TMEM sums drained to int32)"),
-                              "ci8": "tcgen05 kind::f16 (BF16 copies of int8 values, exact FP32 "
-                                     "sums drained to int32 every 512 samples, 384 up to 256 inputs)",
+                              "ci8": "tcgen05 kind::f16 cta_group::2 on SM pairs, int8 values "
+                                     "decoded on chip to F16, exact FP32 sums drained to int32 every 512 "
+                                     "samples",
                               "cf32": "tcgen05 kind::f16 (three BF16 pieces per value, six piece "
                                       "products, FP32 sums drained every 384 samples)"}[fmt],
                    "tuning": tuning,

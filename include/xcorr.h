@@ -109,7 +109,7 @@ typedef struct xcorr_plan_s *xcorr_plan;
 
 /* Launch shape of the tensor-core path (xcorr_plan_set_tuning, xcorr_autotune). */
 typedef struct {
-    int stage_variant;  /* shared-memory ring, 0 .. 10: planes path of up to 256 inputs 0 = 3 x 64 KB,
+    int stage_variant;  /* shared-memory ring, 0 .. 10: planes path of up to 128 inputs 0 = 3 x 64 KB,
                            1 (and 3 .. 10) = 4 x 48 KB, 2 = 6 x 32 KB stages (more inputs: one
                            launch on CTA pairs with one shape); fused path see `unfused`       */
     int groups;         /* channel groups whose unpack overlaps the X kernel; 0 = automatic (<= 8) */
@@ -129,7 +129,7 @@ typedef struct {
                            side in one 128-row tile; and when a launch has fewer tiles
                            than SMs, each tile's stages split over several CTAs whose
                            sums are added atomically into the (cleared) output;
-                           1 = always through E4M3 planes (in HBM up to 256 inputs; a ring of
+                           1 = always through E4M3 planes (in HBM up to 128 inputs; a ring of
                            them that stays in L2 beyond)                                    */
 } xcorr_tuning;
 
@@ -152,7 +152,7 @@ typedef struct {
  * staging buffers on the current device (the plan owns them), and selects the
  * kernels.  *out receives the plan, or NULL on failure.
  * Engines: TENSOR uses the tcgen05 kernels for every format (4-bit as E4M3,
- * int8 as BF16, float as three BF16 pieces); CUDA_CORE takes CI4 / CI8; AUTO
+ * int8 as F16 or BF16, float as three BF16 pieces); CUDA_CORE takes CI4 / CI8; AUTO
  * takes CUDA_CORE for at most 16 channels with fewer than 16 inputs (CI4) or at
  * most 64 inputs (CI8), where its single launch was measured faster than the
  * tensor path's unpack + X, and TENSOR otherwise.  A 4-bit tensor plan starts on

@@ -121,6 +121,11 @@ bool fused_applies(xcorr_plan plan, const void* d_in) {
          reinterpret_cast<uintptr_t>(d_in) % 16 == 0;
 }
 
+// int8 input that is decoded on chip: one launch, no planes.
+bool raw_ci8_applies(xcorr_plan plan, const void* d_in) {
+  return plan->cfg.fmt == XCORR_IN_CI8 && plan->engine == XCORR_ENGINE_TENSOR && xc::raw_pair_takes(plan->n_inputs, d_in);
+}
+
 // Unpack channels [c0, c0 + nc) of the input into the plan's planes.
 cudaError_t unpack_group(xcorr_plan plan, const void* d_in, int n_time, int c0, int nc, cudaStream_t s) {
   const int C = plan->cfg.n_channels, N = plan->n_inputs, T = plan->cfg.max_time_per_exec;
@@ -157,6 +162,15 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     e = xc::launch_xcorr_tc_fused_ci4(static_cast<const uint8_t*>(d_in), C, plan->tune_variant, n_time, C, N,
                                       static_cast<int2*>(target), !target_fresh, plan->status, plan->num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "fused X kernel launch");
+    if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
+    if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
+  } else if (raw_ci8_applies(plan, d_in)) {
+    // int8 input decoded on chip: one launch on the caller's stream
+    if (ev && ((e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventRecord(ev[2], s)) != cudaSuccess))
+      return cuda_fail(e, "profile event");
+    e = xc::launch_xcorr_tc_raw_pair(static_cast<const int8_t*>(d_in), n_time, C, N, static_cast<int2*>(target),
+                                     !target_fresh, plan->status, plan->num_sms, s);
+    if (e != cudaSuccess) return cuda_fail(e, "CTA-pair X kernel launch");
     if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
     if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
   } else if (plan->pair) {
@@ -342,8 +356,8 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   const int elem_bytes = c.fmt == XCORR_IN_CI4 ? 1 : 2;
   const int ppc = c.fmt == XCORR_IN_CF32 ? 6 : 2;
   const size_t acc_bytes = (size_t)c.n_channels * (size_t)n_pairs * 8;
-  // three or more 128-input tiles run on CTA pairs from a small ring of planes; smaller problems
-  // stage all their planes
+  // two or more 128-input tiles run on CTA pairs from a small ring of planes; smaller problems stage
+  // all their planes
   const bool pair = engine == XCORR_ENGINE_TENSOR && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles;
   size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !pair ? (size_t)c.n_channels * ppc *
                                                                      (size_t)c.max_time_per_exec * ni_pad * elem_bytes
@@ -420,8 +434,8 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
     }
   }
   if (pair) {
-    // the planes' columns past n_inputs are read but never written: any finite number will do
-    if ((e = cudaMemset(plan->planes, 0, ring.bytes)) != cudaSuccess ||
+    // a last tile's inputs past n_inputs are read but never written: any finite number will do
+    if ((n_inputs % 128 && (e = cudaMemset(plan->planes, 0, ring.bytes)) != cudaSuccess) ||
         (e = cudaMemset(plan->ring_flags, 0, ring.flag_bytes)) != cudaSuccess) {
       release(plan);
       delete plan;
@@ -659,12 +673,14 @@ xcorr_status xcorr_plan_query(xcorr_plan plan, xcorr_plan_info* info) {
   info->output_bytes = (size_t)plan->cfg.n_channels * plan->n_pairs * 8;
   const bool fused = plan->engine == XCORR_ENGINE_TENSOR && plan->cfg.fmt == XCORR_IN_CI4 && !plan->tune_unfused &&
                      plan->n_inputs % 16 == 0;
+  // (int8: a 16-byte aligned input, nullptr standing for one)
+  const bool one_launch = plan->pair || raw_ci8_applies(plan, nullptr);
   info->kernels_per_execute = fused ? xc::fused_launches(plan->cfg.max_time_per_exec)
-                              : plan->pair                          ? 1
+                              : one_launch                          ? 1
                               : plan->engine == XCORR_ENGINE_TENSOR ? 2 * tensor_groups(plan)
                                                                      : 1;
   info->tuning.stage_variant = plan->tune_variant;
-  info->tuning.groups = fused || plan->pair ? 1 : tensor_groups(plan);
+  info->tuning.groups = fused || one_launch ? 1 : tensor_groups(plan);
   info->tuning.x_streams = plan->tune_x_streams;
   info->tuning.unfused = plan->tune_unfused;
   return XCORR_OK;
@@ -720,7 +736,8 @@ xcorr_status xcorr_autotune(xcorr_plan plan, const void* d_in, int n_time, void*
       for (int xs = 1; xs <= 2 && st == XCORR_OK; ++xs) {
         if (group_choices[gi] == 1 && xs == 2) continue;  // one group has one X launch
         if (uf == 0 && (gi > 0 || xs > 1)) continue;      // the fused kernel is one launch
-        if (uf == 1 && plan->pair && (v > 0 || gi > 0)) continue;  // so is the CTA-pair kernel, of one shape
+        // so are the CTA-pair kernels, of one shape each
+        if (uf == 1 && (plan->pair || raw_ci8_applies(plan, d_in)) && (v > 0 || gi > 0)) continue;
         plan->tune_variant = v;
         plan->tune_groups = group_choices[gi];
         plan->tune_x_streams = xs;

@@ -64,9 +64,9 @@ enum ExecMode : int { MODE_STORE = 0, MODE_ADD = 1, MODE_ATOMIC = 2 };
 constexpr int kMaxGroups = 8;
 constexpr int kProfileEvents = 2 + 2 * kMaxGroups;  // per timed execute
 
-// The whole tensor path in one launch on CTA pairs (xcorr_tc_pair.cu), for three or more 128-input
+// The whole tensor path in one launch on CTA pairs (xcorr_tc_pair.cu), for two or more 128-input
 // tiles: samples unpacked once into a ring of operand planes, correlated from it.
-constexpr int kTcPairMinTiles = 3;
+constexpr int kTcPairMinTiles = 2;
 constexpr size_t kRingBytes = size_t(48) << 20;  // of the 129 MB L2
 struct PairRing {
   int clusters = 0;      // CTA pairs of a launch
@@ -288,6 +288,15 @@ int fused_pair_stage_samples(int variant);
 cudaError_t launch_xcorr_tc_fused_pair_ci4(const uint8_t* in, int row_chans, int variant, int n_time, int n_chan,
                                            int n_inputs, int2* out, bool accumulate, int* status, int num_sms,
                                            cudaStream_t stream);
+
+// Tensor map over an int8 input [t][c][i][2] in boxes of 64 inputs x 1 channel x box_t samples (128-byte
+// swizzle); n_inputs a multiple of 8, a 16-byte aligned pointer.
+bool encode_raw_ci8_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_chan, int n_time, int box_t,
+                         std::string* err);
+// The X-stage on CTA pairs with int8 samples decoded on chip (xcorr_tc_raw_pair.cu): one launch.
+bool raw_pair_takes(int n_inputs, const void* in);
+cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int n_time, int n_chan, int n_inputs, int2* out, bool accumulate,
+                                     int* status, int num_sms, cudaStream_t stream);
 
 // int8 (re, im) samples -> two BF16 planes [c][2][t][ni_pad] (exact).
 cudaError_t launch_unpack_ci8_bf16(const int8_t* in, uint16_t* planes, int n_time, int n_chan, int c0,

@@ -7,7 +7,7 @@
 // Sec. 1, Sec. 2.1, Eq. 1; the unpack and corner turn of Sec. 2.4): 4-bit
 // samples as E4M3 planes, int8 as BF16 planes, float as six BF16 planes of
 // integer digits with one exponent per (channel, 384-sample window, input).
-// For problems of three or more 128-input tiles.
+// For problems of two or more 128-input tiles.
 //
 // Why one launch.  Unpacking to planes in HBM writes 2 (4-bit), 4 (int8) or 12
 // (float) bytes per sample that the X kernel reads back: as much time as the
@@ -49,14 +49,16 @@
 // resident), so they always end; like all waits here they are bounded
 // (sm103_ptx.cuh).  The last CTA to leave clears the flags.
 //
-// Measured (one GB300): 512 inputs x 256 channels x 4096 samples, int8 1.00 ms (1.32 ms for unpack +
-// planes kernel), float 5.2-5.8 ms (7.2-7.3); 338 inputs x 97 channels x 1500, 4-bit, 129 us (252).
+// Measured (one GB300), against unpack + planes kernel: 512 inputs x 256 channels x 4096 samples, float
+// 5.2-5.8 ms (7.2-7.3), int8 1.00 ms (1.32); 338 inputs x 97 channels x 1500, 4-bit, 129 us (252); two
+// tiles: 256 inputs x 256 channels x 2048, float, 1.22 ms (1.40), 250 x 300 x 2048, 4-bit, 355 us (670).
 // A step takes 272 cycles with the MMAs alone, 307-318 from a ring that nobody refills (about 40
 // bytes per cycle and SM from L2, the rate every form of these loads stopped at), 450-470 beside the
-// unpack, which alone would take 250-330.  The rule: three or more tiles, where pairing wastes no
-// tile pair; two tiles (three tile pairs) would leave a quarter of the pairs' rows idle, one tile has
-// nothing to share.  Aligned 4-bit input stays with the fused kernel (497 us against about 600 us
-// here at 512 inputs x 512 channels x 2048 samples): its L2 traffic is the raw bytes.
+// unpack, which alone would take 250-330.  The rule: two or more tiles.  With one tile half of every
+// pair's rows are idle, and the planes kernel wins once there are channels for every SM (128 inputs x
+// 300 channels x 4096, float: 1.11 ms against 1.29 here).  Aligned 4-bit input stays with the fused
+// kernel (497 us against about 600 us here at 512 inputs x 512 channels x 2048 samples: its L2 traffic
+// is the raw bytes), aligned int8 input goes to xcorr_tc_raw_pair.cu (0.87 ms against 1.00).
 //
 // Warp roles (512 threads, one CTA per SM): warps 0-7 drain TMEM into running
 // sums held in registers (warp w: lane quarter w % 4, columns 64 (w / 4) ..
@@ -67,20 +69,16 @@
 // the drain of one block overlap the MMAs of the next.
 #include <type_traits>
 
-#include "fused_pairing.h"
-#include "sm103_ptx.cuh"
+#include "pair_common.cuh"
 #include "unpack_device.cuh"
 #include "xcorr_internal.h"
 
 namespace xc {
 namespace {
 
+using namespace pairs;
 using fused::pair_entries;
-using fused::pair_entry;
 
-constexpr int kBlk = 128;          // inputs per tile side
-constexpr int kHalf = 64;          // column-tile inputs each CTA loads
-constexpr int kEpiWarps = 8;       // two per TMEM lane quarter, 64 columns each
 constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp = 9;
 constexpr int kNegWarp0 = 10;
@@ -88,16 +86,10 @@ constexpr int kNegWarps = 2;
 constexpr int kUnpackWarp0 = 12;
 constexpr int kUnpackWarps = 4;
 constexpr int kThreads = (kUnpackWarp0 + kUnpackWarps) * 32;
-constexpr int kCols = 64;          // tile columns held per epilogue thread (its row)
-constexpr int kChunk = 8;          // columns per shared-memory transpose step
-constexpr int kPitch = kChunk + 1; // 8-byte words per staged row
-constexpr int kAccCols = 256;      // [Re | X] of columns 0-63, [Re | X] of columns 64-127
-constexpr uint32_t kTmemCols = 512;
-constexpr int kStagingBytes = kEpiWarps * 32 * kPitch * 8;
-constexpr int kFactorBytes = kEpiWarps * kCols * 4;  // float input: column factors of a window
+constexpr int kFactorBytes = kEpiWarps * kHalf * 4;  // float input: column factors of a window
 constexpr int kStages = 6;         // of 28 KB: finer stages cover the copies' latency better than 3 x 56 KB
 constexpr int kRowsPerTask = 32;   // an unpack sub-task (integer formats): 32 samples of one channel x
-constexpr int kColsPerTask = 4;    // 4 columns of 128 bytes of raw samples
+constexpr int kHalfPerTask = 4;    // 4 columns of 128 bytes of raw samples
 constexpr int kFetchGroups = 3;    // groups of raw copies in flight per unpack warp
 constexpr int kFetchRows = 16;     // samples per group: 4 copies of 16 bytes per lane (4 samples x 8 units a warp)
 // raw samples on their way to the unpack warps: per lane and copy 16 bytes, and for the last unit of a
@@ -105,7 +97,6 @@ constexpr int kFetchRows = 16;     // samples per group: 4 copies of 16 bytes pe
 constexpr int kFetchSlots = kUnpackWarps * 32 * 4 * kFetchGroups;
 constexpr int kFetchBytes = kFetchSlots * 16 + kFetchSlots / 8 * 4;
 constexpr int kBarrierBytes = 512;
-constexpr uint32_t kSignalBytes = 16;
 constexpr int kSinkSlots = kNegWarps + kEpiWarps;  // one per signalling warp of the odd CTA
 // int8: sums of 512 samples reach at most 2 * 128^2 * 512 = 2^24, still exact in FP32
 constexpr int kWindowCI8 = 512;
@@ -135,7 +126,7 @@ struct Geom {
   static_assert(kPlane % 1024 == 0, "swizzle atoms stay aligned");
   static_assert(kRows % kFetchRows == 0 && kRowsPerTask % kFetchRows == 0, "a group of copies lies in one stage");
   // (a float window has at least 2 x 32 / 16 = 4 groups)
-  static_assert(kFetchGroups < 4 && kFetchGroups < kColsPerTask * (kRowsPerTask / kFetchRows),
+  static_assert(kFetchGroups < 4 && kFetchGroups < kHalfPerTask * (kRowsPerTask / kFetchRows),
                 "the copies in flight reach at most into the next sub-task");
   static_assert(kPlane % (kNegWarps * 32 * 16) == 0, "the negation's passes are whole");
   static_assert((3 * kStages + 5) * 8 + 8 + 16 + 16 * kSinkSlots + 16 <= kBarrierBytes, "barrier area");
@@ -177,22 +168,6 @@ struct P2Params {
   int16_t* exps;         // float input: window exponents [C][exp_windows][exp_pitch]
   int exp_windows, exp_pitch;
 };
-
-struct P2Item {
-  int chan, S, R;  // channel, column tile, this CTA's row tile (-1: none)
-  bool has_row, transposed;
-};
-
-__device__ __forceinline__ P2Item item_of(const P2Params& p, int q, uint32_t rank) {
-  P2Item it;
-  it.chan = q / p.n_entries;
-  int r0, r1;
-  pair_entry(p.nb, q - it.chan * p.n_entries, it.S, r0, r1);
-  it.R = rank == 0 ? r0 : r1;
-  it.has_row = it.R >= 0;
-  it.transposed = it.has_row && it.R < it.S;
-  return it;
-}
 
 // Place of (batch, chunk, channel of the batch) in the unpack order.
 __device__ __forceinline__ int place_of(const P2Params& p, int batch, int chunk, int j) {
@@ -302,7 +277,7 @@ __device__ __forceinline__ void group_at(const P2Params& p, int sub, int g, int&
   } else {
     constexpr int kPer = kRowsPerTask / kFetchRows;
     row = g % kPer * kFetchRows;
-    col = sub % p.col_splits * kColsPerTask + g / kPer;
+    col = sub % p.col_splits * kHalfPerTask + g / kPer;
   }
 }
 
@@ -369,7 +344,7 @@ __device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, i
   constexpr bool FLOAT = FMT == XCORR_IN_CF32;
   const int n_places = p.n_batches * p.n_chunks * p.batch_chans;
   const int n_warps = static_cast<int>(gridDim.x) * kUnpackWarps;
-  const int n_groups = FLOAT ? 2 * (p.chunk / kFetchRows) : kColsPerTask * (kRowsPerTask / kFetchRows);
+  const int n_groups = FLOAT ? 2 * (p.chunk / kFetchRows) : kHalfPerTask * (kRowsPerTask / kFetchRows);
   uint4* buf = reinterpret_cast<uint4*>(fetch) + uw * (kFetchGroups * 128) + lane;
   uint32_t* buf_w = reinterpret_cast<uint32_t*>(fetch + kFetchSlots * 16) + uw * (kFetchGroups * 16) + (lane >> 3);
   const int row_lane = lane >> 3, unit_lane = lane & 7;
@@ -551,8 +526,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   if (warp < kEpiWarps) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
     using Acc = typename std::conditional<FLOAT_OUT, float, int>::type;
-    uint2* stage_rows = staging + warp * 32 * kPitch;
-    float* col_f = factors + warp * kCols;
+    uint2* stage_rows = staging + warp * 32 * kOutPitch;
+    float* col_f = factors + warp * kHalf;
     const int quarter = warp & 3, colh = warp >> 2;
     const uint32_t tempty_even = smem_cluster(tempty, 0);
     const uint32_t sink_even = smem_cluster(sink + kSignalBytes * (kNegWarps + warp), 0);
@@ -560,14 +535,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     int g = 0;
     bool ok = true;
     for (int q = cl; ok && q < n_items; q += n_cl) {
-      const P2Item it = item_of(p, q, rank);
+      const Item it = item_of(p.nb, p.n_entries, q, rank);
       uint2* out_c = static_cast<uint2*>(p.out) + (int64_t)it.chan * p.n_pairs;
       const int row0 = it.R * kBlk + quarter * 32;  // first global row of this warp
-      const int col0 = it.S * kBlk + colh * kCols;  // first global column of this warp
+      const int col0 = it.S * kBlk + colh * kHalf;  // first global column of this warp
       const bool live = it.has_row && row0 < n_inputs && col0 < n_inputs && (it.transposed || col0 <= row0 + 31);
-      Acc acc_re[kCols], acc_im[kCols];
+      Acc acc_re[kHalf], acc_im[kHalf];
 #pragma unroll
-      for (int k = 0; k < kCols; ++k) acc_re[k] = acc_im[k] = Acc(0);
+      for (int k = 0; k < kHalf; ++k) acc_re[k] = acc_im[k] = Acc(0);
       // float input: the window's exponents of this lane's row and, for the slow path, its columns
       const int16_t* exps_w = nullptr;
       int e_row = 0;
@@ -580,7 +555,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
         tc_fence_after();
         const uint32_t taddr =
-            tmem + (static_cast<uint32_t>(quarter * 32) << 16) + buf * kAccCols + colh * 2 * kCols;
+            tmem + (static_cast<uint32_t>(quarter * 32) << 16) + buf * kAccCols + colh * 2 * kHalf;
         if (FLOAT_OUT) {
           // a block's exact integer sums times 2^k, k = E_i + E_j - 12 - 8(p + q).  While every
           // exponent of the window's rows and columns lies in [-45, 45] (kept per window), 2^k is a
@@ -604,10 +579,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           if (fast) {
             const float rf = pow2i(row_k);
 #pragma unroll
-            for (int k = 0; k < kCols / 8; ++k) {
+            for (int k = 0; k < kHalf / 8; ++k) {
               uint32_t re[8], nim[8];
               tmem_ld8(taddr + 8 * k, re);
-              tmem_ld8(taddr + kCols + 8 * k, nim);
+              tmem_ld8(taddr + kHalf + 8 * k, nim);
               const float4 f0 = *reinterpret_cast<const float4*>(col_f + 8 * k);
               const float4 f1 = *reinterpret_cast<const float4*>(col_f + 8 * k + 4);
               const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
@@ -623,10 +598,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           } else {
             const bool row_bad = e_row == kExpNonFinite;
 #pragma unroll
-            for (int k = 0; k < kCols / 8; ++k) {
+            for (int k = 0; k < kHalf / 8; ++k) {
               uint32_t re[8], nim[8];
               tmem_ld8(taddr + 8 * k, re);
-              tmem_ld8(taddr + kCols + 8 * k, nim);
+              tmem_ld8(taddr + kHalf + 8 * k, nim);
               tmem_ld_wait();
               if (!live) continue;
 #pragma unroll
@@ -643,10 +618,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
         } else {
 #pragma unroll
-          for (int k = 0; k < kCols / 8; ++k) {
+          for (int k = 0; k < kHalf / 8; ++k) {
             uint32_t re[8], nim[8];
             tmem_ld8(taddr + 8 * k, re);
-            tmem_ld8(taddr + kCols + 8 * k, nim);
+            tmem_ld8(taddr + kHalf + 8 * k, nim);
             tmem_ld_wait();
             if (!live) continue;
 #pragma unroll
@@ -668,90 +643,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
       }
       if (!ok || !live) continue;
-      if (it.transposed) {
-        // V[b][a] = conj(W[a][b]): the warp's 32 values of output row b are consecutive; row b + 1
-        // starts b + 1 pairs after row b
-        uint2* row = out_c + (int64_t)col0 * (col0 + 1) / 2 + row0 + lane;
-        int len = col0 + 1;
+      RowsOut ro;
+      ColsOut co;
+      if (it.transposed)
+        cols_out(co, out_c, row0, col0, n_inputs, lane);
+      else
+        rows_out(ro, out_c, row0, col0, n_inputs, lane);
 #pragma unroll
-        for (int ch = 0; ch < kCols / 8; ++ch) {
-          uint2* dst[8];
-          uint2 old[8];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            dst[k] = row;
-            row += len++;
-            old[k] = ADD && col0 + ch * 8 + k < n_inputs ? *dst[k] : make_uint2(0u, 0u);
-          }
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const Acc vr = acc_re[ch * 8 + k], vi = -acc_im[ch * 8 + k];
-            uint2 v;
-            if (FLOAT_OUT)
-              v = make_uint2(__float_as_uint(ADD ? vr + __uint_as_float(old[k].x) : vr),
-                             __float_as_uint(ADD ? vi + __uint_as_float(old[k].y) : vi));
-            else
-              v = make_uint2(static_cast<uint32_t>(vr) + old[k].x, static_cast<uint32_t>(vi) + old[k].y);
-            if (col0 + ch * 8 + k < n_inputs) *dst[k] = v;
-          }
-        }
-        continue;
-      }
-      // Per 8-column step a quarter-warp writes 8 consecutive pairs of one row (64 bytes); when
-      // adding, all loads of the lane are in flight together.  The row addresses are made once, and a
-      // tile wholly below the diagonal and inside the inputs takes no comparisons: index arithmetic
-      // per step made the write-out longer than a 2048-sample tile's MMAs.
-      const int sub = lane >> 3, col = lane & 7;
-      uint2* dst[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const int i = row0 + 4 * r + sub;
-        dst[r] = out_c + (int64_t)i * (i + 1) / 2 + col0 + col;
-      }
-      const bool whole = col0 + kCols - 1 <= row0 && row0 + 31 < n_inputs;
-#pragma unroll
-      for (int ch = 0; ch < kCols / kChunk; ++ch) {
-#pragma unroll
-        for (int k = 0; k < kChunk; ++k) {
-          const Acc vr = acc_re[ch * kChunk + k], vi = acc_im[ch * kChunk + k];
-          stage_rows[lane * kPitch + k] = FLOAT_OUT
-                                              ? make_uint2(__float_as_uint(vr), __float_as_uint(vi))
-                                              : make_uint2(static_cast<uint32_t>(vr), static_cast<uint32_t>(vi));
-        }
-        __syncwarp();
-        const int j = col0 + ch * kChunk + col;
+      for (int ch = 0; ch < kHalf; ch += 8) {
         uint2 v[8];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) v[r] = stage_rows[(4 * r + sub) * kPitch + col];
-        if (ADD) {
-          uint2 old[8];
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const int i = row0 + 4 * r + sub;
-            old[r] = whole || (i < n_inputs && j <= i) ? dst[r][ch * kChunk] : make_uint2(0u, 0u);
-          }
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            if (FLOAT_OUT) {
-              v[r].x = __float_as_uint(__uint_as_float(v[r].x) + __uint_as_float(old[r].x));
-              v[r].y = __float_as_uint(__uint_as_float(v[r].y) + __uint_as_float(old[r].y));
-            } else {
-              v[r].x += old[r].x;
-              v[r].y += old[r].y;
-            }
-          }
+        for (int k = 0; k < 8; ++k) {
+          const Acc vr = acc_re[ch + k], vi = it.transposed ? -acc_im[ch + k] : acc_im[ch + k];
+          v[k] = FLOAT_OUT ? make_uint2(__float_as_uint(vr), __float_as_uint(vi))
+                           : make_uint2(static_cast<uint32_t>(vr), static_cast<uint32_t>(vi));
         }
-        if (whole) {
-#pragma unroll
-          for (int r = 0; r < 8; ++r) dst[r][ch * kChunk] = v[r];
-        } else {
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const int i = row0 + 4 * r + sub;
-            if (i < n_inputs && j <= i) dst[r][ch * kChunk] = v[r];
-          }
-        }
-        __syncwarp();
+        if (it.transposed)
+          put_cols<FLOAT_OUT, ADD>(co, v);
+        else
+          put_rows<FLOAT_OUT, ADD>(ro, stage_rows, v, ch, lane);
       }
     }
   } else if (warp < kUnpackWarp0) {
@@ -767,7 +677,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         int pend = -1, pend_n = 0;  // a chunk read but not yet reported, and the stage count at its end
         bool ok = true;
         for (int q = cl, batch = 0; ok && q < n_items; q += n_cl, ++batch) {
-          const P2Item it = item_of(p, q, rank);
+          const Item it = item_of(p.nb, p.n_entries, q, rank);
           const int j = it.chan - (batch * n_cl) / p.n_entries;
           const uint32_t bytes = (it.has_row ? 4 * G::kPlane : 0) + 2 * G::kPlane;
           for (int k = 0; ok && k < p.n_chunks; ++k) {
@@ -1067,7 +977,7 @@ cudaError_t launch_xcorr_tc_pair(const PairLaunch& L, cudaStream_t stream) {
   p.row_bytes = L.n_inputs * in_bytes;
   p.row_step = static_cast<int64_t>(L.n_chan) * p.row_bytes;
   p.unit_cols = (p.row_bytes + 127) / 128;
-  p.col_splits = (p.unit_cols + kColsPerTask - 1) / kColsPerTask;
+  p.col_splits = (p.unit_cols + kHalfPerTask - 1) / kHalfPerTask;
   p.subs = L.fmt == XCORR_IN_CF32 ? p.unit_cols : (r.chunk + kRowsPerTask - 1) / kRowsPerTask * p.col_splits;
   p.ring = static_cast<uint8_t*>(L.ring_mem);
   p.ready = L.flags;

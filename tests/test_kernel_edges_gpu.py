@@ -35,10 +35,10 @@ def test_adding_launch_of_the_fused_kernel(torch, variant, n_sta, n_chan, n_time
 
 
 # ------------------------------------------------ the CTA-pair kernel over its ring of planes ---
-# Three or more 128-input tiles: every tile count's grouping (an odd one leaves a CTA without a row
+# Two or more 128-input tiles: every tile count's grouping (an odd one leaves a CTA without a row
 # tile, transposed tile pairs), input counts that end inside a tile and inside 16, samples that end
 # inside a stage (64 / 32), a chunk (512 / 256 / 384) and an exact window, few and many channels.
-PAIR_SIZES = [(129, 1, 1), (130, 3, 65), (169, 5, 513), (192, 2, 385), (200, 3, 700), (256, 2, 1100), (320, 1, 130),
+PAIR_SIZES = [(65, 2, 40), (128, 3, 300), (129, 1, 1), (130, 3, 65), (169, 5, 513), (192, 2, 385), (200, 3, 700), (256, 2, 1100), (320, 1, 130),
               (331, 2, 96)]
 
 
@@ -167,3 +167,24 @@ def test_pair_ring_kernel_float_edges(torch):
     scale = np.sqrt(autos[:, ii] * autos[:, jj])
     err = np.abs((got[..., 0] - clean[..., 0]) + 1j * (got[..., 1] - clean[..., 1]))
     assert (err[~bad] <= 1e-6 * scale[~bad]).all()
+
+
+# ------------------------------------------- int8 samples decoded on chip, on CTA pairs ---
+@pytest.mark.parametrize("n_sta,n_chan,n_time", [(4, 3, 1), (4, 20, 33), (32, 5, 511), (60, 2, 513), (64, 90, 70), (68, 2, 1024),
+                                                 (128, 3, 1025), (132, 2, 31), (200, 2, 600), (256, 1, 1600), (324, 2, 64)])
+def test_int8_decoded_on_chip(torch, n_sta, n_chan, n_time):
+    """Input counts that are a multiple of 8 (and end inside a half-tile), samples that end inside a
+    stage (32) and a window (512), full-scale codes, three executes that add up."""
+    x = synth.uniform_ci8(3 * n_time, n_chan, n_sta, seed=n_sta)
+    x[:n_time, 0] = -128
+    x[n_time:, 0, 0, 0] = 127
+    xd = torch.from_numpy(x).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="ci8", engine="tensor") as plan:
+        for k in range(3):
+            plan.execute(xd[k * n_time:(k + 1) * n_time].clone())
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+        one = plan.execute_dump(xd[n_time:2 * n_time].clone()).cpu().numpy()
+        plan.sync()
+    check("ci8", got, x, 2 * n_sta)
+    check("ci8", one, x[n_time:2 * n_time], 2 * n_sta)

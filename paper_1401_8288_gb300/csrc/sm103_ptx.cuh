@@ -25,6 +25,14 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
+// ------------------------------------------------------- dependent launches --
+// A kernel launched by launch_dependent (xcorr_internal.h) may start while the stream's previous
+// kernel still runs, once all of that kernel's CTAs have called pdl_release (or left).  Before
+// pdl_wait returns it must not touch global memory: then the previous kernel has completed and its
+// writes are visible.  What comes before -- barriers, tensor memory -- overlaps the previous tail.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- mbarrier --
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");

@@ -157,6 +157,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const uint32_t tmem = *tslot;
   const int n_items = p.n_items;
   const int cl = static_cast<int>(blockIdx.x >> 1), n_cl = static_cast<int>(gridDim.x >> 1);
+  // The start overlaps the previous kernel's tail (128 inputs x 64 channels x 1024 samples: 22.5 -> 20.2 us;
+  // 512 x 256 x 4096: 900 -> 897 us).
+  pdl_release();
+  pdl_wait();
 
   if (warp < kEpiWarps) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
@@ -433,8 +437,7 @@ cudaError_t launch_raw_pair(const CUtensorMap& map, const RParams& p, int num_sm
   int n_cl = max_clusters < num_sms / 2 ? max_clusters : num_sms / 2;
   if (n_cl < 1) n_cl = 1;
   if (p.n_items < n_cl) n_cl = p.n_items;
-  kern<<<2 * n_cl, kThreads, kSmem, stream>>>(map, p);
-  return cudaGetLastError();
+  return launch_dependent(kern, 2 * n_cl, kThreads, kSmem, stream, map, p);
 }
 
 }  // namespace

@@ -188,3 +188,50 @@ def test_int8_decoded_on_chip(torch, n_sta, n_chan, n_time):
         plan.sync()
     check("ci8", got, x, 2 * n_sta)
     check("ci8", one, x[n_time:2 * n_time], 2 * n_sta)
+
+
+# ------------------------------------------------ launches that start over the previous one's tail --
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time", [("ci4", 4, 8, 64), ("ci8", 6, 8, 64), ("ci4", 32, 16, 300), ("ci4", 160, 128, 200),
+                                                     ("ci8", 64, 16, 200), ("ci8", 160, 128, 100)])
+@pytest.mark.parametrize("captured", [False, True])
+def test_back_to_back_launches_see_the_previous_writes(torch, fmt, n_sta, n_chan, n_time, captured):
+    """Eight executes into one accumulator, each on a buffer that the stream has just rewritten (by a
+    kernel of the same stream, and once by a joined one), then the dump: short and long launches."""
+    x = draw(fmt, 8 * n_time, n_chan, n_sta, seed=7 * n_sta + n_time)
+    xd = torch.from_numpy(x).cuda()
+    buf = torch.zeros_like(xd[:n_time])
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt) as plan:
+        out = torch.empty((n_chan, plan.info["n_pairs"], 2), dtype=torch.int32, device="cuda")
+
+        def passes():
+            for k in range(8):
+                part = xd[k * n_time:(k + 1) * n_time]
+                if k == 3:  # written on another stream, joined by events
+                    side = torch.cuda.Stream()
+                    side.wait_stream(torch.cuda.current_stream())
+                    with torch.cuda.stream(side):
+                        torch.add(part, 0, out=buf)
+                    torch.cuda.current_stream().wait_stream(side)
+                else:
+                    torch.add(part, 0, out=buf)
+                plan.execute(buf)
+            plan.dump(out=out)
+
+        stream = torch.cuda.Stream()
+        stream.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(stream):
+            if captured:
+                passes()
+                graph = torch.cuda.CUDAGraph()
+                stream.synchronize()
+                with torch.cuda.graph(graph, stream=stream):
+                    passes()
+                out.zero_()
+                graph.replay()
+                graph.replay()
+            else:
+                passes()
+        torch.cuda.synchronize()
+        got = out.cpu().numpy()
+        plan.sync()
+    assert np.array_equal(got.astype(np.int64), oracle.correlate(oracle.FMT_CI4 if fmt == "ci4" else oracle.FMT_CI8, x))

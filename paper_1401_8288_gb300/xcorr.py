@@ -703,7 +703,8 @@ class Plan:
         torch = self._torch
         shape = (self.n_channels, self.info["n_pairs"], 2)
         if out is None:
-            out = torch.zeros(shape, dtype=self._out_dtype(wide), device="cuda")
+            # wide dumps add to what is there; the others write every entry
+            out = (torch.zeros if wide else torch.empty)(shape, dtype=self._out_dtype(wide), device="cuda")
         flags = (XCORR_DUMP_RESET if reset else 0) | (XCORR_DUMP_ADD_WIDE if wide else 0)
         self.samples = xcorr_dump(self.handle, out.data_ptr(), out.is_cuda, flags,
                                   self._stream(stream))
@@ -724,8 +725,8 @@ class Plan:
         if not x.is_cuda or not x.is_contiguous():
             raise ValueError("input must be a contiguous CUDA tensor")
         if out is None:
-            out = torch.zeros((self.n_channels, self.info["n_pairs"], 2),
-                              dtype=self._out_dtype(wide), device="cuda")
+            out = (torch.zeros if wide else torch.empty)((self.n_channels, self.info["n_pairs"], 2),
+                                                         dtype=self._out_dtype(wide), device="cuda")
         flags = (XCORR_DUMP_RESET if reset else 0) | (XCORR_DUMP_ADD_WIDE if wide else 0)
         self.samples = xcorr_execute_dump(self.handle, x.data_ptr(), x.shape[0], out.data_ptr(),
                                           out.is_cuda, flags, self._stream(stream))

@@ -20,28 +20,6 @@ __device__ __forceinline__ void decode_ci4(const uint4& v, uint4& re, uint4& im)
   ci4_to_e4m3(v.w, re.w, im.w);
 }
 
-// Two int8 samples (re0 im0 re1 im1) -> two BF16 real parts and two imaginary parts, exact (|v| <=
-// 128 needs 8 significant bits).  v + 128 in the low mantissa bits of 2^23 is an exact float, as is
-// its difference to 2^23 + 128; the upper half of that float is its BF16 value.  Five instructions
-// for two values on the ALU and FMA pipes (the I2F conversion runs at an eighth of their rate).
-__device__ __forceinline__ uint32_t bf16_pair_of(uint32_t biased, uint32_t sel0, uint32_t sel1) {
-  const float a = __uint_as_float(__byte_perm(biased, 0x4B000000u, sel0)) - 8388736.0f;
-  const float b = __uint_as_float(__byte_perm(biased, 0x4B000000u, sel1)) - 8388736.0f;
-  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
-}
-__device__ __forceinline__ void ci8_to_bf16(uint32_t w, uint32_t& re, uint32_t& im) {
-  const uint32_t u = w ^ 0x80808080u;  // v + 128 in every byte
-  re = bf16_pair_of(u, 0x7440, 0x7442);
-  im = bf16_pair_of(u, 0x7441, 0x7443);
-}
-// Eight int8 samples -> eight BF16 real parts and eight imaginary parts.
-__device__ __forceinline__ void decode_ci8(const uint4& v, uint4& re, uint4& im) {
-  ci8_to_bf16(v.x, re.x, im.x);
-  ci8_to_bf16(v.y, re.y, im.y);
-  ci8_to_bf16(v.z, re.z, im.z);
-  ci8_to_bf16(v.w, re.w, im.w);
-}
-
 // Float input, per (channel, window, input): find the window's
 // largest magnitude max < 2^(E+1), quantise each component to the integer
 // M = rint(x 2^(22-E)) (|M| < 2^23, error <= 2^-23 max), and write the

@@ -126,6 +126,86 @@ bool raw_ci8_applies(xcorr_plan plan, const void* d_in) {
   return plan->cfg.fmt == XCORR_IN_CI8 && plan->engine == XCORR_ENGINE_TENSOR && xc::raw_pair_takes(plan->n_inputs, d_in);
 }
 
+// Input that would be decoded on chip but for its rows' or its address's alignment is copied piece by
+// piece to padded rows in the plan's planes memory and correlated from there (xcorr_repitch.cu).
+// A piece: `nc` channels x `nt` samples.
+struct Pieces {
+  int pitch = 0;  // inputs from one row to the next; 0: does not apply
+  int nc = 0, nt = 0;
+  int count = 0;
+};
+// At most a GB at a time.  A piece that stays in the L2 saves less than it costs in waves of the X
+// kernel that are not full and in launches (510 inputs x 400 channels x 2048 4-bit samples with pieces
+// of 64 / 96 / 256 MB / 1 GB: 605 / 556 / 522 / 510 us; 510 x 300 x 2048 int8: 807 / 771 / 740 / 725).
+constexpr size_t kPieceBytes = size_t(1) << 30;
+constexpr size_t kOddAddressPieceBytes = size_t(64) << 20;  // kept by plans that need it at odd addresses only
+size_t padded_row_bytes(int fmt, int n_inputs) {
+  return static_cast<size_t>((n_inputs * (fmt == XCORR_IN_CI4 ? 1 : 2) + 15) / 16) * 16;
+}
+Pieces repitch_pieces(xcorr_plan plan, int n_time) {
+  Pieces r;
+  const int fmt = plan->cfg.fmt;
+  if (plan->engine != XCORR_ENGINE_TENSOR || fmt == XCORR_IN_CF32 || (fmt == XCORR_IN_CI4 && plan->tune_unfused))
+    return r;
+  const int C = plan->cfg.n_channels;
+  const size_t row = padded_row_bytes(fmt, plan->n_inputs);
+  const size_t room = plan->planes_bytes < kPieceBytes ? plan->planes_bytes : kPieceBytes;
+  const size_t rows = room / row;  // of one channel and sample each
+  if (rows >= static_cast<size_t>(n_time)) {
+    r.nc = rows / n_time < static_cast<size_t>(C) ? static_cast<int>(rows / n_time) : C;
+    if (r.nc < C) {  // several pieces: whole waves of the X kernel where a piece holds one
+      const int nb = (plan->n_inputs + 127) / 128;
+      const int per_chan = fmt == XCORR_IN_CI4 ? nb * (nb + 1) / 2 : xc::raw_pair_items(nb);
+      const int wave = fmt == XCORR_IN_CI4 ? plan->num_sms : plan->num_sms / 2;
+      const int whole = static_cast<int>(static_cast<int64_t>(r.nc) * per_chan / wave * wave / per_chan);
+      if (whole > 0) r.nc = whole;
+    }
+    r.count = (C + r.nc - 1) / r.nc;
+    r.nt = n_time;
+  } else {  // a long integration: one channel, whole stages of samples at a time
+    r.nc = 1;
+    r.nt = static_cast<int>(rows / 128 * 128);
+    if (r.nt == 0) return r;  // (4-bit under a tight memory limit: the ring of planes)
+    r.count = C * ((n_time + r.nt - 1) / r.nt);
+  }
+  r.pitch = static_cast<int>(fmt == XCORR_IN_CI4 ? row : row / 2);
+  return r;
+}
+
+// The tensor-memory-A kernel's launch shape for a stage variant; the other kernels' variants mean its
+// default here.
+int padded_shape(int v) {
+  return v == xc::kSmallFusedVariant ? 3 : v >= 4 && v <= 6 ? v - 4 : xc::kDefaultFusedVariant - 4;
+}
+
+// Correlate through padded rows.
+cudaError_t run_repitched(xcorr_plan plan, const Pieces& r, const void* d_in, int n_time, int2* target, bool fresh,
+                          cudaStream_t s) {
+  const int C = plan->cfg.n_channels, N = plan->n_inputs;
+  const bool ci4 = plan->cfg.fmt == XCORR_IN_CI4;
+  const size_t row = static_cast<size_t>(N) * (ci4 ? 1 : 2);  // one channel of one sample
+  const uint8_t* in = static_cast<const uint8_t*>(d_in);
+  const uint8_t* end = in + row * C * n_time;
+  const int shape = padded_shape(plan->tune_variant);
+  for (int t0 = 0; t0 < n_time; t0 += r.nt) {
+    const int nt = n_time - t0 < r.nt ? n_time - t0 : r.nt;
+    for (int c0 = 0; c0 < C; c0 += r.nc) {
+      const int nc = C - c0 < r.nc ? C - c0 : r.nc;
+      cudaError_t e = xc::launch_repitch(in + (static_cast<size_t>(t0) * C + c0) * row, end, plan->planes,
+                                         static_cast<int>(row), C, nc, nt, plan->num_sms, s);
+      if (e != cudaSuccess) return e;
+      int2* out = target + static_cast<int64_t>(c0) * plan->n_pairs;
+      const bool add = !fresh || t0 > 0;
+      e = ci4 ? xc::launch_xcorr_tc_fused_ta_ci4(static_cast<const uint8_t*>(plan->planes), nc, shape, nt, nc, N, r.pitch,
+                                                 out, add, plan->status, plan->num_sms, s)
+              : xc::launch_xcorr_tc_raw_pair(static_cast<const int8_t*>(plan->planes), nt, nc, N, r.pitch, out, add,
+                                             plan->status, plan->num_sms, s);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return cudaSuccess;
+}
+
 // Unpack channels [c0, c0 + nc) of the input into the plan's planes.
 cudaError_t unpack_group(xcorr_plan plan, const void* d_in, int n_time, int c0, int nc, cudaStream_t s) {
   const int C = plan->cfg.n_channels, N = plan->n_inputs, T = plan->cfg.max_time_per_exec;
@@ -133,9 +213,6 @@ cudaError_t unpack_group(xcorr_plan plan, const void* d_in, int n_time, int c0, 
     case XCORR_IN_CI4:
       return xc::launch_unpack_ci4_e4m3_channels(static_cast<const uint8_t*>(d_in), static_cast<uint8_t*>(plan->planes),
                                                  n_time, C, c0, nc, N, plan->ni_pad, T, plan->num_sms, s);
-    case XCORR_IN_CI8:
-      return xc::launch_unpack_ci8_bf16(static_cast<const int8_t*>(d_in), static_cast<uint16_t*>(plan->planes), n_time,
-                                        C, c0, nc, N, plan->ni_pad, T, plan->num_sms, s);
     default:
       return xc::launch_unpack_cf32_digits(static_cast<const float*>(d_in), static_cast<uint16_t*>(plan->planes),
                                            plan->exps, n_time, C, c0, nc, N, plan->ni_pad, T, plan->window_samples,
@@ -168,9 +245,17 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     // int8 input decoded on chip: one launch on the caller's stream
     if (ev && ((e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventRecord(ev[2], s)) != cudaSuccess))
       return cuda_fail(e, "profile event");
-    e = xc::launch_xcorr_tc_raw_pair(static_cast<const int8_t*>(d_in), n_time, C, N, static_cast<int2*>(target),
+    e = xc::launch_xcorr_tc_raw_pair(static_cast<const int8_t*>(d_in), n_time, C, N, N, static_cast<int2*>(target),
                                      !target_fresh, plan->status, plan->num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "CTA-pair X kernel launch");
+    if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
+    if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
+  } else if (const Pieces pieces = repitch_pieces(plan, n_time); pieces.pitch) {
+    // the same kernels over padded rows, piece by piece on the caller's stream
+    if (ev && ((e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventRecord(ev[2], s)) != cudaSuccess))
+      return cuda_fail(e, "profile event");
+    if ((e = run_repitched(plan, pieces, d_in, n_time, static_cast<int2*>(target), target_fresh, s)) != cudaSuccess)
+      return cuda_fail(e, "padded rows: copy or X kernel launch");
     if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
     if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
   } else if (plan->pair) {
@@ -324,8 +409,8 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   // AUTO: the engine the per-call device times favour (graph-replayed execute_dump; 4-bit input
   // over inputs 2-256, channels 16-256, K 256-2048; int8 over inputs 2-256, channels 16-64,
   // K 256-1024).  The CUDA-core kernel wins only at most 16 channels: for 4-bit input below 16
-  // inputs (the tensor path then unpacks to planes first: two launches), for int8 input up to 64
-  // inputs (its tensor path always unpacks to BF16 planes first); the tensor cores everywhere else.
+  // inputs (the tensor path then pads the rows first: two launches), for int8 input up to 64 inputs;
+  // the tensor cores everywhere else.
   const int cc_inputs = c.fmt == XCORR_IN_CI4 ? 15 : c.fmt == XCORR_IN_CI8 ? 64 : 0;
   const int engine = c.engine != XCORR_ENGINE_AUTO ? c.engine
                      : (c.n_stations <= cc_inputs / 2 && c.n_channels <= 16) ? XCORR_ENGINE_CUDA_CORE
@@ -358,8 +443,10 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   const size_t acc_bytes = (size_t)c.n_channels * (size_t)n_pairs * 8;
   // two or more 128-input tiles run on CTA pairs from a small ring of planes; smaller problems stage
   // all their planes
-  const bool pair = engine == XCORR_ENGINE_TENSOR && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles;
-  size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !pair ? (size_t)c.n_channels * ppc *
+  // (int8 never needs planes)
+  const bool decoded_ci8 = engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CI8;
+  const bool pair = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles;
+  size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && !pair ? (size_t)c.n_channels * ppc *
                                                                      (size_t)c.max_time_per_exec * ni_pad * elem_bytes
                                                                : 0;
   const int exp_windows = (c.max_time_per_exec + xc::kTcWindowBF16 - 1) / xc::kTcWindowBF16;
@@ -368,12 +455,29 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
                                 ? (size_t)c.n_channels * exp_windows * ni_pad * 2 + 256
                                 : 0;
   xc::PairRing ring;
+  const size_t other = acc_bytes + exps_bytes + 256;
+  const size_t room = c.hbm_budget_bytes > other ? c.hbm_budget_bytes - other : 1;
+  // Memory for padded rows (run_repitched), for integer input whose rows are not whole 16-byte units:
+  // one piece.  Whole rows need it only at an odd address (int8; 4-bit uses its planes memory then).
+  const size_t row_bytes = (size_t)n_inputs * (c.fmt == XCORR_IN_CI4 ? 1 : 2);
+  const size_t padded = padded_row_bytes(c.fmt, n_inputs);
+  size_t piece = padded * c.n_channels * (size_t)c.max_time_per_exec;
+  const size_t piece_cap = row_bytes % 16 != 0 ? kPieceBytes : kOddAddressPieceBytes;
+  if (piece > piece_cap) piece = piece_cap;
+  if (decoded_ci8) {
+    const size_t least = padded * (size_t)(c.max_time_per_exec < 128 ? c.max_time_per_exec : 128);
+    if (c.hbm_budget_bytes && piece > room) piece = room;
+    planes_bytes = piece > least ? piece : least;
+  }
   if (pair) {
-    const size_t other = acc_bytes + exps_bytes + 256;
-    const size_t room = c.hbm_budget_bytes > other ? c.hbm_budget_bytes - other : 1;
     e = xc::pair_ring_layout(c.fmt, n_inputs, c.n_channels, c.max_time_per_exec, c.hbm_budget_bytes ? room : 0, &ring);
     if (e != cudaSuccess) return cuda_fail(e, "ring layout");
     planes_bytes = ring.bytes;
+    if (c.fmt == XCORR_IN_CI4 && row_bytes % 16 != 0) {
+      const size_t left = room > ring.flag_bytes ? room - ring.flag_bytes : 0;
+      if (c.hbm_budget_bytes && piece > left) piece = left;
+      if (piece > planes_bytes) planes_bytes = piece;
+    }
   }
   const size_t dev_bytes = acc_bytes + planes_bytes + ring.flag_bytes + exps_bytes + 256;
   if (c.hbm_budget_bytes && dev_bytes > c.hbm_budget_bytes)
@@ -675,12 +779,14 @@ xcorr_status xcorr_plan_query(xcorr_plan plan, xcorr_plan_info* info) {
                      plan->n_inputs % 16 == 0;
   // (int8: a 16-byte aligned input, nullptr standing for one)
   const bool one_launch = plan->pair || raw_ci8_applies(plan, nullptr);
+  const Pieces pieces = fused || raw_ci8_applies(plan, nullptr) ? Pieces{} : repitch_pieces(plan, plan->cfg.max_time_per_exec);
   info->kernels_per_execute = fused ? xc::fused_launches(plan->cfg.max_time_per_exec)
+                              : pieces.pitch ? pieces.count * (1 + (plan->cfg.fmt == XCORR_IN_CI4 ? xc::fused_launches(pieces.nt) : 1))
                               : one_launch                          ? 1
                               : plan->engine == XCORR_ENGINE_TENSOR ? 2 * tensor_groups(plan)
                                                                      : 1;
   info->tuning.stage_variant = plan->tune_variant;
-  info->tuning.groups = fused || one_launch ? 1 : tensor_groups(plan);
+  info->tuning.groups = fused || one_launch || pieces.pitch ? 1 : tensor_groups(plan);
   info->tuning.x_streams = plan->tune_x_streams;
   info->tuning.unfused = plan->tune_unfused;
   return XCORR_OK;
@@ -726,18 +832,20 @@ xcorr_status xcorr_autotune(xcorr_plan plan, const void* d_in, int n_time, void*
   const int group_choices[] = {1, 2, 4, 8};
   xcorr_tuning winner{plan->tune_variant, plan->tune_groups, plan->tune_x_streams, plan->tune_unfused};
   float winner_ms = 1e30f;
-  // candidates: the fused 4-bit kernel (3 stage shapes) where it applies, then
-  // every planes-based shape
+  // candidates: the fused 4-bit kernels' shapes where one applies (over padded rows: those of the
+  // kernel that takes them), then every planes-based shape
   plan->tune_unfused = 0;
   const bool fused_ok = fused_applies(plan, d_in);
-  for (int uf = fused_ok ? 0 : 1; uf <= 1 && st == XCORR_OK; ++uf)
+  const bool padded_ci4 = !fused_ok && plan->cfg.fmt == XCORR_IN_CI4 && repitch_pieces(plan, n_time).pitch > 0;
+  for (int uf = fused_ok || padded_ci4 ? 0 : 1; uf <= 1 && st == XCORR_OK; ++uf)
   for (int v = 0; v < (uf == 0 ? xc::kFusedVariants : xc::kTcVariants) && st == XCORR_OK; ++v) {
     for (int gi = 0; gi < 4 && st == XCORR_OK; ++gi) {
       for (int xs = 1; xs <= 2 && st == XCORR_OK; ++xs) {
         if (group_choices[gi] == 1 && xs == 2) continue;  // one group has one X launch
         if (uf == 0 && (gi > 0 || xs > 1)) continue;      // the fused kernel is one launch
-        // so are the CTA-pair kernels, of one shape each
-        if (uf == 1 && (plan->pair || raw_ci8_applies(plan, d_in)) && (v > 0 || gi > 0)) continue;
+        if (uf == 0 && padded_ci4 && padded_shape(v) != v - 4 && v != xc::kSmallFusedVariant) continue;
+        // the CTA-pair kernels have one shape each
+        if (uf == 1 && (plan->pair || plan->cfg.fmt == XCORR_IN_CI8) && (v > 0 || gi > 0)) continue;
         plan->tune_variant = v;
         plan->tune_groups = group_choices[gi];
         plan->tune_x_streams = xs;

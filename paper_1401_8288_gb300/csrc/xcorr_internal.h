@@ -149,10 +149,10 @@ namespace xc {
 // Launch a kernel that calls pdl_wait so that its start overlaps the tail of the stream's previous
 // kernel (about 2 us per call on small problems: the launch latency, barrier and tensor-memory setup).
 template <typename... Params, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream,
                              const Args&... args) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
@@ -296,8 +296,9 @@ cudaError_t launch_xcorr_tc_fused_ci4(const uint8_t* in, int row_chans, int vari
                                       cudaStream_t stream);
 
 int fused_ta_stage_samples(int variant);
+// pitch: bytes from one channel to the next (n_inputs, or more where rows were padded), a multiple of 16.
 cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int variant, int n_time, int n_chan,
-                                         int n_inputs, int2* out, bool accumulate, int* status, int num_sms,
+                                         int n_inputs, int pitch, int2* out, bool accumulate, int* status, int num_sms,
                                          cudaStream_t stream);
 
 // The fused 4-bit kernel on CTA pairs (xcorr_tc_fused_pair.cu): two SMs share
@@ -312,14 +313,17 @@ cudaError_t launch_xcorr_tc_fused_pair_ci4(const uint8_t* in, int row_chans, int
 bool encode_raw_ci8_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_chan, int n_time, int box_t,
                          std::string* err);
 // The X-stage on CTA pairs with int8 samples decoded on chip (xcorr_tc_raw_pair.cu): one launch.
-bool raw_pair_takes(int n_inputs, const void* in);
-cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int n_time, int n_chan, int n_inputs, int2* out, bool accumulate,
-                                     int* status, int num_sms, cudaStream_t stream);
+bool raw_pair_takes(int pitch, const void* in);
+int raw_pair_items(int n_tiles);  // work items of one channel
+// pitch: inputs from one channel to the next (n_inputs, or more where rows were padded), a multiple of 8.
+cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int n_time, int n_chan, int n_inputs, int pitch, int2* out,
+                                     bool accumulate, int* status, int num_sms, cudaStream_t stream);
 
-// int8 (re, im) samples -> two BF16 planes [c][2][t][ni_pad] (exact).
-cudaError_t launch_unpack_ci8_bf16(const int8_t* in, uint16_t* planes, int n_time, int n_chan, int c0,
-                                   int nc, int n_inputs, int ni_pad, int max_time, int num_sms,
-                                   cudaStream_t stream);
+// Copies n_chan rows of row_bytes (of the row_chans that make up a sample) x n_time samples to rows of
+// row_bytes rounded up to 16 (xcorr_repitch.cu).  `end`: one past the last byte of the caller's input.
+cudaError_t launch_repitch(const void* in, const void* end, void* out, int row_bytes, int row_chans, int n_chan,
+                           int n_time, int num_sms, cudaStream_t stream);
+
 // float (re, im) samples -> six BF16 planes [c][6][t][ni_pad] of integer digits
 // (re digits 0-2, im digits 0-2) and one exponent per (channel, window, input).
 cudaError_t launch_unpack_cf32_digits(const float* in, uint16_t* planes, int16_t* exps, int n_time, int n_chan,

@@ -492,14 +492,14 @@ cudaError_t launch_xcorr_tc_fused_ci4(const uint8_t* in, int row_chans, int vari
                                       int n_inputs, int2* out, bool accumulate, int* status, int num_sms,
                                       cudaStream_t stream) {
   if (variant == 10)  // the tensor-memory-A kernel's small-problem layout
-    return launch_xcorr_tc_fused_ta_ci4(in, row_chans, 3, n_time, n_chan, n_inputs, out, accumulate, status,
+    return launch_xcorr_tc_fused_ta_ci4(in, row_chans, 3, n_time, n_chan, n_inputs, n_inputs, out, accumulate, status,
                                         num_sms, stream);
   if (variant >= 7)
     return launch_xcorr_tc_fused_pair_ci4(in, row_chans, variant - 7, n_time, n_chan, n_inputs, out, accumulate,
                                           status, num_sms, stream);
   if (variant >= 4)
-    return launch_xcorr_tc_fused_ta_ci4(in, row_chans, variant - 4, n_time, n_chan, n_inputs, out, accumulate, status,
-                                        num_sms, stream);
+    return launch_xcorr_tc_fused_ta_ci4(in, row_chans, variant - 4, n_time, n_chan, n_inputs, n_inputs, out,
+                                        accumulate, status, num_sms, stream);
   const int nb = (n_inputs + kBlk - 1) / kBlk;
   const int kt = fused_stage_samples(variant);
   if (n_time <= 0 || n_inputs % 16 != 0 || reinterpret_cast<uintptr_t>(in) % 16 != 0 ||

@@ -99,11 +99,12 @@ struct TGeom {
 
 struct TParams {
   int n_chan, n_inputs, n_tile_pairs;
+  int pitch;           // inputs from one channel to the next in the raw rows
   int t0;              // first sample of this launch
   int n_kt;            // stages per tile pair
   int64_t n_pairs;
   int accumulate;      // add into out (else store)
-  // small-problem layout: pack_g channels of n_inputs each side by side in one tile (PACK), and
+  // small-problem layout: pack_g channels of pitch inputs each side by side in one tile (PACK), and
   // each tile's stages cut into n_split items of split_kt stages whose results are added with
   // atomics (atomic_out)
   int pack_g, n_split, split_kt, atomic_out;
@@ -169,8 +170,8 @@ __device__ __forceinline__ TItem resolve(const TParams& p, const CUtensorMap* ma
     }
   }
   it.diag = it.I == it.J;
-  if (PACK) {  // the packed view: x = channel * n_inputs + input over one time row
-    it.ax = it.bx = it.c * p.pack_g * p.n_inputs;
+  if (PACK) {  // the packed view: x = channel * pitch + input over one time row
+    it.ax = it.bx = it.c * p.pack_g * p.pitch;
     it.ay = it.by = 0;
   } else {
     it.ax = it.I * kBlk;
@@ -550,7 +551,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_after();
       // 16-pair chunks this warp keeps: none past the inputs (the packed channels), none wholly
       // above the diagonal
-      const int n_ch = (PACK ? (warp * 32 >= p.pack_g * n_inputs || c * p.pack_g + (warp * 32) / n_inputs >= p.n_chan)
+      const int n_ch = (PACK ? (warp * 32 >= p.pack_g * p.pitch || c * p.pack_g + (warp * 32) / p.pitch >= p.n_chan)
                              : row0 >= n_inputs)
                            ? 0
                        : I == J ? (warp * 32 + 31) / kChunk + 1
@@ -598,10 +599,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         lastm[m] = I == J ? rr : kBlk - 1;  // last column of the row in the tile
         rcm[m] = rowc[rr];
         if (PACK) {
-          const int blk = rr / n_inputs, cr = c * p.pack_g + blk;
-          if (blk < p.pack_g && cr < p.n_chan) {
-            firstm[m] = blk * n_inputs;
-            const int i = rr - firstm[m];
+          const int blk = rr / p.pitch, cr = c * p.pack_g + blk;
+          const int i = rr - blk * p.pitch;
+          if (blk < p.pack_g && cr < p.n_chan && i < n_inputs) {
+            firstm[m] = blk * p.pitch;
             row_out[m] = it.out + (int64_t)cr * it.n_pairs + (int64_t)i * (i + 1) / 2;
           }
         } else {
@@ -742,16 +743,17 @@ void small_layout(int n_chan, int n_inputs, int n_kt, int num_sms, int& pack_g, 
 }
 
 cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int variant, int n_time, int n_chan,
-                                         int n_inputs, int2* out, bool accumulate, int* status, int num_sms,
-                                         cudaStream_t stream) {
+                                         int n_inputs, int pitch, int2* out, bool accumulate, int* status,
+                                         int num_sms, cudaStream_t stream) {
   const int nb = (n_inputs + kBlk - 1) / kBlk;
   const int kt = fused_ta_stage_samples(variant);
-  if (n_time <= 0 || n_inputs % 16 != 0 || reinterpret_cast<uintptr_t>(in) % 16 != 0 ||
+  if (n_time <= 0 || pitch < n_inputs || pitch % 16 != 0 || reinterpret_cast<uintptr_t>(in) % 16 != 0 ||
       kFusedWindowCI4 % kt != 0)
     return cudaErrorInvalidValue;
   TParams p{};
   p.n_chan = n_chan;
   p.n_inputs = n_inputs;
+  p.pitch = pitch;
   p.n_tile_pairs = nb * (nb + 1) / 2;
   p.n_pairs = (int64_t)n_inputs * (n_inputs + 1) / 2;
   p.out = out;
@@ -761,13 +763,13 @@ cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int v
   CUtensorMap raw_map;
   if (row_chans < n_chan) return cudaErrorInvalidValue;
   int pack_g = 1;
-  if (small) pack_g = n_inputs <= kBlk / 2 ? kBlk / n_inputs : 1;
+  if (small) pack_g = pitch <= kBlk / 2 ? kBlk / pitch : 1;
   if (pack_g > 1) {
-    // the packed view: one time row is n_chan * n_inputs bytes (channel-major), read in boxes of 128
+    // the packed view: one time row is n_chan * pitch bytes (channel-major), read in boxes of 128
     // (pack_g channels side by side) x 1 x kt; the middle dimension has extent 1
-    if (!encode_raw_ci4_packed_tmap(&raw_map, in, n_inputs, n_chan, row_chans, n_time, kt, nullptr))
+    if (!encode_raw_ci4_packed_tmap(&raw_map, in, pitch, n_chan, row_chans, n_time, kt, nullptr))
       return cudaErrorInvalidValue;
-  } else if (!encode_raw_ci4_tmap(&raw_map, in, n_inputs, n_chan, row_chans, n_time, kt, nullptr)) {
+  } else if (!encode_raw_ci4_tmap(&raw_map, in, pitch, n_chan, row_chans, n_time, kt, nullptr)) {
     return cudaErrorInvalidValue;
   }
   p.pack_g = pack_g;
@@ -780,7 +782,7 @@ cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int v
     int tiles = n_chan * p.n_tile_pairs;
     p.n_split = 1;
     p.split_kt = p.n_kt;
-    if (small) small_layout(n_chan, n_inputs, p.n_kt, num_sms, pack_g, tiles, p.n_split, p.split_kt);
+    if (small) small_layout(n_chan, pitch, p.n_kt, num_sms, pack_g, tiles, p.n_split, p.split_kt);
     p.atomic_out = p.n_split > 1 ? 1 : 0;
     p.n_items = tiles * p.n_split;
     if (p.atomic_out && !p.accumulate) {  // the split items add into a cleared output

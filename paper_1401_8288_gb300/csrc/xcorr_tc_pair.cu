@@ -5,12 +5,12 @@
 // Same operands, K axis, exact blocks and results as xcorr_unpack.cu followed
 // by xcorr_tc.cu (per channel the packed lower triangle of V = sum_t x_t x_t^H;
 // Sec. 1, Sec. 2.1, Eq. 1; the unpack and corner turn of Sec. 2.4): 4-bit
-// samples as E4M3 planes, int8 as BF16 planes, float as six BF16 planes of
-// integer digits with one exponent per (channel, 384-sample window, input).
+// samples as E4M3 planes, float as six BF16 planes of integer digits with one
+// exponent per (channel, 384-sample window, input).
 // For problems of two or more 128-input tiles.
 //
-// Why one launch.  Unpacking to planes in HBM writes 2 (4-bit), 4 (int8) or 12
-// (float) bytes per sample that the X kernel reads back: as much time as the
+// Why one launch.  Unpacking to planes in HBM writes 2 (4-bit) or 12 (float)
+// bytes per sample that the X kernel reads back: as much time as the
 // tensor work itself.  Unpacking on chip inside the tile pairs repeats the
 // decode for every tile pair that needs an input.  Here four warps of every
 // CTA unpack each sample once, a chunk of time ahead of the tile pairs, into a
@@ -50,15 +50,17 @@
 // (sm103_ptx.cuh).  The last CTA to leave clears the flags.
 //
 // Measured (one GB300), against unpack + planes kernel: 512 inputs x 256 channels x 4096 samples, float
-// 5.2-5.8 ms (7.2-7.3), int8 1.00 ms (1.32); 338 inputs x 97 channels x 1500, 4-bit, 129 us (252); two
-// tiles: 256 inputs x 256 channels x 2048, float, 1.22 ms (1.40), 250 x 300 x 2048, 4-bit, 355 us (670).
+// 5.2-5.8 ms (7.2-7.3); 338 inputs x 97 channels x 1500, 4-bit, 129 us (252); two tiles: 256 inputs x
+// 256 channels x 2048, float, 1.22 ms (1.40), 250 x 300 x 2048, 4-bit, 355 us (670).
 // A step takes 272 cycles with the MMAs alone, 307-318 from a ring that nobody refills (about 40
 // bytes per cycle and SM from L2, the rate every form of these loads stopped at), 450-470 beside the
 // unpack, which alone would take 250-330.  The rule: two or more tiles.  With one tile half of every
 // pair's rows are idle, and the planes kernel wins once there are channels for every SM (128 inputs x
-// 300 channels x 4096, float: 1.11 ms against 1.29 here).  Aligned 4-bit input stays with the fused
-// kernel (497 us against about 600 us here at 512 inputs x 512 channels x 2048 samples: its L2 traffic
-// is the raw bytes), aligned int8 input goes to xcorr_tc_raw_pair.cu (0.87 ms against 1.00).
+// 300 channels x 4096, float: 1.11 ms against 1.29 here).  4-bit input comes here when planes are asked
+// for, or under a memory limit too tight for padded rows: otherwise it stays with the fused kernel (492
+// us against about 600 here at 512 inputs x 512 channels x 2048 samples: its L2 traffic is the raw
+// bytes), over padded rows where its own are not aligned (74 against 119 us at 338 x 97 x 1500).  int8
+// input goes to xcorr_tc_raw_pair.cu (0.87 ms against 1.00 with BF16 planes here).
 //
 // Warp roles (512 threads, one CTA per SM): warps 0-7 drain TMEM into running
 // sums held in registers (warp w: lane quarter w % 4, columns 64 (w / 4) ..
@@ -98,10 +100,8 @@ constexpr int kFetchSlots = kUnpackWarps * 32 * 4 * kFetchGroups;
 constexpr int kFetchBytes = kFetchSlots * 16 + kFetchSlots / 8 * 4;
 constexpr int kBarrierBytes = 512;
 constexpr int kSinkSlots = kNegWarps + kEpiWarps;  // one per signalling warp of the odd CTA
-// int8: sums of 512 samples reach at most 2 * 128^2 * 512 = 2^24, still exact in FP32
-constexpr int kWindowCI8 = 512;
 
-// FMT: XCORR_IN_CI4 / CI8 / CF32
+// FMT: XCORR_IN_CI4 / CF32
 template <int FMT>
 struct Geom {
   static constexpr int E = FMT == XCORR_IN_CI4 ? 1 : 2;      // operand bytes
@@ -115,8 +115,8 @@ struct Geom {
   static constexpr uint32_t kSignMask = E == 1 ? 0x80808080u : 0x80008000u;
   static constexpr int kDigits = FMT == XCORR_IN_CF32 ? 3 : 1;  // digit planes per component
   static constexpr int kPairsK = FMT == XCORR_IN_CF32 ? 6 : 1;  // plane pairs on the K axis
-  static constexpr int kWindow = FMT == XCORR_IN_CI4 ? kTcWindowCI4 : FMT == XCORR_IN_CI8 ? kWindowCI8 : kTcWindowBF16;
-  static constexpr int kMaxChunk = FMT == XCORR_IN_CI4 ? 512 : FMT == XCORR_IN_CI8 ? 256 : kTcWindowBF16;
+  static constexpr int kWindow = FMT == XCORR_IN_CI4 ? kTcWindowCI4 : kTcWindowBF16;
+  static constexpr int kMaxChunk = FMT == XCORR_IN_CI4 ? 512 : kTcWindowBF16;
   static constexpr int kSpw = kWindow / kRows;               // stages per window
   static constexpr int kOffStaging = kStages * kStageBytes;
   static constexpr int kOffFactors = kOffStaging + kStagingBytes;
@@ -403,12 +403,9 @@ __device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, i
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         uint4 re, im;
-        if (FMT == XCORR_IN_CI4)
-          decode_ci4(v[i], re, im);
-        else
-          decode_ci8(v[i], re, im);
+        decode_ci4(v[i], re, im);
         const int r = r0 + 4 * i;
-        uint8_t* q = dst + 4 * i * G::kRowB + ((G::E == 1 ? pos ^ ((r >> 1) & 3) : pos ^ (r & 7)) << 4);
+        uint8_t* q = dst + 4 * i * G::kRowB + ((pos ^ ((r >> 1) & 3)) << 4);
         if (have) {
           *reinterpret_cast<uint4*>(q) = re;
           *reinterpret_cast<uint4*>(q + G::kPlane) = im;
@@ -914,9 +911,6 @@ cudaError_t pair_ring_layout(int fmt, int n_inputs, int n_chan, int max_time, si
   if (fmt == XCORR_IN_CI4) {
     e = pair_clusters<XCORR_IN_CI4, false>(&n_cl);
     if (e == cudaSuccess) e = pair_clusters<XCORR_IN_CI4, true>(&n_add);
-  } else if (fmt == XCORR_IN_CI8) {
-    e = pair_clusters<XCORR_IN_CI8, false>(&n_cl);
-    if (e == cudaSuccess) e = pair_clusters<XCORR_IN_CI8, true>(&n_add);
   } else {
     e = pair_clusters<XCORR_IN_CF32, false>(&n_cl);
     if (e == cudaSuccess) e = pair_clusters<XCORR_IN_CF32, true>(&n_add);
@@ -924,9 +918,7 @@ cudaError_t pair_ring_layout(int fmt, int n_inputs, int n_chan, int max_time, si
   if (e != cudaSuccess) return e;
   if (n_add < n_cl) n_cl = n_add;
   const int elem = fmt == XCORR_IN_CI4 ? 1 : 2, rows = 64 / elem, planes = fmt == XCORR_IN_CF32 ? 6 : 2;
-  const int most_chunk = fmt == XCORR_IN_CI4   ? Geom<XCORR_IN_CI4>::kMaxChunk
-                         : fmt == XCORR_IN_CI8 ? Geom<XCORR_IN_CI8>::kMaxChunk
-                                               : Geom<XCORR_IN_CF32>::kMaxChunk;
+  const int most_chunk = fmt == XCORR_IN_CI4 ? Geom<XCORR_IN_CI4>::kMaxChunk : Geom<XCORR_IN_CF32>::kMaxChunk;
   const int nb = (n_inputs + kBlk - 1) / kBlk, ne = pair_entries(nb);
   const int64_t items = (int64_t)n_chan * ne;
   if (items > 0x7FFFFFFF / 2) return cudaErrorInvalidValue;
@@ -958,7 +950,7 @@ cudaError_t pair_ring_layout(int fmt, int n_inputs, int n_chan, int max_time, si
 cudaError_t launch_xcorr_tc_pair(const PairLaunch& L, cudaStream_t stream) {
   const PairRing& r = *L.ring;
   const int elem = L.fmt == XCORR_IN_CI4 ? 1 : 2, rows = 64 / elem;
-  const int in_bytes = L.fmt == XCORR_IN_CI4 ? 1 : L.fmt == XCORR_IN_CI8 ? 2 : 8;
+  const int in_bytes = L.fmt == XCORR_IN_CI4 ? 1 : 8;
   P2Params p{};
   p.n_chan = L.n_chan;
   p.n_inputs = L.n_inputs;
@@ -999,9 +991,6 @@ cudaError_t launch_xcorr_tc_pair(const PairLaunch& L, cudaStream_t stream) {
     case XCORR_IN_CI4:
       return L.accumulate ? launch_pair<XCORR_IN_CI4, true>(p, r.clusters, stream)
                           : launch_pair<XCORR_IN_CI4, false>(p, r.clusters, stream);
-    case XCORR_IN_CI8:
-      return L.accumulate ? launch_pair<XCORR_IN_CI8, true>(p, r.clusters, stream)
-                          : launch_pair<XCORR_IN_CI8, false>(p, r.clusters, stream);
     default:
       return L.accumulate ? launch_pair<XCORR_IN_CF32, true>(p, r.clusters, stream)
                           : launch_pair<XCORR_IN_CF32, false>(p, r.clusters, stream);

@@ -235,3 +235,79 @@ def test_back_to_back_launches_see_the_previous_writes(torch, fmt, n_sta, n_chan
         got = out.cpu().numpy()
         plan.sync()
     assert np.array_equal(got.astype(np.int64), oracle.correlate(oracle.FMT_CI4 if fmt == "ci4" else oracle.FMT_CI8, x))
+
+
+# ------------------------------------------- rows copied to 16-byte units before the on-chip decode ---
+@pytest.mark.parametrize("fmt", ["ci4", "ci8"])
+@pytest.mark.parametrize("n_sta,n_chan,n_time", [(1, 1, 1), (1, 40, 130), (3, 5, 257), (4, 33, 128), (5, 300, 64), (9, 7, 1030), (23, 6, 129),
+                                                 (29, 9, 1100), (31, 2, 40), (33, 3, 300), (61, 4, 515), (65, 3, 129), (135, 2, 200), (131, 40, 90)])
+def test_padded_rows(torch, fmt, n_sta, n_chan, n_time):
+    """Every remainder of a row by 16 bytes, single samples, packed and split small layouts; stores,
+    then an adding execute of a shorter block, from a base address off its 16-byte boundary."""
+    x = draw(fmt, n_time + 3, n_chan, n_sta, seed=n_sta + n_time)
+    bufs = [placed(torch, x[:n_time], 0), placed(torch, x[n_time:], 5)]
+    with xcorr.Plan(n_sta, n_chan, max(n_time, 3), fmt=fmt, engine="tensor") as plan:
+        stream = torch.cuda.current_stream().cuda_stream
+        for variant in (None, 4, 5, 6, 10) if fmt == "ci4" else (None,):
+            if variant is not None:
+                plan.set_tuning(variant, 0, 2, 0)
+            xcorr.xcorr_execute(plan.handle, bufs[0].data_ptr(), n_time, stream)
+            xcorr.xcorr_execute(plan.handle, bufs[1].data_ptr() + 5, 3, stream)
+            got = plan.dump().cpu().numpy()
+            plan.sync()
+            check(fmt, got, x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("offset", list(range(16)))
+@pytest.mark.parametrize("fmt,n_sta", [("ci4", 69), ("ci8", 33), ("ci4", 72)])
+def test_padded_rows_from_any_address(torch, fmt, n_sta, offset):
+    x = draw(fmt, 70, 3, n_sta, seed=offset)
+    buf = placed(torch, x, offset)
+    with xcorr.Plan(n_sta, 3, 70, fmt=fmt, engine="tensor") as plan:
+        xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, 70, torch.cuda.current_stream().cuda_stream)
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check(fmt, got, x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time,spare", [("ci4", 69, 40, 3000, 1 << 22), ("ci8", 69, 40, 1500, 1 << 22),
+                                                           ("ci8", 33, 3, 9000, 1 << 18), ("ci8", 129, 4, 700, 1)])
+def test_padded_rows_in_pieces(torch, fmt, n_sta, n_chan, n_time, spare):
+    """A memory limit that leaves room for a few channels, or for a part of one channel's samples."""
+    n_in = 2 * n_sta
+    x = draw(fmt, n_time, n_chan, n_sta, seed=3)
+    budget = n_chan * n_in * (n_in + 1) // 2 * 8 + 256 + spare
+    for _ in range(40):  # (the least that a plan needs beside its accumulator is the library's to say)
+        try:
+            plan = xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor", hbm_budget_bytes=budget)
+            break
+        except xcorr.XcorrError:
+            budget += 1 << 18
+    with plan:
+        assert plan.info["device_bytes"] <= budget
+        for _ in range(2):
+            plan.execute(torch.from_numpy(x).cuda())
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check(fmt, got, np.concatenate([x, x]), n_in)
+
+
+@pytest.mark.parametrize("fmt,n_sta", [("ci4", 75), ("ci4", 13), ("ci8", 75)])
+def test_padded_rows_in_graphs_and_tuned(torch, fmt, n_sta):
+    n_chan, n_time = 6, 150
+    xs = [draw(fmt, n_time, n_chan, n_sta, seed=s) for s in (1, 2)]
+    buf = torch.from_numpy(xs[0]).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor") as plan:
+        plan.autotune(buf)
+        out = plan.execute_dump(buf)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            plan.execute_dump(buf, out)
+        for k in (1, 0):
+            buf.copy_(torch.from_numpy(xs[k]))
+            out.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            check(fmt, out.cpu().numpy(), xs[k], 2 * n_sta)
+        plan.sync()

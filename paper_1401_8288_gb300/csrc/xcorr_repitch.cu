@@ -3,7 +3,7 @@
 // address off 16 bytes) is copied, still packed, to rows that do, and correlated from there.
 // Unpacking it to planes instead writes and reads two to four times the bytes and left the X-stage
 // to the slower kernels that read planes (4-bit, 338 inputs x 97 channels x 1500 samples: 120 us from
-// a ring of planes, 74 so; 122 x 300 x 2048 from planes in memory: 330, now 63; int8, 122 x 300 x 4096:
+// a ring of planes, 70 so; 122 x 300 x 2048 from planes in memory: 330, now 60; int8, 122 x 300 x 4096:
 // 716, now 290; 510 x 300 x 2048: 820, now 725).
 //
 // Bound by memory: each byte is read once and written once.
@@ -29,7 +29,6 @@ struct RepitchParams {
 // together.  (A row's last piece reads on into the next row: those inputs are never used.)  Only
 // words that hold bytes of the input are read.
 __global__ void __launch_bounds__(256) repitch_kernel(const RepitchParams p) {
-  pdl_release();
   pdl_wait();
   const uint32_t u = blockIdx.x * 256 + threadIdx.x;
   if (u >= p.units) return;

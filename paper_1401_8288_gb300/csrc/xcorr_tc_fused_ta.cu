@@ -251,12 +251,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tslot;
   const int n_items = BATCH ? p.n_batch_items : p.n_items;
-  // A launch of few items lets the next one start over its tail (64 inputs x 64 channels x 1024 samples
-  // behind its memset: 16.4 -> 13.6 us).  A long one holds it back until its own CTAs leave, which
-  // still hides the launch (256 x 256 x 1024: 73.2 -> 69.9): CTAs that start one by one as SMs come free
-  // lose the order that keeps the readers of a channel together (512 x 512 x 2048: 498 us without any
-  // of this, 502 with an early release, 492 so).
-  if (n_items <= 4 * (int)gridDim.x) pdl_release();
+  // The set-up overlaps the previous kernel's end, call after call: 64 inputs x 64 channels x 1024 samples
+  // behind its memset 16.4 -> 12.3 us, 256 x 256 x 1024 73.2 -> 69.9.  No pdl_release: short launches gain
+  // nothing from it, and CTAs that start one by one as SMs come free lose the order that keeps the
+  // readers of a channel together (512 x 512 x 2048: 498 us without any of this, 502 with it, 492 so).
   pdl_wait();
 
   if (warp == kProducerWarp) {

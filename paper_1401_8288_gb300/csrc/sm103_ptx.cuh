@@ -26,10 +26,13 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 // ------------------------------------------------------- dependent launches --
-// A kernel launched by launch_dependent (xcorr_internal.h) may start while the stream's previous
-// kernel still runs, once all of that kernel's CTAs have called pdl_release (or left).  Before
-// pdl_wait returns it must not touch global memory: then the previous kernel has completed and its
-// writes are visible.  What comes before -- barriers, tensor memory -- overlaps the previous tail.
+// A kernel launched by launch_dependent (xcorr_internal.h) may start once all CTAs of the stream's
+// previous kernel have left (or called pdl_release), before its writes are flushed.  Before pdl_wait
+// returns it must not touch global memory: then the previous kernel has completed and its writes are
+// visible.  What comes before -- the launch, barriers, tensor memory -- overlaps the previous end.
+// Only the shortest kernel releases early: CTAs of the next kernel that sit on an SM waiting keep it
+// from that kernel's own better placement (float, 16 inputs x 64 channels x 1024: unpack and X 55 us,
+// with early releases 67).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -300,6 +303,12 @@ __device__ __forceinline__ uint32_t smem_cluster(const void* p, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
   return r;
+}
+
+__device__ __forceinline__ float2 ld_cluster_f2(uint32_t cluster_addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr) : "memory");
+  return v;
 }
 
 // Arrive on a barrier of either CTA, releasing this thread's earlier writes at cluster scope.

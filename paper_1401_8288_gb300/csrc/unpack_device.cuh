@@ -56,20 +56,10 @@ __device__ __forceinline__ void window_scale(int e, float& s1, float& s2) {
   s2 = pow2i(n - a);
 }
 
-__device__ __forceinline__ void digits_of(float x, float s1, float s2, uint16_t (&d)[3]) {
-  const int m = __float2int_rn((x * s1) * s2);
-  const int d2 = ((m + 128) & 255) - 128;
-  const int m1 = (m - d2) >> 8;
-  const int d1 = ((m1 + 128) & 255) - 128;
-  const int d0 = (m1 - d1) >> 8;
-  d[0] = __bfloat16_as_ushort(__float2bfloat16_rn(static_cast<float>(d0)));
-  d[1] = __bfloat16_as_ushort(__float2bfloat16_rn(static_cast<float>(d1)));
-  d[2] = __bfloat16_as_ushort(__float2bfloat16_rn(static_cast<float>(d2)));
-}
-
 // The digits of one component of two inputs, as BF16 pairs: with M + 0x808080 the bytes are d2 + 128
-// and d1 + 128 and the upper half-word d0 + 128 (at most 256), each an exact float by the same
-// addition to 2^23 as above.  Same digits as digits_of, without its I2F and F2F conversions.
+// and d1 + 128 and the upper half-word d0 + 128 (at most 256), each an exact float when put into the
+// low mantissa bits of 2^23, and 2^23 + 128 subtracted; the upper half of that float is its BF16
+// value.  (The conversion instructions, three of each kind a component, run at an eighth of the ALU's rate.)
 __device__ __forceinline__ void digit_pairs(float x0, float s0a, float s0b, float x1, float s1a, float s1b,
                                             uint32_t (&d)[3]) {
   const uint32_t m0 = static_cast<uint32_t>(__float2int_rn((x0 * s0a) * s0b)) + 0x808080u;

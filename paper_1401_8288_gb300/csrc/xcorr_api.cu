@@ -318,20 +318,27 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     const int G = tensor_groups(plan);
     const int per = (C + G - 1) / G;
     const int nxs = plan->tune_x_streams == 1 ? 1 : 2;
-    // fork: the internal streams start after everything queued on s so far
-    if ((e = cudaEventRecord(plan->ev_fork, s)) != cudaSuccess) return cuda_fail(e, "fork event");
-    if ((e = cudaStreamWaitEvent(plan->s_unpack, plan->ev_fork, 0)) != cudaSuccess ||
-        (e = cudaStreamWaitEvent(plan->s_x[0], plan->ev_fork, 0)) != cudaSuccess ||
-        (e = cudaStreamWaitEvent(plan->s_x[1], plan->ev_fork, 0)) != cudaSuccess)
-      return cuda_fail(e, "fork wait");
+    // several groups: the internal streams fork from s after everything queued on it so far (one
+    // group's two launches follow one another on s itself)
+    const bool forked = per < C;
+    cudaStream_t su = forked ? plan->s_unpack : s;
+    if (forked) {
+      if ((e = cudaEventRecord(plan->ev_fork, s)) != cudaSuccess) return cuda_fail(e, "fork event");
+      if ((e = cudaStreamWaitEvent(plan->s_unpack, plan->ev_fork, 0)) != cudaSuccess ||
+          (e = cudaStreamWaitEvent(plan->s_x[0], plan->ev_fork, 0)) != cudaSuccess ||
+          (e = cudaStreamWaitEvent(plan->s_x[1], plan->ev_fork, 0)) != cudaSuccess)
+        return cuda_fail(e, "fork wait");
+    }
     int used = 0;
     for (int g = 0, c0 = 0; c0 < C; ++g, c0 += per) {
       const int nc = (C - c0 < per) ? C - c0 : per;
-      if ((e = unpack_group(plan, d_in, n_time, c0, nc, plan->s_unpack)) != cudaSuccess)
-        return cuda_fail(e, "unpack launch");
-      if ((e = cudaEventRecord(plan->ev_unpacked[g], plan->s_unpack)) != cudaSuccess) return cuda_fail(e, "event");
-      cudaStream_t sx = plan->s_x[g % nxs];
-      if ((e = cudaStreamWaitEvent(sx, plan->ev_unpacked[g], 0)) != cudaSuccess) return cuda_fail(e, "wait");
+      if ((e = unpack_group(plan, d_in, n_time, c0, nc, su)) != cudaSuccess) return cuda_fail(e, "unpack launch");
+      cudaStream_t sx = forked ? plan->s_x[g % nxs] : s;
+      if (forked) {
+        if ((e = cudaEventRecord(plan->ev_unpacked[g], su)) != cudaSuccess) return cuda_fail(e, "event");
+        if ((e = cudaStreamWaitEvent(sx, plan->ev_unpacked[g], 0)) != cudaSuccess) return cuda_fail(e, "wait");
+      }
+      if (ev && !forked && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return cuda_fail(e, "profile event");
       if (ev && (e = cudaEventRecord(ev[2 + 2 * g], sx)) != cudaSuccess) return cuda_fail(e, "profile event");
       L.chan0 = c0;
       L.n_chan = nc;
@@ -340,9 +347,9 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
       if (ev && (e = cudaEventRecord(ev[3 + 2 * g], sx)) != cudaSuccess) return cuda_fail(e, "profile event");
       used = g + 1;
     }
-    if (ev && (e = cudaEventRecord(ev[1], plan->s_unpack)) != cudaSuccess) return cuda_fail(e, "profile event");
+    if (ev && forked && (e = cudaEventRecord(ev[1], su)) != cudaSuccess) return cuda_fail(e, "profile event");
     // join: s continues after both X streams (which waited for every unpack)
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; forked && k < 2; ++k) {
       if ((e = cudaEventRecord(plan->ev_x_done[k], plan->s_x[k])) != cudaSuccess ||
           (e = cudaStreamWaitEvent(s, plan->ev_x_done[k], 0)) != cudaSuccess)
         return cuda_fail(e, "join");

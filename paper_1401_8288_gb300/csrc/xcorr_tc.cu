@@ -89,6 +89,7 @@ struct TcParams {
   int n_pairs_k;      // plane pairs on the K axis
   int spw;            // stages per time window
   int n_tw;           // time windows
+  int split;          // SPLIT: CTAs of a cluster, which share the blocks of one tile pair
   int planes_per_chan;
   int64_t n_pairs;
   int accumulate_first;  // the first block adds into out (else it stores)
@@ -157,7 +158,15 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t
     mma_f16(d, a, b, id, acc);
 }
 
-template <int ESIZE, int KT, int STAGES, bool FLOAT_OUT, bool BATCH>
+// The drained blocks (window, pair) of a tile pair that this CTA takes: all, or with SPLIT its share.
+template <bool SPLIT>
+__device__ __forceinline__ void block_range(const TcParams& p, int n_blocks, int& b0, int& b1) {
+  const int rank = SPLIT ? static_cast<int>(cluster_ctarank()) : 0, n = SPLIT ? p.split : 1;
+  b0 = n_blocks * rank / n;
+  b1 = n_blocks * (rank + 1) / n;
+}
+
+template <int ESIZE, int KT, int STAGES, bool FLOAT_OUT, bool BATCH, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     xcorr_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ TcParams p) {
   using G = Geometry<ESIZE, KT, STAGES>;
@@ -192,8 +201,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_wait();
 
   const int n_items = BATCH ? p.n_batch_items : p.n_chan * p.n_tile_pairs;
+  const int item0 = SPLIT ? static_cast<int>(blockIdx.x) / p.split : static_cast<int>(blockIdx.x);
+  const int item_step = SPLIT ? n_items : static_cast<int>(gridDim.x);
 
   if (warp == kProducerWarp) {
     if (lane == 0) {
@@ -201,13 +213,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       int s = 0;
       uint32_t ph = 0, filled = 0, fill_parity[STAGES] = {};
       bool ok = true;
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
+      for (int item = item0; ok && item < n_items; item += item_step) {
         ItemView v;
         view_item<BATCH>(p, &tmap, item, v);
         const int zc = v.zc, I = v.I, J = v.J;
         const int half = p.planes_per_chan / 2;  // re planes, then im planes
-        const int n_blocks = v.n_tw * p.n_pairs_k;  // drained blocks: (window, pair)
-        for (int blk = 0; ok && blk < n_blocks; ++blk) {
+        int b0, b1;
+        block_range<SPLIT>(p, v.n_tw * p.n_pairs_k, b0, b1);
+        for (int blk = b0; ok && blk < b1; ++blk) {
           const int w = blk / p.n_pairs_k, pk = blk - w * p.n_pairs_k;
           const int pp = p.pair_p[pk], pq = p.pair_q[pk];
           const bool shared = (I == J) && (pp == pq);
@@ -255,12 +268,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t ph = 0;
       int g = 0;  // windows processed by this CTA
       bool ok = true;
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
+      for (int item = item0; ok && item < n_items; item += item_step) {
         ItemView v;
         view_item<BATCH>(p, &tmap, item, v);
         const int I = v.I, J = v.J;
-        const int n_blocks = v.n_tw * p.n_pairs_k;
-        for (int blk = 0; ok && blk < n_blocks; ++blk, ++g) {
+        int b0, b1;
+        block_range<SPLIT>(p, v.n_tw * p.n_pairs_k, b0, b1);
+        for (int blk = b0; ok && blk < b1; ++blk, ++g) {
           const int w = blk / p.n_pairs_k, pk = blk - w * p.n_pairs_k;
           const bool shared = (I == J) && (p.pair_p[pk] == p.pair_q[pk]);
           const int buf = g & 1;
@@ -316,11 +330,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int quarter = warp & 3, colh = warp >> 2;
     int g = 0;
     bool ok = true;
-    for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
+    for (int item = item0; ok && item < n_items; item += item_step) {
       ItemView v;
       view_item<BATCH>(p, &tmap, item, v);
       const int n_inputs = v.n_inputs;
-      const int n_blocks = v.n_tw * p.n_pairs_k;
+      int b0, b1;
+      block_range<SPLIT>(p, v.n_tw * p.n_pairs_k, b0, b1);
       uint2* out_c = v.out_c;
       const int row0 = v.I * kBlk + quarter * 32;  // first global input row of this warp
       const int col0 = v.J * kBlk + colh * kCols;  // first global input column of this warp
@@ -328,7 +343,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       Acc acc_re[kCols], acc_im[kCols];
 #pragma unroll
       for (int q = 0; q < kCols; ++q) acc_re[q] = acc_im[q] = Acc(0);
-      for (int blk = 0; blk < n_blocks; ++blk, ++g) {
+      for (int blk = b0; blk < b1; ++blk, ++g) {
         const int buf = g & 1;
         const uint32_t use = static_cast<uint32_t>(g >> 1);
         if (!mbar_wait_warp(&tfull[buf], use & 1u, abort_flag, p.status, DEV_TIMEOUT_TMEM_FULL)) {
@@ -398,6 +413,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[buf]);
       }
+      if (SPLIT) {
+        // The CTA's part of the sums, column by column, where its stages were (its MMAs have read
+        // them all); after the barrier each CTA adds up and writes every split-th step of columns.
+        if (ok && live) {
+          float2* part = reinterpret_cast<float2*>(stages) + colh * kCols * kBlk + quarter * 32 + lane;
+#pragma unroll
+          for (int q = 0; q < kCols; ++q)
+            part[q * kBlk] = make_float2(static_cast<float>(acc_re[q]), static_cast<float>(acc_im[q]));
+        }
+        cluster_sync();
+      }
       if (!ok || !live) continue;
       // Write the finished tile rows.  Per 8-column step a quarter-warp writes
       // 8 consecutive pairs of one row (64 bytes); when adding into earlier
@@ -406,6 +432,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int sub = lane >> 3, col = lane & 7;
 #pragma unroll
       for (int ch = 0; ch < kCols / kChunk; ++ch) {
+        if (SPLIT) {
+          if (ch % p.split != static_cast<int>(cluster_ctarank())) continue;
+#pragma unroll
+          for (int q = 0; q < kChunk; ++q) acc_re[ch * kChunk + q] = acc_im[ch * kChunk + q] = Acc(0);
+          for (int c = 0; c < p.split; ++c) {  // in rank order: the same sum in every run
+            const uint32_t part = smem_cluster(
+                reinterpret_cast<float2*>(stages) + (colh * kCols + ch * kChunk) * kBlk + quarter * 32 + lane, c);
+#pragma unroll
+            for (int q = 0; q < kChunk; ++q) {
+              const float2 s = ld_cluster_f2(part + q * kBlk * 8);
+              acc_re[ch * kChunk + q] += s.x;
+              acc_im[ch * kChunk + q] += s.y;
+            }
+          }
+        }
 #pragma unroll
         for (int q = 0; q < kChunk; ++q) {
           Acc vr = acc_re[ch * kChunk + q], vi = acc_im[ch * kChunk + q];
@@ -451,6 +492,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
 
+  if (SPLIT) {
+    __syncwarp();
+    if (warp >= kEpiWarps) cluster_sync();  // the epilogue warps' barrier before their sums are read
+    cluster_sync();                         // no CTA leaves while its part may be read
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == kMmaWarp) {
@@ -460,11 +506,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // One instantiation per (operand type, stage variant, output type) in use.
-template <int ESIZE, int V, bool FLOAT_OUT, bool BATCH = false>
+template <int ESIZE, int V, bool FLOAT_OUT, bool BATCH = false, bool SPLIT = false>
 cudaError_t launch_variant(const CUtensorMap* tmap, const TcParams& p, int grid, cudaStream_t stream) {
   constexpr int KT = stage_rows_of(V, ESIZE), S = stages_of(V);
   using G = Geometry<ESIZE, KT, S>;
-  auto kern = xcorr_tc_kernel<ESIZE, KT, S, FLOAT_OUT, BATCH>;
+  static_assert(!SPLIT || S * G::kStageBytes >= kBlk * kBlk * 8, "a CTA's part fits its stages");
+  auto kern = xcorr_tc_kernel<ESIZE, KT, S, FLOAT_OUT, BATCH, SPLIT>;
   static int attr_device = -1;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -474,8 +521,8 @@ cudaError_t launch_variant(const CUtensorMap* tmap, const TcParams& p, int grid,
     if (e != cudaSuccess) return e;
     attr_device = dev;
   }
-  kern<<<grid, kThreads, G::kSmemBytes, stream>>>(*tmap, p);
-  return cudaGetLastError();
+  return launch_dependent_clusters(kern, SPLIT ? p.split : 1, SPLIT ? grid * p.split : grid, kThreads, G::kSmemBytes,
+                                   stream, *tmap, p);
 }
 
 }  // namespace
@@ -540,6 +587,17 @@ cudaError_t launch_xcorr_tc(const CUtensorMap* tmap, const TcLaunch& L, cudaStre
     }
   }
   if (!L.float_out) return cudaErrorInvalidValue;
+  // Few tile pairs: clusters of 2, 4 or 8 CTAs share the blocks of each while that keeps every CTA on
+  // an SM of its own (128 inputs x 64 channels x 1024 samples: 79 -> 54 us).
+  p.split = 1;
+  while (p.split < 8 && items * 2 * p.split <= L.num_sms && 2 * p.split <= p.n_tw * p.n_pairs_k) p.split *= 2;
+  if (p.split > 1) {
+    switch (L.variant) {
+      case 0: return launch_variant<2, 0, true, false, true>(tmap, p, grid, stream);
+      case 1: return launch_variant<2, 1, true, false, true>(tmap, p, grid, stream);
+      default: return launch_variant<2, 2, true, false, true>(tmap, p, grid, stream);
+    }
+  }
   switch (L.variant) {
     case 0: return launch_variant<2, 0, true>(tmap, p, grid, stream);
     case 1: return launch_variant<2, 1, true>(tmap, p, grid, stream);

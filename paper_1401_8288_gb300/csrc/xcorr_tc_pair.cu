@@ -59,7 +59,7 @@
 // 300 channels x 4096, float: 1.11 ms against 1.29 here).  4-bit input comes here when planes are asked
 // for, or under a memory limit too tight for padded rows: otherwise it stays with the fused kernel (492
 // us against about 600 here at 512 inputs x 512 channels x 2048 samples: its L2 traffic is the raw
-// bytes), over padded rows where its own are not aligned (74 against 119 us at 338 x 97 x 1500).  int8
+// bytes), over padded rows where its own are not aligned (70 against 119 us at 338 x 97 x 1500).  int8
 // input goes to xcorr_tc_raw_pair.cu (0.87 ms against 1.00 with BF16 planes here).
 //
 // Warp roles (512 threads, one CTA per SM): warps 0-7 drain TMEM into running

@@ -13,6 +13,7 @@
 
 #include <cstring>
 
+#include "sm103_ptx.cuh"
 #include "unpack_device.cuh"
 #include "xcorr_internal.h"
 
@@ -267,183 +268,128 @@ bool encode_raw_ci4_packed_tmap(CUtensorMap* map, const void* in, int n_inputs, 
 // ----------------------------------------------------- float input --
 namespace {
 
-// Any 4-byte aligned input: the components are read as single floats.
-__global__ void __launch_bounds__(256) unpack_cf32_digits_kernel(const float* __restrict__ in,
-                                                                 uint16_t* __restrict__ planes,
-                                                                 int16_t* __restrict__ exps, int n_time, int n_chan,
-                                                                 int c0, int nc, int n_inputs, int ni_pad,
-                                                                 int64_t comp_stride, int window, int exp_windows) {
-  const int n_w = (n_time + window - 1) / window;
-  const int64_t total = (int64_t)nc * n_w * n_inputs;
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int i = static_cast<int>(q % n_inputs);
-    const int64_t rest = q / n_inputs;
-    const int w = static_cast<int>(rest % n_w);
-    const int c = c0 + static_cast<int>(rest / n_w);
-    const int t0 = w * window, t1 = min(n_time, t0 + window);
-    uint32_t mb = 0u;
-#pragma unroll 8
-    for (int t = t0; t < t1; ++t) {
-      const float* v = in + 2 * (((int64_t)t * n_chan + c) * n_inputs + i);
-      mb = max(mb, max(abs_bits(__ldg(v)), abs_bits(__ldg(v + 1))));
-    }
-    const int e = window_exponent(mb);
-    exps[((int64_t)c * exp_windows + w) * ni_pad + i] = static_cast<int16_t>(e);
-    float s1, s2;
-    window_scale(e, s1, s2);
-    uint16_t* base = planes + (6 * (int64_t)c) * comp_stride + i;
-#pragma unroll 4
-    for (int t = t0; t < t1; ++t) {
-      const float* v = in + 2 * (((int64_t)t * n_chan + c) * n_inputs + i);
-      uint16_t dr[3], dm[3];
-      digits_of(__ldg(v), s1, s2, dr);
-      digits_of(__ldg(v + 1), s1, s2, dm);
-      uint16_t* row = base + (int64_t)t * ni_pad;
-#pragma unroll
-      for (int pc = 0; pc < 3; ++pc) {
-        row[pc * comp_stride] = dr[pc];
-        row[(3 + pc) * comp_stride] = dm[pc];
-      }
-    }
-  }
-}
-
-// As unpack_cf32_digits_kernel for two neighbouring inputs per thread (an even
-// input count and a 16-byte aligned input): 16-byte loads of (re, im) pairs and
-// 4-byte stores of two digits, half the instructions per byte.
-__global__ void __launch_bounds__(256) unpack_cf32_digits_x2_kernel(const float4* __restrict__ in,
-                                                                    uint16_t* __restrict__ planes,
-                                                                    int16_t* __restrict__ exps, int n_time,
-                                                                    int n_chan, int c0, int nc, int n_inputs,
-                                                                    int ni_pad, int64_t comp_stride, int window,
-                                                                    int exp_windows) {
-  const int n_w = (n_time + window - 1) / window;
-  const int half = n_inputs / 2;
-  const int64_t total = (int64_t)nc * n_w * half;
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int i2 = static_cast<int>(q % half);
-    const int64_t rest = q / half;
-    const int w = static_cast<int>(rest % n_w);
-    const int c = c0 + static_cast<int>(rest / n_w);
-    const int t0 = w * window, t1 = min(n_time, t0 + window);
-    const float4* col = in + (int64_t)c * half + i2;  // inputs 2 i2, 2 i2 + 1 of channel c, time 0
-    const int64_t row_step = (int64_t)n_chan * half;  // float4s from one sample to the next
-    uint32_t mb0 = 0u, mb1 = 0u;
-#pragma unroll 8
-    for (int t = t0; t < t1; ++t) {
-      const float4 v = __ldg(col + t * row_step);
-      mb0 = max(mb0, max(abs_bits(v.x), abs_bits(v.y)));
-      mb1 = max(mb1, max(abs_bits(v.z), abs_bits(v.w)));
-    }
-    const int e0 = window_exponent(mb0), e1 = window_exponent(mb1);
-    int16_t* ex = exps + ((int64_t)c * exp_windows + w) * ni_pad + 2 * i2;
-    ex[0] = static_cast<int16_t>(e0);
-    ex[1] = static_cast<int16_t>(e1);
-    float s0a, s0b, s1a, s1b;
-    window_scale(e0, s0a, s0b);
-    window_scale(e1, s1a, s1b);
-    uint32_t* base = reinterpret_cast<uint32_t*>(planes + (6 * (int64_t)c) * comp_stride + 2 * i2);
-    const int64_t cs = comp_stride / 2;  // in uint32 units (comp_stride is a multiple of 16)
-#pragma unroll 4
-    for (int t = t0; t < t1; ++t) {
-      const float4 v = __ldg(col + t * row_step);
-      uint16_t r0[3], m0[3], r1[3], m1[3];
-      digits_of(v.x, s0a, s0b, r0);
-      digits_of(v.y, s0a, s0b, m0);
-      digits_of(v.z, s1a, s1b, r1);
-      digits_of(v.w, s1a, s1b, m1);
-      uint32_t* row = base + (int64_t)t * (ni_pad / 2);
-#pragma unroll
-      for (int pc = 0; pc < 3; ++pc) {
-        row[pc * cs] = r0[pc] | (static_cast<uint32_t>(r1[pc]) << 16);
-        row[(3 + pc) * cs] = m0[pc] | (static_cast<uint32_t>(m1[pc]) << 16);
-      }
-    }
-  }
-}
-
-// Float input read once: a CTA stages one (channel, window, 32 inputs) slice -- the window's
-// samples x 32 inputs x 8 bytes, 96 KB for a 384-sample window -- in shared memory with 16-byte
-// asynchronous copies (each time row of the slice is 256 contiguous bytes), takes each input's window maximum
-// from it, then writes the digits from it.  The two-read kernels above read every float twice
-// from HBM: with a CTA per (channel, window, 256 input pairs) the slices in flight far exceed
-// L2.  Here two CTAs of 256 threads share an SM, so one loads while the other converts.  Thread
-// (pair q, time group g) handles inputs 2q, 2q + 1 of the slice at samples g, g + 16, ...; a warp
-// covers two time rows of 16 pairs (512 contiguous bytes), conflict-free.  Needs n_inputs % 32
-// == 0 and a 16-byte aligned input; same arithmetic as the other kernels, so the same results.
-constexpr int kTileInputs = 32;
-constexpr int kTilePairs = kTileInputs / 2;
+// Float input read once: a CTA stages one (window, 16 columns) slice in shared memory -- a column is a
+// pair of neighbouring inputs of one channel, 16 bytes a sample; the slice is two units of 8 columns,
+// whose digits fill whole 32-byte sectors of the planes' rows (columns that ran on through the
+// channels of an input count that is no multiple of 16 took 494 us with the X kernel for 122 x 300 x
+// 1024, now 345; kernels that read the input twice, 595) -- by asynchronous copies, takes each input's window maximum from it, then writes the digits from it.  Two CTAs of 256
+// threads share an SM, so one loads while the other converts.  Thread (column q, time group g) handles
+// samples g, g + 16, ...; a warp covers two time rows of 16 columns, conflict-free.
+//
+// Bound by memory: 8 bytes read and 12 written per sample (128 inputs x 64 channels x 1024 samples: 40
+// us with conversion instructions for the digits, which run at an eighth of the ALU's rate, now 28).
+// ALIGNED: a 16-byte aligned input, one copy per pair; else (a 4-byte aligned one) four.
+constexpr int kTileCols = 16;
+constexpr int kUnitCols = 8;
 constexpr int kTileGroups = 16;
-constexpr int kTileThreads = kTilePairs * kTileGroups;
-__global__ void __launch_bounds__(kTileThreads, 2) unpack_cf32_digits_tile_kernel(
-    const float4* __restrict__ in, uint16_t* __restrict__ planes, int16_t* __restrict__ exps, int n_time, int n_chan,
+constexpr int kTileThreads = kTileCols * kTileGroups;
+template <bool ALIGNED>
+__global__ void __launch_bounds__(kTileThreads, 2) unpack_cf32_digits_kernel(
+    const float* __restrict__ in, uint16_t* __restrict__ planes, int16_t* __restrict__ exps, int n_time, int n_chan,
     int c0, int nc, int n_inputs, int ni_pad, int64_t comp_stride, int window, int exp_windows) {
-  extern __shared__ float4 slice[];  // [window][kTilePairs]
-  __shared__ uint32_t part[2][kTileGroups][kTilePairs];
-  __shared__ int win_e[2][kTilePairs];
+  extern __shared__ float4 slice[];  // [window][kTileCols]
+  __shared__ uint32_t part[2][kTileGroups][kTileCols];
+  __shared__ int win_e[2][kTileCols];
+  pdl_wait();
   const int n_w = (n_time + window - 1) / window;
-  const int n_groups = n_inputs / kTileInputs;
   const int half = n_inputs / 2;
-  const int q = threadIdx.x % kTilePairs, g = threadIdx.x / kTilePairs;
-  for (int64_t blk = blockIdx.x; blk < (int64_t)nc * n_w * n_groups; blk += gridDim.x) {
-    const int ig = static_cast<int>(blk % n_groups);
-    const int64_t rest = blk / n_groups;
-    const int w = static_cast<int>(rest % n_w);
-    const int c = c0 + static_cast<int>(rest / n_w);
+  const int per_chan = (half + kUnitCols - 1) / kUnitCols;  // units of one channel
+  const int64_t n_units = (int64_t)nc * per_chan;
+  // slices: the units of one channel (of two, for an odd number of units), then the windows, then the channels
+  const int chans = per_chan % 2 ? 2 : 1, per_step = per_chan * chans / 2;
+  const int64_t n_slices = (int64_t)((nc + chans - 1) / chans) * n_w * per_step;
+  const int q = threadIdx.x % kTileCols, g = threadIdx.x / kTileCols;
+  for (int64_t blk = blockIdx.x; blk < n_slices; blk += gridDim.x) {
+    const int64_t step = blk / per_step;
+    const int w = static_cast<int>(step % n_w);
+    const int64_t unit = step / n_w * per_chan * chans + 2 * (blk - step * per_step) + q / kUnitCols;
+    const int cc = static_cast<int>(unit / per_chan), col = static_cast<int>(unit % per_chan) * kUnitCols + q % kUnitCols;
+    const bool have = unit < n_units && col < half;
+    const int c = c0 + cc, i = 2 * col;
     const int t0 = w * window, len = min(n_time, t0 + window) - t0;
-    // the slice's rows into shared memory, once: asynchronous 16-byte copies, all of a thread's
-    // rows in flight together
-    const float4* col = in + (int64_t)c * half + ig * kTilePairs + q;
-    const int64_t row_step = (int64_t)n_chan * half;
-    for (int r = g; r < len; r += kTileGroups) {
-      const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&slice[r * kTilePairs + q]));
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(col + (t0 + r) * row_step)
-                   : "memory");
+    // the slice's rows, all of a thread's copies in flight together
+    const float* src = in + (((int64_t)t0 * n_chan + c) * n_inputs + i) * 2;
+    const int64_t row_step = (int64_t)n_chan * n_inputs * 2;
+    if (have) {
+      for (int r = g; r < len; r += kTileGroups) {
+        const uint32_t dst = smem_u32(&slice[r * kTileCols + q]);
+        if (ALIGNED) {
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + r * row_step) : "memory");
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * k), "l"(src + r * row_step + k)
+                         : "memory");
+        }
+      }
     }
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     uint32_t mb0 = 0u, mb1 = 0u;
-    for (int r = g; r < len; r += kTileGroups) {
-      const float4 v = slice[r * kTilePairs + q];
-      mb0 = max(mb0, max(abs_bits(v.x), abs_bits(v.y)));
-      mb1 = max(mb1, max(abs_bits(v.z), abs_bits(v.w)));
+    if (have) {
+      for (int r = g; r < len; r += kTileGroups) {
+        const float4 v = slice[r * kTileCols + q];
+        mb0 = max(mb0, max(abs_bits(v.x), abs_bits(v.y)));
+        mb1 = max(mb1, max(abs_bits(v.z), abs_bits(v.w)));
+      }
     }
     part[0][g][q] = mb0;
     part[1][g][q] = mb1;
     __syncthreads();
-    if (threadIdx.x < 2 * kTilePairs) {
-      const int k = threadIdx.x / kTilePairs, pq = threadIdx.x % kTilePairs;
+    if (threadIdx.x < 2 * kTileCols) {  // thread (k, q): input k of its own column
+      const int k = threadIdx.x / kTileCols;
       uint32_t m = 0u;
 #pragma unroll
-      for (int gg = 0; gg < kTileGroups; ++gg) m = max(m, part[k][gg][pq]);
+      for (int gg = 0; gg < kTileGroups; ++gg) m = max(m, part[k][gg][q]);
       const int e = window_exponent(m);
-      win_e[k][pq] = e;
-      exps[((int64_t)c * exp_windows + w) * ni_pad + ig * kTileInputs + 2 * pq + k] = static_cast<int16_t>(e);
+      win_e[k][q] = e;
+      if (have) exps[((int64_t)c * exp_windows + w) * ni_pad + i + k] = static_cast<int16_t>(e);
     }
     __syncthreads();
     float s0a, s0b, s1a, s1b;
     window_scale(win_e[0][q], s0a, s0b);
     window_scale(win_e[1][q], s1a, s1b);
-    uint32_t* base = reinterpret_cast<uint32_t*>(planes + (6 * (int64_t)c) * comp_stride + ig * kTileInputs + 2 * q);
+    uint32_t* base = reinterpret_cast<uint32_t*>(planes + (6 * (int64_t)c) * comp_stride + i);
     const int64_t cs = comp_stride / 2;  // in uint32 units (comp_stride is a multiple of 16)
-    for (int r = g; r < len; r += kTileGroups) {
-      const float4 v = slice[r * kTilePairs + q];
-      uint16_t r0[3], m0[3], r1[3], m1[3];
-      digits_of(v.x, s0a, s0b, r0);
-      digits_of(v.y, s0a, s0b, m0);
-      digits_of(v.z, s1a, s1b, r1);
-      digits_of(v.w, s1a, s1b, m1);
-      uint32_t* row = base + (int64_t)(t0 + r) * (ni_pad / 2);
+    if (have) {
+      for (int r = g; r < len; r += kTileGroups) {
+        const float4 v = slice[r * kTileCols + q];
+        uint32_t re[3], im[3];
+        digit_pairs(v.x, s0a, s0b, v.z, s1a, s1b, re);
+        digit_pairs(v.y, s0a, s0b, v.w, s1a, s1b, im);
+        uint32_t* row = base + (int64_t)(t0 + r) * (ni_pad / 2);
 #pragma unroll
-      for (int pc = 0; pc < 3; ++pc) {
-        row[pc * cs] = r0[pc] | (static_cast<uint32_t>(r1[pc]) << 16);
-        row[(3 + pc) * cs] = m0[pc] | (static_cast<uint32_t>(m1[pc]) << 16);
+        for (int pc = 0; pc < 3; ++pc) {
+          row[pc * cs] = re[pc];
+          row[(3 + pc) * cs] = im[pc];
+        }
       }
     }
     __syncthreads();  // the slice is refilled by the next block of work
   }
+}
+
+template <bool ALIGNED>
+cudaError_t launch_cf32_digits(const float* in, uint16_t* planes, int16_t* exps, int n_time, int n_chan, int c0, int nc,
+                               int n_inputs, int ni_pad, int max_time, int window, int exp_windows,
+                               cudaStream_t stream) {
+  const size_t smem = (size_t)window * kTileCols * sizeof(float4);
+  static int attr_device = -1;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && attr_device != dev) {
+    e = cudaFuncSetAttribute(unpack_cf32_digits_kernel<ALIGNED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
+    if (e == cudaSuccess) attr_device = dev;
+  }
+  if (e != cudaSuccess) return e;
+  const int per_chan = (n_inputs / 2 + kUnitCols - 1) / kUnitCols, chans = per_chan % 2 ? 2 : 1;
+  const int64_t slices =
+      (int64_t)((nc + chans - 1) / chans) * ((n_time + window - 1) / window) * (per_chan * chans / 2);
+  const unsigned grid = static_cast<unsigned>(slices < 2LL * sms ? slices : 2LL * sms);
+  return launch_dependent(unpack_cf32_digits_kernel<ALIGNED>, grid, kTileThreads, smem, stream, in, planes, exps, n_time,
+                          n_chan, c0, nc, n_inputs, ni_pad, (int64_t)max_time * ni_pad, window, exp_windows);
 }
 
 }  // namespace
@@ -451,41 +397,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) unpack_cf32_digits_tile_kerne
 cudaError_t launch_unpack_cf32_digits(const float* in, uint16_t* planes, int16_t* exps, int n_time, int n_chan,
                                       int c0, int nc, int n_inputs, int ni_pad, int max_time, int window,
                                       int exp_windows, cudaStream_t stream) {
-  const int64_t comp_stride = (int64_t)max_time * ni_pad;
-  if (n_inputs % kTileInputs == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) {
-    // read once through shared memory: 2 CTAs per SM, each looping over its slices
-    const size_t smem = (size_t)window * kTilePairs * sizeof(float4);
-    static int attr_device = -1;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess && attr_device != dev) {
-      e = cudaFuncSetAttribute(unpack_cf32_digits_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem);
-      if (e == cudaSuccess) attr_device = dev;
-    }
-    if (e != cudaSuccess) return e;
-    const int64_t slices = (int64_t)nc * ((n_time + window - 1) / window) * (n_inputs / kTileInputs);
-    const int64_t grid = slices < 2LL * sms ? slices : 2LL * sms;
-    unpack_cf32_digits_tile_kernel<<<(unsigned)grid, kTileThreads, smem, stream>>>(
-        reinterpret_cast<const float4*>(in), planes, exps, n_time, n_chan, c0, nc, n_inputs, ni_pad, comp_stride,
-        window, exp_windows);
-    return cudaGetLastError();
-  }
-  const bool x2 = n_inputs % 2 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;
-  const int64_t work = (int64_t)nc * ((n_time + window - 1) / window) * (x2 ? n_inputs / 2 : n_inputs);
-  int64_t blocks = (work + 255) / 256;
-  if (blocks < 1) blocks = 1;
-  if (blocks > (1 << 20)) blocks = 1 << 20;
-  if (x2)
-    unpack_cf32_digits_x2_kernel<<<(unsigned)blocks, 256, 0, stream>>>(
-        reinterpret_cast<const float4*>(in), planes, exps, n_time, n_chan, c0, nc, n_inputs, ni_pad, comp_stride,
-        window, exp_windows);
-  else
-    unpack_cf32_digits_kernel<<<(unsigned)blocks, 256, 0, stream>>>(in, planes,
-                                                                    exps, n_time, n_chan, c0, nc, n_inputs, ni_pad,
-                                                                    comp_stride, window, exp_windows);
-  return cudaGetLastError();
+  return (reinterpret_cast<uintptr_t>(in) % 16 == 0 ? launch_cf32_digits<true> : launch_cf32_digits<false>)(
+      in, planes, exps, n_time, n_chan, c0, nc, n_inputs, ni_pad, max_time, window, exp_windows, stream);
 }
 
 }  // namespace xc

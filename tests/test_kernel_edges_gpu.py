@@ -311,3 +311,47 @@ def test_padded_rows_in_graphs_and_tuned(torch, fmt, n_sta):
             torch.cuda.synchronize()
             check(fmt, out.cpu().numpy(), xs[k], 2 * n_sta)
         plan.sync()
+
+
+# --------------------------------------------- float input of one tile: any address, shared blocks ---
+@pytest.mark.parametrize("n_sta,n_chan,n_time,offset", [(1, 1, 1, 0), (1, 3, 385, 4), (4, 16, 384, 0), (7, 5, 800, 8), (9, 30, 383, 12), (16, 19, 1153, 0),
+                                                        (33, 38, 769, 0), (61, 2, 1536, 4), (64, 9, 100, 0), (64, 76, 400, 0), (63, 77, 390, 8),
+                                                        (64, 160, 385, 0)])
+@pytest.mark.parametrize("variant", [0, 1, 2])
+def test_float_one_tile(torch, variant, n_sta, n_chan, n_time, offset):
+    """Clusters of 8, 4, 2 and single CTAs per tile, columns that end inside a slice of 16, windows that
+    end inside a stage, every 4-byte address; a store, then an adding execute; equal in two runs."""
+    x = draw("cf32", n_time, n_chan, n_sta, seed=n_sta + n_time)
+    buf = placed(torch, x, offset)
+    got = []
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="cf32") as plan:
+        plan.set_tuning(variant, 0, 2, 0)
+        for _ in range(2):
+            for _ in range(2):
+                xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, n_time, torch.cuda.current_stream().cuda_stream)
+            got.append(plan.dump().cpu().numpy())
+            plan.sync()
+    assert np.array_equal(got[0], got[1])
+    check("cf32", got[0], np.concatenate([x, x]), 2 * n_sta)
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, 1e-40])
+def test_float_one_tile_edges(torch, value):
+    """One non-finite or subnormal sample: its input's visibilities, and no other's."""
+    n_sta, n_chan, n_time = 19, 4, 800
+    x = draw("cf32", n_time, n_chan, n_sta, seed=5)
+    x[401, 2, 7, 1, 0] = value
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="cf32") as plan:
+        got = plan.execute_dump(torch.from_numpy(x).cuda()).cpu().numpy()
+        plan.sync()
+    ii, jj = np.tril_indices(2 * n_sta)
+    hit = np.zeros(got.shape[:2], dtype=bool)
+    if not np.isfinite(value):
+        hit[2] = (ii == 15) | (jj == 15)
+        assert not np.isfinite(got[hit]).any()
+        x[401, 2, 7, 1, 0] = 0
+    want = oracle.correlate(oracle.FMT_CF32, x)
+    autos = want[:, np.arange(2 * n_sta) * (np.arange(2 * n_sta) + 3) // 2, 0]
+    scale = np.sqrt(autos[:, ii] * autos[:, jj])
+    err = np.abs((got[..., 0] - want[..., 0]) + 1j * (got[..., 1] - want[..., 1]))
+    assert (err[~hit] <= 1e-6 * scale[~hit]).all()

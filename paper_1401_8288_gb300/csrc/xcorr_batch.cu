@@ -4,9 +4,12 @@
 // A batch holds n subarrays (each its own station count, channel count and
 // integration length, 4+4-bit input).  One execute runs a single launch of an
 // X kernel over the union of their work items (subarray, channel, I, J),
-// sorted longest first and dealt round-robin to the persistent CTAs, so a
-// large subarray's tail is filled with the small ones' items instead of
-// leaving SMs idle between per-instance launches.  Sec. 2.1: each sub-band
+// sorted longest first and dealt evenly to the persistent CTAs, so a large
+// subarray's tail is filled with the small ones' items instead of leaving SMs
+// idle between per-instance launches.  The fused kernel's items of a subarray
+// of at most 64 inputs hold several channels side by side (24 subarrays of 8
+// to 128 stations: 161 us a pass with a tile per channel, dealt round-robin;
+// 125 with both).  Sec. 2.1: each sub-band
 // (here each subarray) is an independent X-stage.
 //
 // Stage variants 3-5 (the default when every subarray has a multiple of 16
@@ -126,6 +129,31 @@ xcorr_status ensure_planes(xcorr_batch b) {
   return XCORR_OK;
 }
 
+// Items run on CTA (index % CTAs), round after round, longest first.  Dealt in that order the first
+// CTAs get the longest item of every round; here each round's longest goes to the CTA with the least
+// so far (24 subarrays of 8 to 128 stations: 139 stages on the busiest CTA instead of 148, of 134 on
+// average).  An item costs its stages and about two more to set up and write out.
+constexpr int kItemOverhead = 2;
+void deal(uint4* items, const std::vector<int>& cost, int num_ctas) {
+  const int n = (int)cost.size(), ctas = std::min(n, num_ctas);
+  if (n <= num_ctas) return;
+  std::vector<int64_t> load(ctas, 0);
+  std::vector<std::vector<uint4>> list(ctas);
+  std::vector<int> by_load(ctas);
+  for (int first = 0; first < n; first += ctas) {
+    for (int k = 0; k < ctas; ++k) by_load[k] = k;
+    std::stable_sort(by_load.begin(), by_load.end(), [&](int a, int c) { return load[a] < load[c]; });
+    for (int k = 0; k < std::min(ctas, n - first); ++k) {
+      list[by_load[k]].push_back(items[first + k]);
+      load[by_load[k]] += cost[first + k];
+    }
+  }
+  // the CTAs with an item in the last, shorter round come first
+  std::stable_sort(list.begin(), list.end(),
+                   [](const std::vector<uint4>& a, const std::vector<uint4>& c) { return a.size() > c.size(); });
+  for (int q = 0; q < n; ++q) items[q] = list[q % ctas][q / ctas];
+}
+
 // (Re)build the subarray descriptors and the item list for the batch's variant and the given
 // inputs (the fused kernel reads them through its tensor maps) and outputs.
 xcorr_status build_tables(xcorr_batch b, const void* const* d_ins, void* const* d_outs) {
@@ -170,10 +198,14 @@ xcorr_status build_tables(xcorr_batch b, const void* const* d_ins, void* const* 
     const int C = b->cfg[s].n_channels;
     const int nb = (b->n_inputs[s] + 127) / 128;
     std::string err;
-    int n_kt;
+    int n_kt, groups = C;
     if (fused) {
       xc::TaSubDesc& d = b->fdescs_host[s];
-      if (d_ins && !xc::encode_raw_ci4_tmap(&d.tmap, d_ins[s], b->n_inputs[s], C, C, n_time, kt, &err))
+      d.n_chan = C;
+      d.pack_g = xc::fused_ta_pack(b->n_inputs[s]);
+      groups = (C + d.pack_g - 1) / d.pack_g;
+      if (d_ins && !(d.pack_g > 1 ? xc::encode_raw_ci4_packed_tmap(&d.tmap, d_ins[s], b->n_inputs[s], C, C, n_time, kt, &err)
+                                  : xc::encode_raw_ci4_tmap(&d.tmap, d_ins[s], b->n_inputs[s], C, C, n_time, kt, &err)))
         return bfail(XCORR_ERR_INVALID_ARG, "subarray " + std::to_string(s) + ": " + err);
       d.out = d_outs ? static_cast<int2*>(d_outs[s]) : nullptr;
       d.n_pairs = b->n_pairs[s];
@@ -195,7 +227,7 @@ xcorr_status build_tables(xcorr_batch b, const void* const* d_ins, void* const* 
       d.n_tw = (d.n_kt + xc::kTcWindowCI4 / kt - 1) / (xc::kTcWindowCI4 / kt);
       n_kt = d.n_kt;
     }
-    for (int c = 0; c < C; ++c)
+    for (int c = 0; c < groups; ++c)
       for (int I = 0; I < nb; ++I)
         for (int J = 0; J <= I; ++J) {
           items.push_back(make_uint4((unsigned)s, (unsigned)c, (unsigned)I, (unsigned)J));
@@ -215,6 +247,11 @@ xcorr_status build_tables(xcorr_batch b, const void* const* d_ins, void* const* 
     ++b->class_n[cls[order[k]]];
   }
   for (int k = 0, off = 0; k < b->n_classes; off += b->class_n[k], ++k) b->class_off[k] = off;
+  for (int k = 0; k < b->n_classes; ++k) {
+    std::vector<int> by_rank(b->class_n[k]);
+    for (int q = 0; q < b->class_n[k]; ++q) by_rank[q] = cost[order[b->class_off[k] + q]] + kItemOverhead;
+    deal(sorted.data() + b->class_off[k], by_rank, b->num_sms);
+  }
   if (b->items_dev && (int)sorted.size() != b->n_items) {
     cudaFree(b->items_dev);
     b->items_dev = nullptr;

@@ -213,10 +213,13 @@ struct SubDescHost {
 };
 // A subarray of a batch run by the fused 4-bit kernel (A operand in tensor memory).
 struct TaSubDesc {
-  CUtensorMap tmap;  // its raw CI4 input: boxes of 128 inputs x 1 channel x the stage height
+  // its raw CI4 input: boxes of 128 inputs x 1 channel x the stage height, or with pack_g > 1 of pack_g
+  // channels side by side (an item's channel is then the group's number)
+  CUtensorMap tmap;
   int2* out;         // its int2 [C][P] visibilities
   int64_t n_pairs;
   int n_inputs, n_tile_pairs, n_kt, accumulate;
+  int n_chan, pack_g;
 };
 static_assert(sizeof(TaSubDesc) % 64 == 0, "tensor maps in a descriptor array stay 64-byte aligned");
 cudaError_t launch_xcorr_tc_fused_ta_batch(const TaSubDesc* subs, const uint4* items, int n_items, int variant,
@@ -305,6 +308,8 @@ cudaError_t launch_xcorr_tc_fused_ci4(const uint8_t* in, int row_chans, int vari
                                       cudaStream_t stream);
 
 int fused_ta_stage_samples(int variant);
+// Channels of n_inputs (a multiple of 16) that the kernel can hold side by side in one tile.
+int fused_ta_pack(int n_inputs);
 // pitch: bytes from one channel to the next (n_inputs, or more where rows were padded), a multiple of 16.
 cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int variant, int n_time, int n_chan,
                                          int n_inputs, int pitch, int2* out, bool accumulate, int* status, int num_sms,

@@ -125,6 +125,7 @@ struct TItem {
   int2* out;
   int64_t n_pairs;
   int c, I, J, n_inputs, n_kt;
+  int pack_g, pitch, n_chan;  // channels side by side in the tile (1: none); c is then their group
   int t_first;             // first sample of the item
   int ax, ay, bx, by;      // TMA coordinates (input or channel-input column, channel) of the row and column tiles
   bool diag, valid;
@@ -143,6 +144,9 @@ __device__ __forceinline__ TItem resolve(const TParams& p, const CUtensorMap* ma
     it.n_pairs = s->n_pairs;
     it.n_inputs = s->n_inputs;
     it.n_kt = s->n_kt;
+    it.pack_g = s->pack_g;
+    it.pitch = s->n_inputs;
+    it.n_chan = s->n_chan;
     it.c = static_cast<int>(w.y);
     it.I = static_cast<int>(w.z);
     it.J = static_cast<int>(w.w);
@@ -152,6 +156,9 @@ __device__ __forceinline__ TItem resolve(const TParams& p, const CUtensorMap* ma
     it.out = p.out;
     it.n_pairs = p.n_pairs;
     it.n_inputs = p.n_inputs;
+    it.pack_g = PACK ? p.pack_g : 1;
+    it.pitch = p.pitch;
+    it.n_chan = p.n_chan;
     int tile = item;
     it.n_kt = p.n_kt;
     it.t_first = p.t0;
@@ -170,8 +177,8 @@ __device__ __forceinline__ TItem resolve(const TParams& p, const CUtensorMap* ma
     }
   }
   it.diag = it.I == it.J;
-  if (PACK) {  // the packed view: x = channel * pitch + input over one time row
-    it.ax = it.bx = it.c * p.pack_g * p.pitch;
+  if (PACK || (BATCH && it.pack_g > 1)) {  // the packed view: x = channel * pitch + input over one time row
+    it.ax = it.bx = it.c * it.pack_g * it.pitch;
     it.ay = it.by = 0;
   } else {
     it.ax = it.I * kBlk;
@@ -526,6 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++g) {
       const TItem it = resolve<BATCH, SMALL, PACK, KT>(p, &raw_map, item, n_items);
       const int c = it.c, I = it.I, J = it.J, n_inputs = it.n_inputs;
+      const bool packed = PACK || (BATCH && it.pack_g > 1);
       const int t128 = 128 * it.n_kt * KT;  // 128 T over the padded block (padding decodes to u = 8 + 8i)
       const bool magic = t128 <= 128 * kMagicSamples;
       int2* out_c = it.out + (int64_t)c * it.n_pairs;
@@ -549,8 +557,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_after();
       // 16-pair chunks this warp keeps: none past the inputs (the packed channels), none wholly
       // above the diagonal
-      const int n_ch = (PACK ? (warp * 32 >= p.pack_g * p.pitch || c * p.pack_g + (warp * 32) / p.pitch >= p.n_chan)
-                             : row0 >= n_inputs)
+      const int n_ch = (packed ? (warp * 32 >= it.pack_g * it.pitch || c * it.pack_g + (warp * 32) / it.pitch >= it.n_chan)
+                               : row0 >= n_inputs)
                            ? 0
                        : I == J ? (warp * 32 + 31) / kChunk + 1
                                 : kBlk / kChunk;
@@ -596,11 +604,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         firstm[m] = 0;
         lastm[m] = I == J ? rr : kBlk - 1;  // last column of the row in the tile
         rcm[m] = rowc[rr];
-        if (PACK) {
-          const int blk = rr / p.pitch, cr = c * p.pack_g + blk;
-          const int i = rr - blk * p.pitch;
-          if (blk < p.pack_g && cr < p.n_chan && i < n_inputs) {
-            firstm[m] = blk * p.pitch;
+        if (packed) {
+          const int blk = rr / it.pitch, cr = c * it.pack_g + blk;
+          const int i = rr - blk * it.pitch;
+          if (blk < it.pack_g && cr < it.n_chan && i < n_inputs) {
+            firstm[m] = blk * it.pitch;
             row_out[m] = it.out + (int64_t)cr * it.n_pairs + (int64_t)i * (i + 1) / 2;
           }
         } else {
@@ -727,11 +735,13 @@ cudaError_t launch_ta(const CUtensorMap& raw_map, const TParams& p, int grid, cu
 // and (3) the small-problem layout on 128 x (2 + 2).
 int fused_ta_stage_samples(int variant) { return variant == 0 || variant == 3 ? 128 : variant == 1 ? 96 : 64; }
 
+int fused_ta_pack(int n_inputs) { return n_inputs <= kBlk / 2 ? kBlk / n_inputs : 1; }
+
 // The small-problem layout of a launch: channels packed per tile and the time split.
 void small_layout(int n_chan, int n_inputs, int n_kt, int num_sms, int& pack_g, int& tiles, int& n_split,
                   int& split_kt) {
   const int nb = (n_inputs + kBlk - 1) / kBlk;
-  pack_g = n_inputs <= kBlk / 2 ? kBlk / n_inputs : 1;
+  pack_g = fused_ta_pack(n_inputs);
   tiles = pack_g > 1 ? (n_chan + pack_g - 1) / pack_g : n_chan * (nb * (nb + 1) / 2);
   // as many splits as keep the items within one wave of the SMs, each at least one stage long
   n_split = tiles >= num_sms ? 1 : num_sms / tiles;
@@ -761,7 +771,7 @@ cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int v
   CUtensorMap raw_map;
   if (row_chans < n_chan) return cudaErrorInvalidValue;
   int pack_g = 1;
-  if (small) pack_g = pitch <= kBlk / 2 ? kBlk / pitch : 1;
+  if (small) pack_g = fused_ta_pack(pitch);
   if (pack_g > 1) {
     // the packed view: one time row is n_chan * pitch bytes (channel-major), read in boxes of 128
     // (pack_g channels side by side) x 1 x kt; the middle dimension has extent 1

@@ -355,3 +355,19 @@ def test_float_one_tile_edges(torch, value):
     scale = np.sqrt(autos[:, ii] * autos[:, jj])
     err = np.abs((got[..., 0] - want[..., 0]) + 1j * (got[..., 1] - want[..., 1]))
     assert (err[~hit] <= 1e-6 * scale[~hit]).all()
+
+
+@pytest.mark.parametrize("shape", [3, 4, 5])
+@pytest.mark.parametrize("subs", [[(8, 1, 1), (8, 9, 200), (16, 5, 129), (24, 3, 300), (32, 3, 64)],
+                                  [(8, 700, 70), (24, 151, 33), (40, 30, 260), (72, 40, 100), (32, 2, 1000), (64, 200, 20)]])
+def test_batch_packs_channels(torch, shape, subs):
+    """Channel groups that end inside a tile, beside subarrays that pack nothing; fewer and more items
+    than SMs, so that the dealing has short last rounds."""
+    xs = [draw("ci4", t, c, s, seed=s + c + t) for s, c, t in subs]
+    batch = xcorr.Batch(subs)
+    batch.set_variant(shape)
+    outs = batch.execute([torch.from_numpy(x).cuda() for x in xs])
+    batch.sync()
+    for x, out in zip(xs, outs):
+        check("ci4", out.cpu().numpy(), x, 2 * x.shape[2])
+    batch.close()

@@ -178,19 +178,20 @@ int padded_shape(int v) {
   return v == xc::kSmallFusedVariant ? 3 : v >= 4 && v <= 6 ? v - 4 : xc::kDefaultFusedVariant - 4;
 }
 
-// Correlate through padded rows.
-cudaError_t run_repitched(xcorr_plan plan, const Pieces& r, const void* d_in, int n_time, int2* target, bool fresh,
-                          cudaStream_t s) {
+// Correlate nch channels through padded rows: d_in at the first of them, in rows of the plan's channels,
+// target at its visibilities.
+cudaError_t run_repitched(xcorr_plan plan, const Pieces& r, const void* d_in, int nch, int n_time, int2* target,
+                          bool fresh, cudaStream_t s) {
   const int C = plan->cfg.n_channels, N = plan->n_inputs;
   const bool ci4 = plan->cfg.fmt == XCORR_IN_CI4;
   const size_t row = static_cast<size_t>(N) * (ci4 ? 1 : 2);  // one channel of one sample
   const uint8_t* in = static_cast<const uint8_t*>(d_in);
-  const uint8_t* end = in + row * C * n_time;
+  const uint8_t* end = in + row * (static_cast<size_t>(C) * (n_time - 1) + nch);
   const int shape = padded_shape(plan->tune_variant);
   for (int t0 = 0; t0 < n_time; t0 += r.nt) {
     const int nt = n_time - t0 < r.nt ? n_time - t0 : r.nt;
-    for (int c0 = 0; c0 < C; c0 += r.nc) {
-      const int nc = C - c0 < r.nc ? C - c0 : r.nc;
+    for (int c0 = 0; c0 < nch; c0 += r.nc) {
+      const int nc = nch - c0 < r.nc ? nch - c0 : r.nc;
       cudaError_t e = xc::launch_repitch(in + (static_cast<size_t>(t0) * C + c0) * row, end, plan->planes,
                                          static_cast<int>(row), C, nc, nt, plan->num_sms, s);
       if (e != cudaSuccess) return e;
@@ -198,7 +199,7 @@ cudaError_t run_repitched(xcorr_plan plan, const Pieces& r, const void* d_in, in
       const bool add = !fresh || t0 > 0;
       e = ci4 ? xc::launch_xcorr_tc_fused_ta_ci4(static_cast<const uint8_t*>(plan->planes), nc, shape, nt, nc, N, r.pitch,
                                                  out, add, plan->status, plan->num_sms, s)
-              : xc::launch_xcorr_tc_raw_pair(static_cast<const int8_t*>(plan->planes), nt, nc, N, r.pitch, out, add,
+              : xc::launch_xcorr_tc_raw_pair(static_cast<const int8_t*>(plan->planes), nc, nt, nc, N, r.pitch, out, add,
                                              plan->status, plan->num_sms, s);
       if (e != cudaSuccess) return e;
     }
@@ -218,6 +219,28 @@ cudaError_t unpack_group(xcorr_plan plan, const void* d_in, int n_time, int c0, 
                                            plan->exps, n_time, C, c0, nc, N, plan->ni_pad, T, plan->window_samples,
                                            plan->exp_windows, s);
   }
+}
+
+int even_groups(int C, int n, int* edge) {
+  const int most = C < xc::kMaxGroups ? C : xc::kMaxGroups, G = n < most ? n : most;
+  for (int g = 0; g <= G; ++g) edge[g] = static_cast<int>(static_cast<int64_t>(C) * g / G);
+  return G;
+}
+
+// The channel groups of a host-to-host execute that moves `bytes` in and out.  A column of at least a
+// quarter of a sample's channels comes up at the link's rate beside a copy down (256 MB each way, rows of
+// 16 to 512 KB: 1.58-1.61 ms); an eighth does not (2.1 ms).  Nothing comes down during the first group's
+// way up, so that one is narrow; its head start no longer matters where the copies take milliseconds.  A
+// group costs about 10 us.  (512 inputs x 128 channels x 1024 samples, 67 MB up, 134 MB down: one group
+// 1140 us, four equal ones 897, these 853; the copies alone 749.  1024 samples of 256 inputs x 64 channels,
+// 33 MB in all: 227, 182, 183.  524 MB each way: four equal ones 3.88 ms, these 4.39.)
+int host_groups(int C, size_t bytes, int* edge) {
+  const size_t mb = bytes >> 20;
+  if (mb < 24 || C < 8) return even_groups(C, mb < 8 ? 1 : 2, edge);
+  if (mb >= 512) return even_groups(C, 4, edge);
+  const int sixteenths[5] = {0, 2, 6, 11, 16};
+  for (int g = 0; g <= 4; ++g) edge[g] = static_cast<int>(static_cast<int64_t>(C) * sixteenths[g] / 16);
+  return 4;
 }
 
 // Correlate n_time samples into target (the plan's accumulator, or the
@@ -245,7 +268,7 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     // int8 input decoded on chip: one launch on the caller's stream
     if (ev && ((e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventRecord(ev[2], s)) != cudaSuccess))
       return cuda_fail(e, "profile event");
-    e = xc::launch_xcorr_tc_raw_pair(static_cast<const int8_t*>(d_in), n_time, C, N, N, static_cast<int2*>(target),
+    e = xc::launch_xcorr_tc_raw_pair(static_cast<const int8_t*>(d_in), C, n_time, C, N, N, static_cast<int2*>(target),
                                      !target_fresh, plan->status, plan->num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "CTA-pair X kernel launch");
     if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
@@ -254,7 +277,7 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     // the same kernels over padded rows, piece by piece on the caller's stream
     if (ev && ((e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventRecord(ev[2], s)) != cudaSuccess))
       return cuda_fail(e, "profile event");
-    if ((e = run_repitched(plan, pieces, d_in, n_time, static_cast<int2*>(target), target_fresh, s)) != cudaSuccess)
+    if ((e = run_repitched(plan, pieces, d_in, C, n_time, static_cast<int2*>(target), target_fresh, s)) != cudaSuccess)
       return cuda_fail(e, "padded rows: copy or X kernel launch");
     if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
     if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
@@ -706,7 +729,9 @@ xcorr_status xcorr_execute_dump_host(xcorr_plan plan, const void* h_in, int n_ti
       }
   uint8_t* stage = static_cast<uint8_t*>(plan->host_stage);
   const size_t out_chan_bytes = static_cast<size_t>(plan->n_pairs) * 8;
-  if (!(plan->engine == XCORR_ENGINE_TENSOR && fused_applies(plan, stage))) {
+  const bool fused = plan->engine == XCORR_ENGINE_TENSOR && fused_applies(plan, stage), raw = raw_ci8_applies(plan, stage);
+  const Pieces pieces = fused || raw ? Pieces{} : repitch_pieces(plan, n_time);
+  if (!fused && !raw && !pieces.pitch) {
     // one piece: up, X-stage, down, in order on the caller's stream
     if ((e = cudaMemcpyAsync(stage, h_in, row_bytes * n_time, cudaMemcpyHostToDevice, s)) != cudaSuccess)
       return cuda_fail(e, "input copy");
@@ -717,30 +742,29 @@ xcorr_status xcorr_execute_dump_host(xcorr_plan plan, const void* h_in, int n_ti
     // channel groups: group g goes up on s_unpack, is correlated on s_x[g % 2] (a
     // launch can start on the SMs the previous one's tail leaves idle) and comes
     // down on s_down while later groups are still moving
-    // by default as many groups as keep each 2-D copy row >= 64 KB: narrower rows
-    // halve the copy engines' rate (measured: 210 GB/s at 64 KB, 104 GB/s at 32 KB)
-    const size_t min_width = size_t(64) << 10;
-    int G = n_groups > 0 ? n_groups : static_cast<int>(row_bytes / min_width < 1 ? 1 : row_bytes / min_width);
-    G = G > xc::kMaxGroups ? xc::kMaxGroups : G;
-    G = G > C ? C : G;
+    int edge[xc::kMaxGroups + 1];  // group g: channels edge[g] .. edge[g + 1] - 1
+    const int G = n_groups > 0 ? even_groups(C, n_groups, edge)
+                               : host_groups(C, row_bytes * n_time + out_chan_bytes * C, edge);
     if ((e = cudaEventRecord(plan->ev_fork, s)) != cudaSuccess) return cuda_fail(e, "fork event");
     for (cudaStream_t t : {plan->s_unpack, plan->s_x[0], plan->s_x[1], plan->s_down})
       if ((e = cudaStreamWaitEvent(t, plan->ev_fork, 0)) != cudaSuccess) return cuda_fail(e, "fork wait");
     for (int g = 0; g < G; ++g) {
-      const int c0 = static_cast<int>(static_cast<int64_t>(C) * g / G);
-      const int c1 = static_cast<int>(static_cast<int64_t>(C) * (g + 1) / G);
+      const int c0 = edge[g], c1 = edge[g + 1];
       if (c1 <= c0) continue;
       const size_t off = chan_bytes * c0, width = chan_bytes * (c1 - c0);
-      cudaStream_t sx = plan->s_x[g & 1];
+      cudaStream_t sx = plan->s_x[pieces.pitch ? 0 : g & 1];  // (padded rows: one piece of memory)
       int2* out_g = static_cast<int2*>(plan->acc) + static_cast<int64_t>(c0) * plan->n_pairs;
       if ((e = cudaMemcpy2DAsync(stage + off, row_bytes, static_cast<const uint8_t*>(h_in) + off, row_bytes, width,
                                  n_time, cudaMemcpyHostToDevice, plan->s_unpack)) != cudaSuccess ||
           (e = cudaEventRecord(plan->ev_up[g], plan->s_unpack)) != cudaSuccess ||
           (e = cudaStreamWaitEvent(sx, plan->ev_up[g], 0)) != cudaSuccess)
         return cuda_fail(e, "group input copy");
-      if ((e = xc::launch_xcorr_tc_fused_ci4(stage + off, C, plan->tune_variant, n_time, c1 - c0, N, out_g, false,
-                                             plan->status, plan->num_sms, sx)) != cudaSuccess)
-        return cuda_fail(e, "fused X kernel launch");
+      e = fused ? xc::launch_xcorr_tc_fused_ci4(stage + off, C, plan->tune_variant, n_time, c1 - c0, N, out_g, false,
+                                                plan->status, plan->num_sms, sx)
+          : raw ? xc::launch_xcorr_tc_raw_pair(reinterpret_cast<const int8_t*>(stage + off), C, n_time, c1 - c0, N, N, out_g,
+                                               false, plan->status, plan->num_sms, sx)
+                : run_repitched(plan, pieces, stage + off, c1 - c0, n_time, out_g, true, sx);
+      if (e != cudaSuccess) return cuda_fail(e, "X kernel launch");
       if ((e = cudaEventRecord(plan->ev_group_done[g], sx)) != cudaSuccess ||
           (e = cudaStreamWaitEvent(plan->s_down, plan->ev_group_done[g], 0)) != cudaSuccess ||
           (e = cudaMemcpyAsync(static_cast<uint8_t*>(h_out) + out_chan_bytes * c0, out_g, out_chan_bytes * (c1 - c0),

@@ -324,14 +324,15 @@ cudaError_t launch_xcorr_tc_fused_pair_ci4(const uint8_t* in, int row_chans, int
 
 // Tensor map over an int8 input [t][c][i][2] in boxes of 64 inputs x 1 channel x box_t samples (128-byte
 // swizzle); n_inputs a multiple of 8, a 16-byte aligned pointer.
-bool encode_raw_ci8_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_chan, int n_time, int box_t,
+bool encode_raw_ci8_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_chan, int row_chans, int n_time, int box_t,
                          std::string* err);
 // The X-stage on CTA pairs with int8 samples decoded on chip (xcorr_tc_raw_pair.cu): one launch.
 bool raw_pair_takes(int pitch, const void* in);
 int raw_pair_items(int n_tiles);  // work items of one channel
 // pitch: inputs from one channel to the next (n_inputs, or more where rows were padded), a multiple of 8.
-cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int n_time, int n_chan, int n_inputs, int pitch, int2* out,
-                                     bool accumulate, int* status, int num_sms, cudaStream_t stream);
+// `in` points at the first of n_chan channels; time rows hold row_chans channels.
+cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int row_chans, int n_time, int n_chan, int n_inputs, int pitch,
+                                     int2* out, bool accumulate, int* status, int num_sms, cudaStream_t stream);
 
 // Copies n_chan rows of row_bytes (of the row_chans that make up a sample) x n_time samples to rows of
 // row_bytes rounded up to 16 (xcorr_repitch.cu).  `end`: one past the last byte of the caller's input.

@@ -447,9 +447,9 @@ bool raw_pair_takes(int pitch, const void* in) {
   return pitch % 8 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;
 }
 
-cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int n_time, int n_chan, int n_inputs, int pitch, int2* out,
-                                     bool accumulate, int* status, int num_sms, cudaStream_t stream) {
-  if (!raw_pair_takes(pitch, in) || pitch < n_inputs || n_time < 1) return cudaErrorInvalidValue;
+cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int row_chans, int n_time, int n_chan, int n_inputs, int pitch,
+                                     int2* out, bool accumulate, int* status, int num_sms, cudaStream_t stream) {
+  if (!raw_pair_takes(pitch, in) || pitch < n_inputs || row_chans < n_chan || n_time < 1) return cudaErrorInvalidValue;
   RParams p{};
   p.n_inputs = n_inputs;
   p.nb = (n_inputs + kBlk - 1) / kBlk;
@@ -463,7 +463,7 @@ cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int n_time, int n_chan, i
   p.out = out;
   p.status = status;
   CUtensorMap map;
-  if (!encode_raw_ci8_tmap(&map, in, pitch, n_chan, n_time, kRows, nullptr)) return cudaErrorInvalidValue;
+  if (!encode_raw_ci8_tmap(&map, in, pitch, n_chan, row_chans, n_time, kRows, nullptr)) return cudaErrorInvalidValue;
   return accumulate ? launch_raw_pair<true>(map, p, num_sms, stream) : launch_raw_pair<false>(map, p, num_sms, stream);
 }
 

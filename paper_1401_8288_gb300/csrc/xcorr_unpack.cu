@@ -212,9 +212,9 @@ bool encode_raw_ci4_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_c
   return true;
 }
 
-bool encode_raw_ci8_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_chan, int n_time, int box_t,
+bool encode_raw_ci8_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_chan, int row_chans, int n_time, int box_t,
                          std::string* err) {
-  if (const RawMapMemo* m = raw_memo_find(in, n_inputs, n_chan, n_chan, n_time, box_t, 64, 2)) {
+  if (const RawMapMemo* m = raw_memo_find(in, n_inputs, n_chan, row_chans, n_time, box_t, 64, 2)) {
     *map = m->map;
     return true;
   }
@@ -223,7 +223,7 @@ bool encode_raw_ci8_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_c
   std::memset(map, 0, sizeof(*map));
   const cuuint64_t row = (cuuint64_t)n_inputs * 2;
   cuuint64_t dims[3] = {(cuuint64_t)n_inputs, (cuuint64_t)n_chan, (cuuint64_t)n_time};
-  cuuint64_t strides[2] = {row, row * (cuuint64_t)n_chan};
+  cuuint64_t strides[2] = {row, row * (cuuint64_t)row_chans};
   cuuint32_t box[3] = {64, 1, (cuuint32_t)box_t};
   cuuint32_t elem_strides[3] = {1, 1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<void*>(in), dims, strides, box, elem_strides,
@@ -233,7 +233,7 @@ bool encode_raw_ci8_tmap(CUtensorMap* map, const void* in, int n_inputs, int n_c
     if (err) *err = "cuTensorMapEncodeTiled (raw int8 input) failed with CUresult " + std::to_string((int)r);
     return false;
   }
-  raw_memo_put(*map, in, n_inputs, n_chan, n_chan, n_time, box_t, 64, 2);
+  raw_memo_put(*map, in, n_inputs, n_chan, row_chans, n_time, box_t, 64, 2);
   return true;
 }
 

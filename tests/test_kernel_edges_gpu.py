@@ -371,3 +371,16 @@ def test_batch_packs_channels(torch, shape, subs):
     for x, out in zip(xs, outs):
         check("ci4", out.cpu().numpy(), x, 2 * x.shape[2])
     batch.close()
+
+
+@pytest.mark.parametrize("n_groups", [0, 1, 3, 8])
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time", [("ci4", 128, 9, 300), ("ci4", 37, 70, 700), ("ci8", 64, 11, 130), ("ci8", 70, 130, 400),
+                                                     ("ci8", 101, 10, 129), ("ci4", 131, 64, 1500), ("ci4", 1, 3, 5)])
+def test_host_to_host_in_groups(torch, fmt, n_sta, n_chan, n_time, n_groups):
+    """Channel groups of every on-chip route: whole rows, rows that are padded, int8; twice, on new data."""
+    for seed in (1, 2):
+        x = draw(fmt, n_time, n_chan, n_sta, seed=seed)
+        with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor") as plan:
+            out = plan.execute_dump_host(torch.from_numpy(x).pin_memory(), n_groups=n_groups)
+            plan.sync()
+        check(fmt, out.numpy(), x, 2 * n_sta)

@@ -57,6 +57,7 @@ struct xcorr_batch_s {
   // fused classes: item range and shape of each, in items_dev
   int n_classes = 0;
   int class_variant[kBatchClasses] = {}, class_off[kBatchClasses] = {}, class_n[kBatchClasses] = {};
+  int class_stages[kBatchClasses] = {};  // of an item on average
   cudaStream_t class_stream[kBatchClasses] = {};
   cudaEvent_t ev_fork = nullptr, ev_class_done[kBatchClasses] = {};
   std::vector<int> solo;        // subarrays with a shape of their own, largest first
@@ -250,6 +251,9 @@ xcorr_status build_tables(xcorr_batch b, const void* const* d_ins, void* const* 
   for (int k = 0; k < b->n_classes; ++k) {
     std::vector<int> by_rank(b->class_n[k]);
     for (int q = 0; q < b->class_n[k]; ++q) by_rank[q] = cost[order[b->class_off[k] + q]] + kItemOverhead;
+    int64_t total = 0;
+    for (int v : by_rank) total += v - kItemOverhead;
+    b->class_stages[k] = b->class_n[k] ? static_cast<int>(total / b->class_n[k]) : 0;
     deal(sorted.data() + b->class_off[k], by_rank, b->num_sms);
   }
   if (b->items_dev && (int)sorted.size() != b->n_items) {
@@ -275,7 +279,8 @@ xcorr_status build_tables(xcorr_batch b, const void* const* d_ins, void* const* 
 xcorr_status enqueue(xcorr_batch b, const void* const* d_ins, cudaStream_t s) {
   cudaError_t e;
   if (fused_mode(b) && b->n_classes == 1 && b->solo.empty()) {
-    e = xc::launch_xcorr_tc_fused_ta_batch(b->fdescs_dev, b->items_dev, b->n_items, b->class_variant[0] - kFusedBase,
+    e = xc::launch_xcorr_tc_fused_ta_batch(b->fdescs_dev, b->items_dev, b->n_items, b->class_stages[0],
+                                           b->class_variant[0] - kFusedBase,
                                            b->status, b->num_sms, s);
     if (e != cudaSuccess) return bfail(XCORR_ERR_CUDA, std::string("fused batch launch: ") + cudaGetErrorString(e));
     return XCORR_OK;
@@ -307,7 +312,7 @@ xcorr_status enqueue(xcorr_batch b, const void* const* d_ins, cudaStream_t s) {
       cudaStream_t sk = b->class_stream[k];
       if ((e = cudaStreamWaitEvent(sk, b->ev_fork, 0)) != cudaSuccess ||
           (e = xc::launch_xcorr_tc_fused_ta_batch(b->fdescs_dev, b->items_dev + b->class_off[k], b->class_n[k],
-                                                  b->class_variant[k] - kFusedBase, b->status, b->num_sms, sk)) !=
+                                                  b->class_stages[k], b->class_variant[k] - kFusedBase, b->status, b->num_sms, sk)) !=
               cudaSuccess ||
           (e = cudaEventRecord(b->ev_class_done[k], sk)) != cudaSuccess ||
           (e = cudaStreamWaitEvent(s, b->ev_class_done[k], 0)) != cudaSuccess)

@@ -222,8 +222,9 @@ struct TaSubDesc {
   int n_chan, pack_g;
 };
 static_assert(sizeof(TaSubDesc) % 64 == 0, "tensor maps in a descriptor array stay 64-byte aligned");
-cudaError_t launch_xcorr_tc_fused_ta_batch(const TaSubDesc* subs, const uint4* items, int n_items, int variant,
-                                           int* status, int num_sms, cudaStream_t stream);
+// mean_stages: stages of an item on average, which decide on the launch's epilogue.
+cudaError_t launch_xcorr_tc_fused_ta_batch(const TaSubDesc* subs, const uint4* items, int n_items, int mean_stages,
+                                           int variant, int* status, int num_sms, cudaStream_t stream);
 // One launch of the batch X kernel over items (subarray, channel, I, J).
 cudaError_t launch_xcorr_tc_batch(const void* subs, const uint4* items, int n_items, int variant, int* status,
                                   int num_sms, cudaStream_t stream);

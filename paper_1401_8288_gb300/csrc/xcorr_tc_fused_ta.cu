@@ -31,12 +31,21 @@
 //
 // The per-input sums S = sum_t u that undo the offset (see xcorr_tc_fused.cu)
 // come from the A path for the rows (dp4a over the codes each thread holds)
-// and from the B path for the columns (byte lanes, as in the other kernel).
+// and from the B path for the columns (byte lanes, as in the other kernel); the
+// decoders leave them as each thread holds them and the epilogue adds them up.
 //
-// Warp roles (448 threads, one CTA per SM): warps 0-3 drain the accumulator
-// and write the output; warps 4-11 decode (warp w writes the A lanes of TMEM
-// quarter w % 4, 16 inputs, and a share of B); warp 12 is the TMA producer
-// with the L2 prefetch; warp 13 owns tensor memory and issues the MMAs.
+// What bounds it.  A 128-sample stage takes 0.75 us: 1440 cycles, of which
+// shared memory moves 160 KB in 1250 (TMA 32, A and B read 32, B's planes
+// written 32, the MMAs' B operand 64), the tensor pipe works 1024 and the
+// decoders' ALU instructions issue 870.  Sixteen decoder warps instead of eight
+// take longer (0.92 us).  What an item adds on top is its epilogue's share of
+// the same shared-memory and L1 path, about 1.5 us, as its staging and stores
+// move another 330 KB.
+//
+// Warp roles (one CTA per SM): the first 4 or 8 warps (Roles) drain the
+// accumulator and write the output; the next 8 decode (warp w writes the A lanes
+// of TMEM quarter w % 4, 16 inputs, and a share of B); then the TMA producer
+// with the L2 prefetch and the warp that owns tensor memory and issues the MMAs.
 // Every wait is bounded (sm103_ptx.cuh).
 //
 // A batch mode (xcorr_batch.cu) runs the same pipeline over the tile pairs of
@@ -50,29 +59,47 @@ namespace {
 
 using namespace fused;
 
-constexpr int kEpiWarps = 4;
-constexpr int kDecWarp0 = 4;
 constexpr int kDecWarps = 8;  // two per tensor-memory lane quarter
-constexpr int kProducerWarp = kDecWarp0 + kDecWarps;
-constexpr int kMmaWarp = kProducerWarp + 1;
-constexpr int kThreads = (kMmaWarp + 1) * 32;
+// EPI epilogue warps: one or two per lane quarter, which then halve its columns.
+template <int EPI>
+struct Roles {
+  static constexpr int kDecWarp0 = EPI, kProducerWarp = kDecWarp0 + kDecWarps, kMmaWarp = kProducerWarp + 1;
+  static constexpr int kThreads = (kMmaWarp + 1) * 32;
+};
 constexpr int kDecThreads = kDecWarps * 32;
 constexpr int kChunk = 16;
-constexpr int kPitch = kChunk + 1;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kStashCol = 256;                       // 128 columns of corrected Im after the accumulator
 constexpr uint32_t kAcol0 = 384;                          // then the A stages
 constexpr int kStagingBytes = kBlk * kBlk * 4;            // Re accumulator bits of a whole tile pair
 constexpr int kRowcBytes = kBlk * 8;                      // per-row correction constants
-constexpr int kSumsBytes = 2 * 2 * kBlk * 8;              // [item parity][rows I, columns J][input] (8P, 8Q)
+constexpr int kSumsBytes = 2 * kBlk * 8 + 2 * kBlk * 4;   // columns: [item parity][input] (8P, 8Q); Re, Im code sums
 // Every partial sum of u_a u_b is n 2^-18 with 0 <= n <= 450 T (and |n| <= 225 T for Im).
 // For T <= kMagicSamples, |n| < 2^22 and n + 1.5 2^23 is exact in FP32, so one FFMA
 // against that constant turns the accumulator into n (in the low bits of the result).
 constexpr int kMagicSamples = 9320;
 constexpr float kMagic = 12582912.0f;       // 1.5 * 2^23
 constexpr int kMagicBits = 0x4B400000;
-constexpr int kScratchBytes = kDecWarps * 8 * kPitch * 8; // [decoder warp][chunk][input] (P, Q), padded rows
+// Every decoder thread's code sums of an item, as it holds them: four 16-byte words of column sums (Re of
+// inputs 0-7 and 8-15 of its chunk, then Im) and one of row sums, [word][thread].
+constexpr int kDumpBytes = 5 * kDecThreads * 16;
 constexpr int kBarrierBytes = 512;
+
+// The epilogue warps' own barrier, and its OR-reduction form.
+template <int EPI>
+__device__ __forceinline__ void epi_bar_sync() {
+  asm volatile("bar.sync 2, %0;" ::"n"(EPI * 32) : "memory");
+}
+template <int EPI>
+__device__ __forceinline__ bool epi_bar_or(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 2, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(v ? 1u : 0u), "n"(EPI * 32)
+      : "memory");
+  return r != 0;
+}
 
 template <int KT, int RAW, int DEC>
 struct TGeom {
@@ -88,8 +115,8 @@ struct TGeom {
   static constexpr int kOffStaging = kOffBpl + DEC * kBStage;
   static constexpr int kOffRowc = kOffStaging + kStagingBytes;
   static constexpr int kOffSums = kOffRowc + kRowcBytes;
-  static constexpr int kOffScratch = kOffSums + kSumsBytes;
-  static constexpr int kOffBarriers = kOffScratch + kScratchBytes;
+  static constexpr int kOffDump = kOffSums + kSumsBytes;
+  static constexpr int kOffBarriers = kOffDump + kDumpBytes;
   static constexpr int kSmem = 1024 + kOffBarriers + kBarrierBytes;
   static_assert(KT % 32 == 0, "stages hold whole MMA steps and whole 32-row B passes");
   static_assert(DEC * kAcols <= static_cast<int>(kTmemCols - kAcol0), "A stages fit beside the accumulator");
@@ -205,13 +232,15 @@ __device__ __forceinline__ int staging_swizzle(int row) { return ((row & 1) << 2
 // ADD: the launch adds into out with plain loads and stores (else it stores, or adds with atomics).  An
 // added pair costs a load that waits for L2 or HBM; issued one by one between the stores these made an
 // adding launch 7x slower than a storing one (1125 us against 154 us at 1024 inputs x 64 channels x 1024
-// samples).  With a chunk's sixteen loads in flight together the epilogue stays beside the next tile
-// pair's MMAs: 216 us for the same launch.  A kernel of its own, so that the storing launch carries none of the loads
+// samples).  Eight warps with eight loads of a thread in flight: 199 us for the same launch (four warps
+// with sixteen: 213).  A kernel of its own, so that the storing launch carries none of the loads'
 // registers (0.3 % at 512 inputs when it did).
-template <int KT, int RAW, int DEC, bool BATCH, bool SMALL, bool PACK, bool ADD>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int KT, int RAW, int DEC, bool BATCH, bool SMALL, bool PACK, bool ADD, int EPI>
+__global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
     xcorr_tc_fused_ta_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ TParams p) {
   using G = TGeom<KT, RAW, DEC>;
+  constexpr int kDecWarp0 = Roles<EPI>::kDecWarp0, kProducerWarp = Roles<EPI>::kProducerWarp,
+                kMmaWarp = Roles<EPI>::kMmaWarp;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* raw = smem;
@@ -219,16 +248,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* staging = reinterpret_cast<uint32_t*>(smem + G::kOffStaging);  // Re [row][16-byte chunk ^ swz(row)]
   int2* rowc = reinterpret_cast<int2*>(smem + G::kOffRowc);                 // [row]
   int2* sums = reinterpret_cast<int2*>(smem + G::kOffSums);
-  int2* scratch = reinterpret_cast<int2*>(smem + G::kOffScratch);
+  int* code_sums = reinterpret_cast<int*>(smem + G::kOffSums + 2 * kBlk * 8);  // [Re, Im][column]
+  uint4* dump = reinterpret_cast<uint4*>(smem + G::kOffDump);
   uint64_t* raw_full = reinterpret_cast<uint64_t*>(smem + G::kOffBarriers);
   uint64_t* raw_empty = raw_full + RAW;
   uint64_t* dec_full = raw_empty + RAW;
   uint64_t* dec_empty = dec_full + DEC;
   uint64_t* tfull = dec_empty + DEC;  // the accumulator holds an item
   uint64_t* tempty = tfull + 1;       // the epilogue has the item in registers
-  uint64_t* sfull = tempty + 1;       // [2] an item's input sums are written
-  uint64_t* sempty = sfull + 2;       // [2] the epilogue is done with them
-  uint64_t* mma_done = sempty + 2;
+  uint64_t* sfull = tempty + 1;       // an item's code sums are dumped
+  uint64_t* sempty = sfull + 1;       // the epilogue has read them
+  uint64_t* mma_done = sempty + 1;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(mma_done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
 
@@ -243,11 +273,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&dec_empty[s], 1);
     }
     mbar_init(tfull, 1);
-    mbar_init(tempty, kEpiWarps);
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&sfull[b], 1);
-      mbar_init(&sempty[b], kEpiWarps);
-    }
+    mbar_init(tempty, EPI);
+    mbar_init(sfull, kDecWarps);
+    mbar_init(sempty, 4);
     mbar_init(mma_done, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -420,58 +448,17 @@ __global__ void __launch_bounds__(kThreads, 1)
           dph ^= 1u;
         }
       }
-      // row sums: the four lanes holding one input's samples are lanes 4k .. 4k + 3
-#pragma unroll
-      for (int m = 1; m <= 2; m <<= 1) {
-        sar0 += __shfl_xor_sync(0xFFFFFFFFu, sar0, m);
-        sai0 += __shfl_xor_sync(0xFFFFFFFFu, sai0, m);
-        sar1 += __shfl_xor_sync(0xFFFFFFFFu, sar1, m);
-        sai1 += __shfl_xor_sync(0xFFFFFFFFu, sai1, m);
-      }
-      // column sums of this warp: lanes L, L + 8, L + 16, L + 24 hold chunk L
-      int2 pq[16];
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int sr = static_cast<int>((s_re[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
-        const int si = static_cast<int>((s_im[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
-        pq[e] = make_int2(sr + si, si - sr);
-      }
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        pq[e].x += __shfl_xor_sync(0xFFFFFFFFu, pq[e].x, 8);
-        pq[e].y += __shfl_xor_sync(0xFFFFFFFFu, pq[e].y, 8);
-        pq[e].x += __shfl_xor_sync(0xFFFFFFFFu, pq[e].x, 16);
-        pq[e].y += __shfl_xor_sync(0xFFFFFFFFu, pq[e].y, 16);
-      }
-      if (lane < 8) {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) scratch[(dw * 8 + lane) * kPitch + e] = pq[e];
-      }
-      dec_bar_sync(kDecThreads);
-      const int buf = g & 1;
-      if (ok) ok = mbar_wait_warp(&sempty[buf], ((g >> 1) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_TMEM_EMPTY);
-      if (ok) {
-        int2* rows = sums + (buf * 2) * kBlk;
-        if ((lane & 3) == 0) {
-          const int e = 16 * ib + (lane >> 2);
-          rows[e] = make_int2(8 * static_cast<int>(sar0 + sai0), 8 * (static_cast<int>(sai0) - static_cast<int>(sar0)));
-          rows[e + 8] =
-              make_int2(8 * static_cast<int>(sar1 + sai1), 8 * (static_cast<int>(sai1) - static_cast<int>(sar1)));
-        }
-        if (tid < kBlk) {
-          const int e = tid;
-          int2 s = make_int2(0, 0);
-#pragma unroll
-          for (int w = 0; w < kDecWarps; ++w) {
-            const int2 x = scratch[(w * 8 + (e >> 4)) * kPitch + (e & 15)];
-            s.x += x.x;
-            s.y += x.y;
-          }
-          sums[(buf * 2 + 1) * kBlk + e] = make_int2(8 * s.x, 8 * s.y);
-        }
-      }
-      if (dec_bar_or(!ok || *abort_flag, kDecThreads)) break;
-      if (tid == 0) mbar_arrive(&sfull[buf]);
+      // The code sums go out as they are: the epilogue adds them up while the decode runs on.  (Added up
+      // here, by 72 shuffles and two barriers of all decoder warps, they held the decode up for half a
+      // microsecond of every item: 512 inputs x 512 channels x 2048 samples 495 us, now 485.)
+      if (!ok || !mbar_wait_warp(sempty, (g & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_TMEM_EMPTY)) break;
+      dump[tid] = make_uint4(s_re[0], s_re[1], s_re[2], s_re[3]);
+      dump[kDecThreads + tid] = make_uint4(s_re[4], s_re[5], s_re[6], s_re[7]);
+      dump[2 * kDecThreads + tid] = make_uint4(s_im[0], s_im[1], s_im[2], s_im[3]);
+      dump[3 * kDecThreads + tid] = make_uint4(s_im[4], s_im[5], s_im[6], s_im[7]);
+      dump[4 * kDecThreads + tid] = make_uint4(sar0, sai0, sar1, sai1);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sfull);
     }
   } else if (warp == kMmaWarp) {
     if (lane == 0) {
@@ -519,16 +506,19 @@ __global__ void __launch_bounds__(kThreads, 1)
       mma_commit(mma_done);
       mbar_wait(mma_done, 0, &never, p.status, DEV_TIMEOUT_DRAIN);
     }
-  } else if (warp < kEpiWarps) {
-    // Epilogue, warp w = tile rows 32w .. 32w + 31 (TMEM lanes of quarter w).  Phase 1 only moves
+  } else if (warp < EPI) {
+    // Epilogue, warp w = tile rows 32q .. 32q + 31 with q = w % 4 (TMEM lanes of quarter q), and half of
+    // the columns where there are eight warps.  Phase 1 only moves
     // the accumulator out, so that it is free as soon as possible: Re bits to the shared-memory
     // staging tile, Im bits to the TMEM stash.  Phase 2, while the MMAs run the next tile pair,
     // converts, applies the offset corrections and writes the rows.  It reads the stash with
     // 16-lane x 256-bit loads, which give thread t columns 2 (t % 4), + 1 (and 8 on) of rows
     // t / 4 and t / 4 + 8, and phase 1 stages each row's Re in that column order, so four threads
     // write 16 consecutive pairs of a row straight from registers.
-    const int r_own = warp * 32 + lane;  // this thread's tile row in phase 1
-    const uint32_t taddr = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+    const int quarter = warp & 3, ch0 = (warp >> 2) * (kBlk / kChunk / 2);  // its first chunk of columns
+    constexpr int kMostCh = kBlk / kChunk * 4 / EPI;  // ... of at most
+    const int r_own = quarter * 32 + lane;  // this thread's tile row in phase 1
+    const uint32_t taddr = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
     int g = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++g) {
       const TItem it = resolve<BATCH, SMALL, PACK, KT>(p, &raw_map, item, n_items);
@@ -537,8 +527,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int t128 = 128 * it.n_kt * KT;  // 128 T over the padded block (padding decodes to u = 8 + 8i)
       const bool magic = t128 <= 128 * kMagicSamples;
       int2* out_c = it.out + (int64_t)c * it.n_pairs;
-      const int row0 = I * kBlk + warp * 32;
-      const int buf = g & 1;
+      const int row0 = I * kBlk + quarter * 32;
       if (ADD && !SMALL) {
         // the sums this tile pair adds to, pulled into L2 while its MMAs run: each thread
         // prefetches the 128-byte lines of its own row's segment (pairs J*128 .. min(J*128 + 127, i))
@@ -551,40 +540,91 @@ __global__ void __launch_bounds__(kThreads, 1)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(l < a ? a : l));
         }
       }
-      if (!mbar_wait_warp(tfull, g & 1, abort_flag, p.status, DEV_TIMEOUT_TMEM_FULL) ||
-          !mbar_wait_warp(&sfull[buf], (g >> 1) & 1, abort_flag, p.status, DEV_TIMEOUT_TMEM_FULL))
-        break;
+      // (a warp whose wait runs out still meets the others at the barrier, where all of them leave)
+      bool ok = mbar_wait_warp(tfull, g & 1, abort_flag, p.status, DEV_TIMEOUT_TMEM_FULL);
       tc_fence_after();
       // 16-pair chunks this warp keeps: none past the inputs (the packed channels), none wholly
       // above the diagonal
-      const int n_ch = (packed ? (warp * 32 >= it.pack_g * it.pitch || c * it.pack_g + (warp * 32) / it.pitch >= it.n_chan)
+      const int n_ch = !ok ? 0
+                       : (packed ? (quarter * 32 >= it.pack_g * it.pitch || c * it.pack_g + (quarter * 32) / it.pitch >= it.n_chan)
                                : row0 >= n_inputs)
                            ? 0
-                       : I == J ? (warp * 32 + 31) / kChunk + 1
-                                : kBlk / kChunk;
+                       : min(ch0 + kMostCh, I == J ? (quarter * 32 + 31) / kChunk + 1 : kBlk / kChunk);
       {
         uint4* srow = reinterpret_cast<uint4*>(staging + r_own * kBlk);
         const int sw = staging_swizzle(r_own);
-        for (int ch = 0; ch < n_ch; ++ch) {
-          uint32_t re[16], nim[16];
-          tmem_ld16(taddr + kChunk * ch, re);
-          tmem_ld16(taddr + 128 + kChunk * ch, nim);
-          tmem_ld_wait();
-          tmem_st16(taddr + kStashCol + kChunk * ch, nim);
-          // 16-byte piece q of the chunk holds columns 2q, 2q + 1, 8 + 2q, 9 + 2q (phase 2's order)
+        for (int ch = ch0; ch < n_ch; ch += 2) {  // (n_ch is even) two chunks' loads in flight
+          uint32_t re[2][16], nim[2][16];
 #pragma unroll
-          for (int q = 0; q < kChunk / 4; ++q)
-            srow[((kChunk * ch) / 4 + q) ^ sw] = make_uint4(re[2 * q], re[2 * q + 1], re[8 + 2 * q], re[9 + 2 * q]);
+          for (int h = 0; h < 2; ++h) {
+            tmem_ld16(taddr + kChunk * (ch + h), re[h]);
+            tmem_ld16(taddr + 128 + kChunk * (ch + h), nim[h]);
+          }
+          tmem_ld_wait();
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            tmem_st16(taddr + kStashCol + kChunk * (ch + h), nim[h]);
+            // 16-byte piece q of the chunk holds columns 2q, 2q + 1, 8 + 2q, 9 + 2q (phase 2's order)
+#pragma unroll
+            for (int q = 0; q < kChunk / 4; ++q)
+              srow[((kChunk * (ch + h)) / 4 + q) ^ sw] =
+                  make_uint4(re[h][2 * q], re[h][2 * q + 1], re[h][8 + 2 * q], re[h][9 + 2 * q]);
+          }
         }
-        // Re = n_re - 8 P_a - 8 P_b + 128 T,  Im = -n_im - 8 Q_a + 8 Q_b: the row's part
-        const int2 rs = sums[(buf * 2) * kBlk + r_own];  // (8P, 8Q) of this row's input
-        rowc[r_own] = make_int2(t128 - rs.x - (magic ? kMagicBits : 0), -rs.y + (magic ? kMagicBits : 0));
       }
       // the accumulator (columns 0-255) is free once its loads have landed; the stash stores
       // (columns 256-383) need only land before phase 2 reads them
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty);
+      // The code sums.  Columns: warp w adds up word w of the 32 threads of each chunk (lane = chunk + 8 x
+      // phase % 4), in 16-bit lanes for two threads (each at most 15 T / 32 <= 17,460), then wider.
+      if (warp < 4) {
+        ok = ok && mbar_wait_warp(sfull, g & 1, abort_flag, p.status, DEV_TIMEOUT_TMEM_FULL);
+        int s[8] = {};
+#pragma unroll
+        for (int k = 0; k < kDecWarps; k += 2) {
+          const uint4 x = dump[warp * kDecThreads + 32 * k + lane], y = dump[warp * kDecThreads + 32 * k + 32 + lane];
+          const uint32_t w[4] = {x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            s[2 * q] += static_cast<int>(w[q] & 0xFFFFu);
+            s[2 * q + 1] += static_cast<int>(w[q] >> 16);
+          }
+        }
+        // row: its four lanes of decoder warp (ib / 2) + 4 (ib % 2), inputs lane / 4 and + 8
+        const int ib = r_own >> 4, dw = (ib >> 1) + 4 * (ib & 1);
+        const uint2* ra = reinterpret_cast<const uint2*>(dump + 4 * kDecThreads + dw * 32 + 4 * (r_own & 7)) + ((r_own >> 3) & 1);
+        int row_re = 0, row_im = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint2 x = ra[2 * k];
+          row_re += static_cast<int>(x.x);
+          row_im += static_cast<int>(x.y);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sempty);
+        // Re = n_re - 8 P_a - 8 P_b + 128 T,  Im = -n_im - 8 Q_a + 8 Q_b with P = S_re + S_im, Q = S_im -
+        // S_re: the row's part
+        rowc[r_own] = make_int2(t128 - 8 * (row_re + row_im) - (magic ? kMagicBits : 0),
+                                -8 * (row_im - row_re) + (magic ? kMagicBits : 0));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          s[q] += __shfl_xor_sync(0xFFFFFFFFu, s[q], 8);
+          s[q] += __shfl_xor_sync(0xFFFFFFFFu, s[q], 16);
+        }
+        if (lane < 8) {
+          int4* dst = reinterpret_cast<int4*>(code_sums + (warp >> 1) * kBlk + 16 * lane + 8 * (warp & 1));
+          dst[0] = make_int4(s[0], s[1], s[2], s[3]);
+          dst[1] = make_int4(s[4], s[5], s[6], s[7]);
+        }
+      }
+      if (epi_bar_or<EPI>(!ok)) break;
+      if (warp < 4) {
+        const int c_re = code_sums[r_own], c_im = code_sums[kBlk + r_own];
+        sums[(g & 1) * kBlk + r_own] = make_int2(8 * (c_re + c_im), 8 * (c_im - c_re));
+      }
+      epi_bar_sync<EPI>();
       // phase 2 reads stash lanes that other threads of the warp stored
       tmem_st_wait();
       tc_fence_before();
@@ -592,14 +632,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_after();
       // phase 2: thread (rg, q) = (lane / 4, lane % 4) owns rows 32 warp + rg + 8m (m = 0..3) and,
       // in each 16-column chunk, columns 2q, 2q + 1, 8 + 2q, 9 + 2q
-      const int2* cs = sums + (buf * 2 + (I == J ? 0 : 1)) * kBlk;  // (8P, 8Q) of the columns
+      const int2* cs = sums + (g & 1) * kBlk;  // (8P, 8Q) of the columns
       const int q4 = lane & 3, rg = lane >> 2;
       int2* row_out[4];  // the row's pairs (j = first .. last of the tile), or null
       int firstm[4], lastm[4];
       int2 rcm[4];
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const int rr = warp * 32 + rg + 8 * m;
+        const int rr = quarter * 32 + rg + 8 * m;
         row_out[m] = nullptr;
         firstm[m] = 0;
         lastm[m] = I == J ? rr : kBlk - 1;  // last column of the row in the tile
@@ -616,7 +656,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (i < n_inputs) row_out[m] = out_c + (int64_t)i * (i + 1) / 2 + J * kBlk;
         }
       }
-      for (int ch = 0; ch < n_ch; ++ch) {
+      for (int ch = ch0; ch < n_ch; ++ch) {
         uint32_t im[2][8];  // [rows 0-15 | 16-31 of the warp][2j + h .. : column 8j + 2q + e of row rg + 8h]
         tmem_ld_16x256b_x2(taddr + kStashCol + kChunk * ch, im[0]);
         tmem_ld_16x256b_x2(taddr + (16u << 16) + kStashCol + kChunk * ch, im[1]);
@@ -624,27 +664,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int4 s0 = *reinterpret_cast<const int4*>(cs + jc);  // (8P, 8Q) of columns jc, jc + 1
         const int4 s1 = *reinterpret_cast<const int4*>(cs + jc + 8);
         const int sp[4] = {s0.x, s0.z, s1.x, s1.z}, sq[4] = {s0.y, s0.w, s1.y, s1.w};
-        int2 old[4][4];  // the chunk's earlier sums
-        if (ADD) {
-#pragma unroll
-          for (int m = 0; m < 4; ++m)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int j = jc + 8 * (k >> 1) + (k & 1);
-              old[m][k] = row_out[m] != nullptr && j <= lastm[m] && j >= firstm[m] ? row_out[m][j - firstm[m]]
-                                                                                   : make_int2(0, 0);
-            }
-        } else {
-#pragma unroll
-          for (int m = 0; m < 4; ++m)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) old[m][k] = make_int2(0, 0);
-        }
-        tmem_ld_wait();
+        int2 old[2][4] = {};  // ADD: the earlier sums of two of the thread's rows, in flight together
+        if (!ADD) tmem_ld_wait();
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
+          if (ADD && m % 2 == 0) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const int mm = m + (k >> 2), j = jc + 8 * ((k >> 1) & 1) + (k & 1);
+              old[k >> 2][k & 3] = row_out[mm] != nullptr && j <= lastm[mm] && j >= firstm[mm]
+                                       ? row_out[mm][j - firstm[mm]]
+                                       : make_int2(0, 0);
+            }
+            if (m == 0) tmem_ld_wait();
+          }
           if (row_out[m] == nullptr) continue;
-          const int rr = warp * 32 + rg + 8 * m;
+          const int rr = quarter * 32 + rg + 8 * m;
           const int first = firstm[m], last = lastm[m];
           if (jc > last || jc + 9 < first) continue;
           const uint4 re4 =
@@ -667,8 +702,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 nr = __float2int_rn(__uint_as_float(xr) * 262144.0f);
                 ni = __float2int_rn(__uint_as_float(xi) * 262144.0f);
               }
-              v[e] = make_int2(nr + rcm[m].x - sp[2 * jj + e] + old[m][2 * jj + e].x,
-                               -ni + rcm[m].y + sq[2 * jj + e] + old[m][2 * jj + e].y);
+              v[e] = make_int2(nr + rcm[m].x - sp[2 * jj + e] + old[m & 1][2 * jj + e].x,
+                               -ni + rcm[m].y + sq[2 * jj + e] + old[m & 1][2 * jj + e].y);
             }
             // (first is a multiple of 16 and j0 even: a pair of columns starts inside the row or before it)
             if (j0 > last || j0 < first) continue;
@@ -692,9 +727,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      // the input sums are free
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sempty[buf]);
     }
   }
 
@@ -706,10 +738,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-template <int KT, int RAW, int DEC, bool BATCH, bool SMALL, bool PACK, bool ADD>
+template <int KT, int RAW, int DEC, bool BATCH, bool SMALL, bool PACK, bool ADD, int EPI>
 cudaError_t launch_ta_kernel(const CUtensorMap& raw_map, const TParams& p, int grid, cudaStream_t stream) {
   using G = TGeom<KT, RAW, DEC>;
-  auto kern = xcorr_tc_fused_ta_kernel<KT, RAW, DEC, BATCH, SMALL, PACK, ADD>;
+  auto kern = xcorr_tc_fused_ta_kernel<KT, RAW, DEC, BATCH, SMALL, PACK, ADD, EPI>;
   static int attr_device = -1;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -719,14 +751,28 @@ cudaError_t launch_ta_kernel(const CUtensorMap& raw_map, const TParams& p, int g
     if (e != cudaSuccess) return e;
     attr_device = dev;
   }
-  return launch_dependent(kern, grid, kThreads, G::kSmem, stream, raw_map, p);
+  return launch_dependent(kern, grid, Roles<EPI>::kThreads, G::kSmem, stream, raw_map, p);
 }
+
+// Eight epilogue warps write a tile pair in 5.5 us, four in 6.8, the time it takes to decode 1160 samples;
+// past that the four win, as they leave the decoders 128 registers (152 channels of 512 inputs, ten tile
+// pairs a CTA: 1024 samples 90.7 us with eight, 95.3 with four; 1152 98.2 and 97.9; 2048 149.3 and 146.1).
+// An adding epilogue waits for the earlier sums, so its line lies higher (1024 samples 122 us with eight,
+// 135 with four; 2048 equal; 4096 287 and 285), as does that of a batch, whose items' lengths are mixed
+// (24 subarrays of 1150 samples an item on average 117 us with eight, 127 with four; ten of 3660 101 and 99).
+constexpr int kShortSamples = 1088, kShortAddedSamples = 2048;
 
 template <int KT, int RAW, int DEC, bool BATCH = false, bool SMALL = false, bool PACK = false>
 cudaError_t launch_ta(const CUtensorMap& raw_map, const TParams& p, int grid, cudaStream_t stream) {
-  if (!BATCH && p.accumulate && !p.atomic_out)
-    return launch_ta_kernel<KT, RAW, DEC, false, SMALL, PACK, !BATCH>(raw_map, p, grid, stream);
-  return launch_ta_kernel<KT, RAW, DEC, BATCH, SMALL, PACK, false>(raw_map, p, grid, stream);
+  const int samples = p.n_kt * KT;
+  if (!BATCH && p.accumulate && !p.atomic_out) {
+    if (!SMALL && samples > kShortAddedSamples)
+      return launch_ta_kernel<KT, RAW, DEC, false, false, false, !BATCH, 4>(raw_map, p, grid, stream);
+    return launch_ta_kernel<KT, RAW, DEC, false, SMALL, PACK, !BATCH, 8>(raw_map, p, grid, stream);
+  }
+  if (!SMALL && samples > (BATCH ? kShortAddedSamples : kShortSamples))
+    return launch_ta_kernel<KT, RAW, DEC, BATCH, false, false, false, 4>(raw_map, p, grid, stream);
+  return launch_ta_kernel<KT, RAW, DEC, BATCH, SMALL, PACK, false, 8>(raw_map, p, grid, stream);
 }
 
 }  // namespace
@@ -822,8 +868,8 @@ namespace xc {
 // The batch form: one launch over items (subarray, channel, I, J) of several 4-bit problems, each
 // with its own descriptor (raw tensor map with box_t = the variant's stage height, output, sizes;
 // one exactly-summed block each: n_kt * KT <= kFusedWindowCI4).
-cudaError_t launch_xcorr_tc_fused_ta_batch(const TaSubDesc* subs, const uint4* items, int n_items, int variant,
-                                           int* status, int num_sms, cudaStream_t stream) {
+cudaError_t launch_xcorr_tc_fused_ta_batch(const TaSubDesc* subs, const uint4* items, int n_items, int mean_stages,
+                                           int variant, int* status, int num_sms, cudaStream_t stream) {
   if (n_items <= 0) return cudaSuccess;
   TParams p{};
   p.status = status;
@@ -832,6 +878,7 @@ cudaError_t launch_xcorr_tc_fused_ta_batch(const TaSubDesc* subs, const uint4* i
   p.subs = subs;
   p.items = items;
   p.n_batch_items = n_items;
+  p.n_kt = mean_stages;  // (the kernel takes every item's own)
   CUtensorMap unused{};
   const int grid = n_items < num_sms ? n_items : num_sms;
   switch (variant) {

@@ -384,3 +384,29 @@ def test_host_to_host_in_groups(torch, fmt, n_sta, n_chan, n_time, n_groups):
             out = plan.execute_dump_host(torch.from_numpy(x).pin_memory(), n_groups=n_groups)
             plan.sync()
         check(fmt, out.numpy(), x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("variant", [4, 5, 6])
+@pytest.mark.parametrize("n_sta,n_chan,n_time", [(64, 5, 1088), (64, 5, 1089), (72, 170, 1152), (136, 30, 2049), (64, 320, 2300)])
+def test_epilogue_of_short_and_long_items(torch, variant, n_sta, n_chan, n_time):
+    """Both numbers of epilogue warps on either side of their lines, storing then adding; several items a CTA."""
+    x = draw("ci4", n_time, n_chan, n_sta, seed=n_time)
+    xd = torch.from_numpy(x).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="ci4", engine="tensor") as plan:
+        plan.set_tuning(variant, 0, 2, 0)
+        plan.execute(xd)
+        plan.execute(xd[:n_time // 2].contiguous())
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check("ci4", got, np.concatenate([x, x[:n_time // 2]]), 2 * n_sta)
+
+
+def test_batch_of_long_items(torch):
+    subs = [(64, 30, 2500), (16, 40, 3000), (72, 50, 2100)]
+    xs = [draw("ci4", t, c, s, seed=s + c + t) for s, c, t in subs]
+    batch = xcorr.Batch(subs)
+    outs = batch.execute([torch.from_numpy(x).cuda() for x in xs])
+    batch.sync()
+    for x, out in zip(xs, outs):
+        check("ci4", out.cpu().numpy(), x, 2 * x.shape[2])
+    batch.close()

@@ -352,6 +352,8 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
       uint32_t s_re[8], s_im[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) s_re[q] = s_im[q] = 0u;
+      uint32_t a_re[4] = {0u, 0u, 0u, 0u}, a_im[4] = {0u, 0u, 0u, 0u};  // byte lanes: at most 15 R a stage
+      constexpr int kWiden = 255 / (15 * G::kRowsB);                      // stages that they hold
       bool ok = true;
       for (int tb = 0; tb < cur.n_kt; ++tb) {
         if (!mbar_wait_warp(&raw_full[r], rph, abort_flag, p.status, DEV_TIMEOUT_FULL) ||
@@ -365,6 +367,7 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
         // A operand: two blocks of 16 samples x 16 inputs per ldmatrix (thread t addresses row
         // 16 sb + t, both blocks under the same swizzle since 16 sb = 0 mod 8), decoded in
         // registers, stored to TMEM eight columns at a time
+        uint32_t br0 = 0u, bi0 = 0u, br1 = 0u, bi1 = 0u;  // the stage's codes per byte: <= 15 KT / 16
         const uint32_t ta = tmem + a_lanes + kAcol0 + static_cast<uint32_t>(d * G::kAcols);
         static_assert(KT % 32 == 0, "whole pairs of 16-sample blocks");
         // four blocks per pair of stores (sixteen columns), then a pair of blocks if KT / 16 is
@@ -382,11 +385,10 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
             offset_codes(x1, re[4 * h + 1], im[4 * h + 1]);
             offset_codes(x2, re[4 * h + 2], im[4 * h + 2]);
             offset_codes(x3, re[4 * h + 3], im[4 * h + 3]);
-            // the two blocks' codes of one input add per byte (<= 30) before the dp4a
-            sar0 = __dp4a(re[4 * h] + re[4 * h + 2], 0x01010101u, sar0);
-            sai0 = __dp4a(im[4 * h] + im[4 * h + 2], 0x01010101u, sai0);
-            sar1 = __dp4a(re[4 * h + 1] + re[4 * h + 3], 0x01010101u, sar1);
-            sai1 = __dp4a(im[4 * h + 1] + im[4 * h + 3], 0x01010101u, sai1);
+            br0 += re[4 * h] + re[4 * h + 2];
+            bi0 += im[4 * h] + im[4 * h + 2];
+            br1 += re[4 * h + 1] + re[4 * h + 3];
+            bi1 += im[4 * h + 1] + im[4 * h + 3];
           }
           if (nb == 2) {
             tmem_st_16x128b_x4(ta + 4 * sb, re);
@@ -396,6 +398,10 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
             tmem_st_16x128b_x2(ta + KT / 4 + 4 * sb, im[0], im[1], im[2], im[3]);
           }
         }
+        sar0 = __dp4a(br0, 0x01010101u, sar0);
+        sai0 = __dp4a(bi0, 0x01010101u, sai0);
+        sar1 = __dp4a(br1, 0x01010101u, sar1);
+        sai1 = __dp4a(bi1, 0x01010101u, sai1);
         // B operand: real and imaginary planes in shared memory at the raw chunk's swizzled offset
         {
           constexpr int R = G::kRowsB;
@@ -405,7 +411,6 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
           uint4 v[R];
 #pragma unroll
           for (int k = 0; k < R; ++k) v[k] = *reinterpret_cast<const uint4*>(src + (phase + 32 * k) * 128);
-          uint32_t a_re[4] = {0u, 0u, 0u, 0u}, a_im[4] = {0u, 0u, 0u, 0u};  // byte lanes: <= 15 R <= 60
 #pragma unroll
           for (int k = 0; k < R; ++k) {
             uint4 re, im;
@@ -421,13 +426,16 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
             *reinterpret_cast<uint4*>(re_t + off) = re;
             *reinterpret_cast<uint4*>(im_t + off) = im;
           }
-          // widen to 16-bit lanes: inputs (4q, 4q+1) -> word 2q, (4q+2, 4q+3) -> word 2q+1
+          // widen to 16-bit lanes when the bytes are full (every stage: 1 % slower): inputs (4q, 4q+1) -> word 2q, (4q+2, 4q+3) -> word 2q+1
+          if (tb % kWiden == kWiden - 1 || tb + 1 == cur.n_kt) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            lane_add(s_re[2 * q], __byte_perm(a_re[q], 0u, 0x4140), p.one);
-            lane_add(s_re[2 * q + 1], __byte_perm(a_re[q], 0u, 0x4342), p.one);
-            lane_add(s_im[2 * q], __byte_perm(a_im[q], 0u, 0x4140), p.one);
-            lane_add(s_im[2 * q + 1], __byte_perm(a_im[q], 0u, 0x4342), p.one);
+            for (int q = 0; q < 4; ++q) {
+              lane_add(s_re[2 * q], __byte_perm(a_re[q], 0u, 0x4140), p.one);
+              lane_add(s_re[2 * q + 1], __byte_perm(a_re[q], 0u, 0x4342), p.one);
+              lane_add(s_im[2 * q], __byte_perm(a_im[q], 0u, 0x4140), p.one);
+              lane_add(s_im[2 * q + 1], __byte_perm(a_im[q], 0u, 0x4342), p.one);
+              a_re[q] = a_im[q] = 0u;
+            }
           }
         }
         // the MMA reads A through tensor memory and B through the async proxy

@@ -601,8 +601,13 @@ xcorr_status xcorr_execute(xcorr_plan plan, const void* d_in, int n_time, void* 
   return XCORR_OK;
 }
 
-xcorr_status xcorr_dump(xcorr_plan plan, void* out, int out_on_device, unsigned flags, void* stream,
-                        int64_t* n_samples) {
+}  // extern "C"
+
+namespace {
+
+// store: a wide output is written, not added to.
+xcorr_status dump(xcorr_plan plan, void* out, int out_on_device, unsigned flags, bool store, void* stream,
+                  int64_t* n_samples) {
   xc::NvtxRange range("xcorr_dump");
   xcorr_status st = plan_ok(plan);
   if (st != XCORR_OK) return st;
@@ -623,9 +628,9 @@ xcorr_status xcorr_dump(xcorr_plan plan, void* out, int out_on_device, unsigned 
   }
   if (wide) {
     if (plan->cfg.fmt == XCORR_IN_CF32)
-      e = xc::launch_fold_wide_f64(static_cast<const float2*>(plan->acc), static_cast<double*>(out), total, s);
+      e = xc::launch_fold_wide_f64(static_cast<const float2*>(plan->acc), static_cast<double*>(out), total, !store, s);
     else
-      e = xc::launch_fold_wide_i64(static_cast<const int2*>(plan->acc), static_cast<int64_t*>(out), total, s);
+      e = xc::launch_fold_wide_i64(static_cast<const int2*>(plan->acc), static_cast<int64_t*>(out), total, !store, s);
     if (e != cudaSuccess) return cuda_fail(e, "fold launch");
   } else {
     e = cudaMemcpyAsync(out, plan->acc, bytes, out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
@@ -639,6 +644,21 @@ xcorr_status xcorr_dump(xcorr_plan plan, void* out, int out_on_device, unsigned 
     plan->fresh = true;
   }
   return XCORR_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+xcorr_status xcorr_dump(xcorr_plan plan, void* out, int out_on_device, unsigned flags, void* stream,
+                        int64_t* n_samples) {
+  return dump(plan, out, out_on_device, flags, false, stream, n_samples);
+}
+
+// For the Python binding, which makes the wide output itself: xcorr_dump with XCORR_DUMP_ADD_WIDE into
+// device memory that holds zeros, without the zeros.
+xcorr_status xcorr_dump_wide_new_(xcorr_plan plan, void* out, unsigned flags, void* stream, int64_t* n_samples) {
+  return dump(plan, out, 1, flags | XCORR_DUMP_ADD_WIDE, true, stream, n_samples);
 }
 
 xcorr_status xcorr_accum_load(xcorr_plan plan, const void* src, int src_on_device, int64_t n_samples, void* stream) {

@@ -275,7 +275,7 @@ xcorr_status execute_into(xcorr_plan plan, const void* d_in, int n_time, void* t
 xcorr_status read_device_status(xcorr_plan plan);
 
 cudaError_t launch_fold_wide_i64(const int2* acc, int64_t* out, int64_t n_pairs_total,
-                                 cudaStream_t stream);
+                                 bool add, cudaStream_t stream);
 
 // Encode the 3-D tensor map over planes of elem_bytes-byte numbers (dims:
 // input, time, channel * planes_per_chan + plane), box 128 bytes x box_t rows.
@@ -345,6 +345,6 @@ cudaError_t launch_repitch(const void* in, const void* end, void* out, int row_b
 cudaError_t launch_unpack_cf32_digits(const float* in, uint16_t* planes, int16_t* exps, int n_time, int n_chan,
                                       int c0, int nc, int n_inputs, int ni_pad, int max_time, int window,
                                       int exp_windows, cudaStream_t stream);
-cudaError_t launch_fold_wide_f64(const float2* acc, double* out, int64_t n_pairs_total, cudaStream_t stream);
+cudaError_t launch_fold_wide_f64(const float2* acc, double* out, int64_t n_pairs_total, bool add, cudaStream_t stream);
 
 }  // namespace xc

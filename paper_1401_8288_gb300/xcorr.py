@@ -119,6 +119,7 @@ def load():
                 "xcorr_plan_create": [ctypes.POINTER(vp), ctypes.POINTER(xcorr_config)],
                 "xcorr_execute": [vp, vp, i, vp],
                 "xcorr_dump": [vp, vp, i, u, vp, ctypes.POINTER(i64)],
+                "xcorr_dump_wide_new_": [vp, vp, u, vp, ctypes.POINTER(i64)],
                 "xcorr_execute_dump": [vp, vp, i, vp, i, u, vp, ctypes.POINTER(i64)],
                 "xcorr_accum_load": [vp, vp, i, i64, vp],
                 "xcorr_sync": [vp, vp],
@@ -209,6 +210,13 @@ def xcorr_execute(plan, d_in: int, n_time: int, stream: int = 0) -> None:
 def xcorr_dump(plan, out: int, out_on_device: bool, flags: int = 0, stream: int = 0) -> int:
     n = ctypes.c_int64()
     _check(load().xcorr_dump(plan, out, int(out_on_device), flags, stream, ctypes.byref(n)))
+    return n.value
+
+
+def _dump_wide_new(plan, out: int, flags: int = 0, stream: int = 0) -> int:
+    """A wide dump into device memory that needs no clearing."""
+    n = ctypes.c_int64()
+    _check(load().xcorr_dump_wide_new_(plan, out, flags, stream, ctypes.byref(n)))
     return n.value
 
 
@@ -702,9 +710,13 @@ class Plan:
     def dump(self, out=None, reset: bool = True, wide: bool = False, stream=None):
         torch = self._torch
         shape = (self.n_channels, self.info["n_pairs"], 2)
-        if out is None:
-            # wide dumps add to what is there; the others write every entry
-            out = (torch.zeros if wide else torch.empty)(shape, dtype=self._out_dtype(wide), device="cuda")
+        new = out is None
+        if new:  # (every entry is written)
+            out = torch.empty(shape, dtype=self._out_dtype(wide), device="cuda")
+        if new and wide:
+            self.samples = _dump_wide_new(self.handle, out.data_ptr(), XCORR_DUMP_RESET if reset else 0,
+                                          self._stream(stream))
+            return out
         flags = (XCORR_DUMP_RESET if reset else 0) | (XCORR_DUMP_ADD_WIDE if wide else 0)
         self.samples = xcorr_dump(self.handle, out.data_ptr(), out.is_cuda, flags,
                                   self._stream(stream))
@@ -724,9 +736,11 @@ class Plan:
         torch = self._torch
         if not x.is_cuda or not x.is_contiguous():
             raise ValueError("input must be a contiguous CUDA tensor")
+        if out is None and wide:  # (the two calls that a wide xcorr_execute_dump is)
+            self.execute(x, stream=stream)
+            return self.dump(reset=reset, wide=True, stream=stream)
         if out is None:
-            out = (torch.zeros if wide else torch.empty)((self.n_channels, self.info["n_pairs"], 2),
-                                                         dtype=self._out_dtype(wide), device="cuda")
+            out = torch.empty((self.n_channels, self.info["n_pairs"], 2), dtype=self._out_dtype(wide), device="cuda")
         flags = (XCORR_DUMP_RESET if reset else 0) | (XCORR_DUMP_ADD_WIDE if wide else 0)
         self.samples = xcorr_execute_dump(self.handle, x.data_ptr(), x.shape[0], out.data_ptr(),
                                           out.is_cuda, flags, self._stream(stream))

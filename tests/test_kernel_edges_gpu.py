@@ -410,3 +410,22 @@ def test_batch_of_long_items(torch):
     for x, out in zip(xs, outs):
         check("ci4", out.cpu().numpy(), x, 2 * x.shape[2])
     batch.close()
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time", [("ci4", 1, 1, 3), ("ci4", 9, 5, 70), ("ci8", 65, 3, 40), ("cf32", 1, 1, 9), ("cf32", 33, 5, 400)])
+def test_wide_dump_into_a_new_buffer(torch, fmt, n_sta, n_chan, n_time):
+    """The buffer a wide dump makes itself holds what adding to zeros gives (odd and even pair counts),
+    also where the allocator hands out memory that held other numbers."""
+    x = torch.from_numpy(draw(fmt, n_time, n_chan, n_sta, seed=2)).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt) as plan:
+        zeros = torch.zeros((n_chan, plan.info["n_pairs"], 2), dtype=torch.float64 if fmt == "cf32" else torch.int64, device="cuda")
+        plan.execute(x)
+        plan.dump(out=zeros, reset=False, wide=True)
+        torch.full_like(zeros, -7)
+        torch.cuda.synchronize()
+        assert torch.equal(plan.dump(wide=True), zeros) and plan.samples == n_time
+        torch.full_like(zeros, -7)
+        assert torch.equal(plan.execute_dump(x, wide=True), zeros)
+        empty = plan.dump(wide=True)  # nothing integrated since the reset
+        assert not empty.any() and plan.samples == 0
+        plan.sync()

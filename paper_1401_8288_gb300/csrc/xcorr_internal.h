@@ -173,6 +173,9 @@ cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned bloc
   return launch_dependent_clusters(kernel, 1, grid, block, smem, stream, args...);
 }
 
+// Zeros to `pairs` 8-byte sums, by a kernel that the next one may start behind (xcorr_dump.cu).
+cudaError_t launch_clear(void* out, int64_t pairs, cudaStream_t stream);
+
 // Launchers; each returns the launch's cudaError_t.
 cudaError_t launch_unpack_ci4_e4m3(const uint8_t* in, uint8_t* planes, int n_time, int n_chan,
                                    int n_inputs, int ni_pad, int max_time, int num_sms,

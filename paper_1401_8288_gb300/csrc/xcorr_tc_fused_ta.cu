@@ -848,7 +848,7 @@ cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int v
     p.atomic_out = p.n_split > 1 ? 1 : 0;
     p.n_items = tiles * p.n_split;
     if (p.atomic_out && !p.accumulate) {  // the split items add into a cleared output
-      cudaError_t e = cudaMemsetAsync(out, 0, (size_t)n_chan * p.n_pairs * sizeof(int2), stream);
+      cudaError_t e = launch_clear(out, (int64_t)n_chan * p.n_pairs, stream);
       if (e != cudaSuccess) return e;
       p.accumulate = 1;
     }

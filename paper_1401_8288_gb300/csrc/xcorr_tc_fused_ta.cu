@@ -135,7 +135,8 @@ struct TParams {
   // each tile's stages cut into n_split items of split_kt stages whose results are added with
   // atomics (atomic_out)
   int pack_g, n_split, split_kt, atomic_out;
-  int n_items;         // items of a non-batch launch: tiles x n_split
+  int tail_first;      // items before this one are whole tiles (only the last ones are split)
+  int n_items;         // items of a non-batch launch: tail_first whole tiles, then the others x n_split
   int2* out;
   int* status;
   uint32_t one;        // 1: a multiplier the compiler cannot fold (see lane_add)
@@ -156,6 +157,7 @@ struct TItem {
   int t_first;             // first sample of the item
   int ax, ay, bx, by;      // TMA coordinates (input or channel-input column, channel) of the row and column tiles
   bool diag, valid;
+  bool split;              // a part of a tile's stages: its sums are added with atomics
 };
 
 template <bool BATCH, bool SMALL, bool PACK, int KT>
@@ -190,10 +192,13 @@ __device__ __forceinline__ TItem resolve(const TParams& p, const CUtensorMap* ma
     it.n_kt = p.n_kt;
     it.t_first = p.t0;
     if (SMALL) {  // the time split of the small-problem layout
-      tile = item / p.n_split;
-      const int split = item - tile * p.n_split;
-      it.n_kt = min(p.split_kt, p.n_kt - split * p.split_kt);
-      it.t_first = p.t0 + split * p.split_kt * KT;
+      if (item >= p.tail_first) {
+        tile = p.tail_first + (item - p.tail_first) / p.n_split;
+        const int split = (item - p.tail_first) % p.n_split;
+        it.n_kt = min(p.split_kt, p.n_kt - split * p.split_kt);
+        it.t_first = p.t0 + split * p.split_kt * KT;
+        it.split = p.atomic_out != 0;
+      }
     }
     if (PACK) {  // tile = a group of pack_g channels, one diagonal tile pair
       it.c = tile;
@@ -717,7 +722,7 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
             if (j0 > last || j0 < first) continue;
             int2* dst = row_out[m] + (j0 - first);
             const int nv = j0 + 1 <= last ? 2 : 1;
-            if (SMALL && !ADD && p.atomic_out) {  // time-split items of one tile add into the same pairs
+            if (SMALL && !ADD && it.split) {  // time-split items of one tile add into the same pairs
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 if (e < nv) {
@@ -778,6 +783,8 @@ cudaError_t launch_ta(const CUtensorMap& raw_map, const TParams& p, int grid, cu
       return launch_ta_kernel<KT, RAW, DEC, false, false, false, !BATCH, 4>(raw_map, p, grid, stream);
     return launch_ta_kernel<KT, RAW, DEC, false, SMALL, PACK, !BATCH, 8>(raw_map, p, grid, stream);
   }
+  if (SMALL && !PACK && p.tail_first > 0 && samples > kShortSamples)
+    return launch_ta_kernel<KT, RAW, DEC, false, SMALL, false, false, 4>(raw_map, p, grid, stream);
   if (!SMALL && samples > (BATCH ? kShortAddedSamples : kShortSamples))
     return launch_ta_kernel<KT, RAW, DEC, BATCH, false, false, false, 4>(raw_map, p, grid, stream);
   return launch_ta_kernel<KT, RAW, DEC, BATCH, SMALL, PACK, false, 8>(raw_map, p, grid, stream);
@@ -791,6 +798,8 @@ int fused_ta_stage_samples(int variant) { return variant == 0 || variant == 3 ? 
 
 int fused_ta_pack(int n_inputs) { return n_inputs <= kBlk / 2 ? kBlk / n_inputs : 1; }
 
+constexpr int kTailStages = 16, kTailParts = 4;
+
 // The small-problem layout of a launch: channels packed per tile and the time split.
 void small_layout(int n_chan, int n_inputs, int n_kt, int num_sms, int& pack_g, int& tiles, int& n_split,
                   int& split_kt) {
@@ -802,6 +811,23 @@ void small_layout(int n_chan, int n_inputs, int n_kt, int num_sms, int& pack_g, 
   if (n_split > n_kt) n_split = n_kt;
   split_kt = (n_kt + n_split - 1) / n_split;
   n_split = (n_kt + split_kt - 1) / split_kt;
+}
+
+// A last wave that leaves half of the SMs or more idle: its tiles' stages are split over them, up to four
+// parts a tile (sixteen parts that add into the same pairs wait for one another: 128 inputs x 160 channels
+// x 2048 samples 34.3 -> 35.3 us).  The stages that a tile is spared have to pay for the clearing and the
+// atomics: sixteen do (128 x 160 x 2800 43.4 -> 38.2, x 4096 59.3 -> 46.9; 200 x 64 x 4096 79.7 -> 68.2;
+// 256 x 256 x 4096 165 -> 157), twelve do not (256 x 256 x 2048 87.9 -> 90.9).
+void split_tail(int tiles, int num_sms, TParams& p) {
+  const int whole = tiles / num_sms * num_sms, rest = tiles - whole;
+  if (rest == 0 || 2 * rest > num_sms) return;
+  int n = num_sms / rest < kTailParts ? num_sms / rest : kTailParts;
+  if (n > p.n_kt) n = p.n_kt;
+  const int kt = (p.n_kt + n - 1) / n;
+  if (p.n_kt - kt < kTailStages) return;
+  p.tail_first = whole;
+  p.split_kt = kt;
+  p.n_split = (p.n_kt + kt - 1) / kt;
 }
 
 cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int variant, int n_time, int n_chan,
@@ -845,17 +871,23 @@ cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int v
     p.n_split = 1;
     p.split_kt = p.n_kt;
     if (small) small_layout(n_chan, pitch, p.n_kt, num_sms, pack_g, tiles, p.n_split, p.split_kt);
+    p.tail_first = 0;
+    if (kt == 128 && pack_g == 1 && p.n_split == 1 && !p.accumulate) split_tail(tiles, num_sms, p);
     p.atomic_out = p.n_split > 1 ? 1 : 0;
-    p.n_items = tiles * p.n_split;
-    if (p.atomic_out && !p.accumulate) {  // the split items add into a cleared output
-      cudaError_t e = launch_clear(out, (int64_t)n_chan * p.n_pairs, stream);
+    p.n_items = p.tail_first + (tiles - p.tail_first) * p.n_split;
+    if (p.atomic_out && !p.accumulate) {  // the split items add into a cleared output (the whole tiles of their channels overwrite theirs)
+      const int c0 = pack_g > 1 ? 0 : p.tail_first / p.n_tile_pairs;
+      cudaError_t e = launch_clear(out + c0 * p.n_pairs, (n_chan - c0) * p.n_pairs, stream);
       if (e != cudaSuccess) return e;
       p.accumulate = 1;
     }
     const int grid = p.n_items < num_sms ? p.n_items : num_sms;
     cudaError_t e;
     switch (variant) {
-      case 0: e = launch_ta<128, 2, 2>(raw_map, p, grid, stream); break;
+      case 0:
+        e = p.n_split > 1 ? launch_ta<128, 2, 2, false, true, false>(raw_map, p, grid, stream)
+                          : launch_ta<128, 2, 2>(raw_map, p, grid, stream);
+        break;
       case 1: e = launch_ta<96, 3, 2>(raw_map, p, grid, stream); break;
       case 2: e = launch_ta<64, 4, 4>(raw_map, p, grid, stream); break;
       default:  // the small-problem layout; with neither packing nor a split it is shape 0's launch

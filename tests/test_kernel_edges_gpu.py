@@ -429,3 +429,25 @@ def test_wide_dump_into_a_new_buffer(torch, fmt, n_sta, n_chan, n_time):
         empty = plan.dump(wide=True)  # nothing integrated since the reset
         assert not empty.any() and plan.samples == 0
         plan.sync()
+
+
+@pytest.mark.parametrize("n_sta,n_chan,n_time", [(64, 153, 2700), (72, 60, 4001), (64, 40, 3300), (136, 12, 4100), (61, 155, 2900), (100, 70, 4000),
+                                                 (64, 228, 2817), (64, 229, 2817), (40, 76, 4225), (40, 38, 2049)])
+@pytest.mark.parametrize("variant", [4, 10])
+def test_last_wave_split_over_the_idle_sms(torch, variant, n_sta, n_chan, n_time):
+    """Whole tiles, then parts of the last ones added into cleared channels; one part of one stage, part
+    counts that leave a short last part, launches that are a last wave altogether; then an adding
+    execute. Twice into a buffer that held other numbers."""
+    x = draw("ci4", n_time, n_chan, n_sta, seed=n_sta + n_time)
+    xd = torch.from_numpy(x).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="ci4", engine="tensor") as plan:
+        plan.set_tuning(variant, 0, 2, 0)
+        out = torch.full((n_chan, plan.info["n_pairs"], 2), -5, dtype=torch.int32, device="cuda")
+        for _ in range(2):
+            plan.execute_dump(xd, out)
+        check("ci4", out.cpu().numpy(), x, 2 * n_sta)
+        plan.execute(xd)
+        plan.execute(xd[:100].contiguous())
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check("ci4", got, np.concatenate([x, x[:100]]), 2 * n_sta)

@@ -30,7 +30,7 @@ __device__ __forceinline__ uint64_t global_ns() {
 // previous kernel have left (or called pdl_release), before its writes are flushed.  Before pdl_wait
 // returns it must not touch global memory: then the previous kernel has completed and its writes are
 // visible.  What comes before -- the launch, barriers, tensor memory -- overlaps the previous end.
-// Only the shortest kernel releases early: CTAs of the next kernel that sit on an SM waiting keep it
+// Only the shortest kernels release early: CTAs of the next kernel that sit on an SM waiting keep it
 // from that kernel's own better placement (float, 16 inputs x 64 channels x 1024: unpack and X 55 us,
 // with early releases 67).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

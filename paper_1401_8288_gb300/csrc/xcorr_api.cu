@@ -98,6 +98,8 @@ xcorr_status check_execute(xcorr_plan plan, const void* d_in, int n_time) {
   return XCORR_OK;
 }
 
+int packed_channels(xcorr_plan plan) { return (plan->cfg.n_channels + plan->pack - 1) / plan->pack; }
+
 // Channel groups of the tensor path: the tuned count, else enough tile pairs
 // per group for about four waves of the persistent X kernel.
 int tensor_groups(xcorr_plan plan) {
@@ -106,11 +108,11 @@ int tensor_groups(xcorr_plan plan) {
     g = plan->tune_groups;
   } else {
     const int nb = (plan->n_inputs + 127) / 128;
-    const int64_t items = (int64_t)plan->cfg.n_channels * nb * (nb + 1) / 2;
+    const int64_t items = (int64_t)packed_channels(plan) * nb * (nb + 1) / 2;
     g = items / (4LL * plan->num_sms);
   }
   if (g > xc::kMaxGroups) g = xc::kMaxGroups;
-  if (g > plan->cfg.n_channels) g = plan->cfg.n_channels;
+  if (g > packed_channels(plan)) g = packed_channels(plan);
   return g < 1 ? 1 : static_cast<int>(g);
 }
 
@@ -216,7 +218,7 @@ cudaError_t unpack_group(xcorr_plan plan, const void* d_in, int n_time, int c0, 
                                                  n_time, C, c0, nc, N, plan->ni_pad, T, plan->num_sms, s);
     default:
       return xc::launch_unpack_cf32_digits(static_cast<const float*>(d_in), static_cast<uint16_t*>(plan->planes),
-                                           plan->exps, n_time, C, c0, nc, N, plan->ni_pad, T, plan->window_samples,
+                                           plan->exps, n_time, C, c0, nc, N, plan->pack, plan->ni_pad, T, plan->window_samples,
                                            plan->exp_windows, s);
   }
 }
@@ -304,11 +306,12 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
     if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
   } else if (plan->engine == XCORR_ENGINE_TENSOR) {
-    const int variant = xc::planes_variant(plan->tune_variant);
+    const int variant = plan->pack > 1 ? 0 : xc::planes_variant(plan->tune_variant);
+    const int row_inputs = plan->pack > 1 ? plan->ni_pad : N, Cp = packed_channels(plan);
     if (plan->tmap_ntime != n_time || plan->tmap_variant != variant) {
       std::string err;
-      if (!xc::encode_plane_tmap(&plan->tmap, plan->planes, plan->elem_bytes, N, plan->ni_pad, n_time,
-                                 plan->cfg.max_time_per_exec, C * plan->planes_per_chan,
+      if (!xc::encode_plane_tmap(&plan->tmap, plan->planes, plan->elem_bytes, row_inputs, plan->ni_pad, n_time,
+                                 plan->cfg.max_time_per_exec, Cp * plan->planes_per_chan,
                                  xc::tc_stage_samples(plan->elem_bytes, variant), &err))
         return fail(XCORR_ERR_CUDA, err);
       plan->tmap_ntime = n_time;
@@ -319,7 +322,10 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     L.variant = variant;
     L.float_out = plan->cfg.fmt == XCORR_IN_CF32;
     L.n_time = n_time;
-    L.n_inputs = N;
+    L.n_inputs = row_inputs;
+    L.pack = plan->pack;
+    L.true_inputs = N;
+    L.true_chans = C;
     L.planes_per_chan = plan->planes_per_chan;
     if (plan->cfg.fmt == XCORR_IN_CF32) {
       // the six digit products d_p d_q with p + q <= 2
@@ -339,11 +345,11 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     L.status = plan->status;
     L.num_sms = plan->num_sms;
     const int G = tensor_groups(plan);
-    const int per = (C + G - 1) / G;
+    const int per = (Cp + G - 1) / G;
     const int nxs = plan->tune_x_streams == 1 ? 1 : 2;
     // several groups: the internal streams fork from s after everything queued on it so far (one
     // group's two launches follow one another on s itself)
-    const bool forked = per < C;
+    const bool forked = per < Cp;
     cudaStream_t su = forked ? plan->s_unpack : s;
     if (forked) {
       if ((e = cudaEventRecord(plan->ev_fork, s)) != cudaSuccess) return cuda_fail(e, "fork event");
@@ -353,9 +359,11 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
         return cuda_fail(e, "fork wait");
     }
     int used = 0;
-    for (int g = 0, c0 = 0; c0 < C; ++g, c0 += per) {
-      const int nc = (C - c0 < per) ? C - c0 : per;
-      if ((e = unpack_group(plan, d_in, n_time, c0, nc, su)) != cudaSuccess) return cuda_fail(e, "unpack launch");
+    for (int g = 0, c0 = 0; c0 < Cp; ++g, c0 += per) {
+      const int nc = (Cp - c0 < per) ? Cp - c0 : per;
+      const int first = c0 * plan->pack, last = (c0 + nc) * plan->pack < C ? (c0 + nc) * plan->pack : C;
+      if ((e = unpack_group(plan, d_in, n_time, first, last - first, su)) != cudaSuccess)
+        return cuda_fail(e, "unpack launch");
       cudaStream_t sx = forked ? plan->s_x[g % nxs] : s;
       if (forked) {
         if ((e = cudaEventRecord(plan->ev_unpacked[g], su)) != cudaSuccess) return cuda_fail(e, "event");
@@ -466,23 +474,41 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
                                            prop.name + " sm_" + std::to_string(prop.major * 10 + prop.minor));
 
   const int n_inputs = 2 * c.n_stations;
-  const int ni_pad = (n_inputs + 15) / 16 * 16;
+  int ni_pad = (n_inputs + 15) / 16 * 16;
   const int64_t n_pairs = n_pairs_of(n_inputs);
   const int elem_bytes = c.fmt == XCORR_IN_CI4 ? 1 : 2;
   const int ppc = c.fmt == XCORR_IN_CF32 ? 6 : 2;
   const size_t acc_bytes = (size_t)c.n_channels * (size_t)n_pairs * 8;
+  // Float input of at most 64 inputs: channels side by side in the 128 rows of a tile, which costs the same
+  // however few are used, as many as shorten the longest CTA's work; none past the last channel under a
+  // memory limit.  (16 inputs x 64 channels x 1024 samples: 57 us with a tile per channel, 28 so; 40 x
+  // 500 x 1024: 589, 290.  Always as many as fit: 16 x 16 x 256 17.3 -> 20.0, 50 x 33 x 700 32.6 -> 41.8.)
+  int pack = 1;
+  if (engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CF32 && n_inputs <= 64) {
+    const int blocks = 6 * ((c.max_time_per_exec + xc::kTcWindowBF16 - 1) / xc::kTcWindowBF16);
+    int64_t best = 0;
+    for (int k = 1; k <= 128 / ni_pad && k <= c.n_channels; k *= 2) {  // the blocks that the busiest CTA drains
+      const int64_t tiles = (c.n_channels + k - 1) / k, split = xc::tc_float_split(tiles, blocks, prop.multiProcessorCount);
+      const int64_t cost = (tiles + prop.multiProcessorCount - 1) / prop.multiProcessorCount * ((blocks + split - 1) / split);
+      if (k > 1 && (cost >= best || (c.n_channels % k && c.hbm_budget_bytes))) continue;
+      best = cost;
+      pack = k;
+    }
+  }
+  const int plane_chans = (c.n_channels + pack - 1) / pack;
+  ni_pad *= pack;
   // two or more 128-input tiles run on CTA pairs from a small ring of planes; smaller problems stage
   // all their planes
   // (int8 never needs planes)
   const bool decoded_ci8 = engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CI8;
   const bool pair = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles;
-  size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && !pair ? (size_t)c.n_channels * ppc *
+  size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && !pair ? (size_t)plane_chans * ppc *
                                                                      (size_t)c.max_time_per_exec * ni_pad * elem_bytes
                                                                : 0;
   const int exp_windows = (c.max_time_per_exec + xc::kTcWindowBF16 - 1) / xc::kTcWindowBF16;
   // (+ 256: the drain reads a tile's 128 column exponents past the last row's ni_pad)
   const size_t exps_bytes = (engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CF32)
-                                ? (size_t)c.n_channels * exp_windows * ni_pad * 2 + 256
+                                ? (size_t)plane_chans * exp_windows * ni_pad * 2 + 256
                                 : 0;
   xc::PairRing ring;
   const size_t other = acc_bytes + exps_bytes + 256;
@@ -522,6 +548,7 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   plan->num_sms = prop.multiProcessorCount;
   plan->n_inputs = n_inputs;
   plan->ni_pad = ni_pad;
+  plan->pack = pack;
   plan->n_pairs = n_pairs;
   plan->engine = engine;
   plan->max_integration = max_int;

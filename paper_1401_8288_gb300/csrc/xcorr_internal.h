@@ -85,7 +85,8 @@ struct xcorr_plan_s {
   int device = 0;
   int num_sms = 0;
   int n_inputs = 0;  // N_i
-  int ni_pad = 0;    // plane row pitch (inputs), multiple of 16
+  int ni_pad = 0;    // plane row pitch (inputs), multiple of 16: of pack channels side by side
+  int pack = 1;      // float input of at most 64 inputs: channels that share a plane row and a tile
   int64_t n_pairs = 0;
   int engine = 0;
   int64_t max_integration = 0;
@@ -192,7 +193,10 @@ struct TcLaunch {
   int elem_bytes = 1;       // 1: E4M3 planes (kind::f8f6f4), 2: BF16 planes (kind::f16)
   int variant = 0;          // stage shape, 0 .. kTcVariants - 1
   bool float_out = false;   // float accumulator (float input) or exact int32
+  // with pack > 1, "channels" here are groups of pack channels, each n_inputs / pack wide in the planes,
+  // of which true_inputs are inputs; the output's true_chans channels are single ones
   int n_time = 0, chan0 = 0, n_chan = 0, n_inputs = 0;
+  int pack = 1, true_inputs = 0, true_chans = 0;
   int planes_per_chan = 2;  // re planes then im planes: 2 (one piece) or 6 (three)
   int n_pairs_k = 1;        // plane pairs on the virtual K axis
   int pair_p[8] = {0}, pair_q[8] = {0};
@@ -205,6 +209,7 @@ struct TcLaunch {
   int num_sms = 0;
 };
 int tc_stage_samples(int elem_bytes, int variant);
+int tc_float_split(int64_t items, int n_blocks, int num_sms);
 
 // One subarray of a batch, as the batch X kernel reads it from device memory
 // (host and device share this layout; it inherits the tensor map's alignment).
@@ -346,7 +351,7 @@ cudaError_t launch_repitch(const void* in, const void* end, void* out, int row_b
 // float (re, im) samples -> six BF16 planes [c][6][t][ni_pad] of integer digits
 // (re digits 0-2, im digits 0-2) and one exponent per (channel, window, input).
 cudaError_t launch_unpack_cf32_digits(const float* in, uint16_t* planes, int16_t* exps, int n_time, int n_chan,
-                                      int c0, int nc, int n_inputs, int ni_pad, int max_time, int window,
+                                      int c0, int nc, int n_inputs, int pack, int ni_pad, int max_time, int window,
                                       int exp_windows, cudaStream_t stream);
 cudaError_t launch_fold_wide_f64(const float2* acc, double* out, int64_t n_pairs_total, bool add, cudaStream_t stream);
 

@@ -90,6 +90,9 @@ struct TcParams {
   int spw;            // stages per time window
   int n_tw;           // time windows
   int split;          // SPLIT: CTAs of a cluster, which share the blocks of one tile pair
+  // PACK: a tile is pack channels side by side, pitch rows each (input i of the tile is channel
+  // i * pitch_inv >> 16 of the group), true_inputs of them inputs; true_chans channels in the output
+  int pack, pitch, pitch_inv, true_inputs, true_chans;
   int planes_per_chan;
   int64_t n_pairs;
   int accumulate_first;  // the first block adds into out (else it stores)
@@ -166,7 +169,7 @@ __device__ __forceinline__ void block_range(const TcParams& p, int n_blocks, int
   b1 = n_blocks * (rank + 1) / n;
 }
 
-template <int ESIZE, int KT, int STAGES, bool FLOAT_OUT, bool BATCH, bool SPLIT>
+template <int ESIZE, int KT, int STAGES, bool FLOAT_OUT, bool BATCH, bool SPLIT, bool PACK>
 __global__ void __launch_bounds__(kThreads, 1)
     xcorr_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ TcParams p) {
   using G = Geometry<ESIZE, KT, STAGES>;
@@ -482,25 +485,31 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncwarp();
         const int j = col0 + ch * kChunk + col;
+        // the pair (i, j)'s place, or null
+        auto place = [&](int r) -> uint2* {
+          const int i = row0 + 4 * r + sub;
+          if (!PACK) return i < n_inputs && j <= i ? out_c + (int64_t)i * (i + 1) / 2 + j : nullptr;
+          const int blk = i * p.pitch_inv >> 16, il = i - blk * p.pitch, jl = j - blk * p.pitch;
+          const int c = v.chan * p.pack + blk;
+          return blk < p.pack && c < p.true_chans && il < p.true_inputs && jl >= 0 && jl <= il
+                     ? static_cast<uint2*>(p.out) + c * p.n_pairs + il * (il + 1) / 2 + jl
+                     : nullptr;
+        };
         uint32_t valid = 0;
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const int i = row0 + 4 * r + sub;
-          if (i < n_inputs && j <= i) valid |= 1u << r;
-        }
+        for (int r = 0; r < 8; ++r)
+          if (place(r) != nullptr) valid |= 1u << r;
         uint2 old[8];
         if (add) {  // (continuing an integration: rarer, kept out of the register budget)
 #pragma unroll 1
           for (int r = 0; r < 8; ++r) {
-            const int i = row0 + 4 * r + sub;
-            old[r] = (valid >> r) & 1u ? out_c[(int64_t)i * (i + 1) / 2 + j] : make_uint2(0u, 0u);
+            old[r] = (valid >> r) & 1u ? *place(r) : make_uint2(0u, 0u);
           }
         }
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
           if ((valid >> r) & 1u) {
             const int rr = 4 * r + sub;
-            const int i = row0 + rr;
             uint2 v = stage_rows[rr * kPitch + col];
             if (add) {
               if (FLOAT_OUT) {
@@ -511,7 +520,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 v.y += old[r].y;
               }
             }
-            out_c[(int64_t)i * (i + 1) / 2 + j] = v;
+            *place(r) = v;
           }
         }
         __syncwarp();
@@ -533,12 +542,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // One instantiation per (operand type, stage variant, output type) in use.
-template <int ESIZE, int V, bool FLOAT_OUT, bool BATCH = false, bool SPLIT = false>
+template <int ESIZE, int V, bool FLOAT_OUT, bool BATCH = false, bool SPLIT = false, bool PACK = false>
 cudaError_t launch_variant(const CUtensorMap* tmap, const TcParams& p, int grid, cudaStream_t stream) {
   constexpr int KT = stage_rows_of(V, ESIZE), S = stages_of(V);
   using G = Geometry<ESIZE, KT, S>;
   static_assert(!SPLIT || S * G::kStageBytes >= kBlk * kBlk * 8, "a CTA's part fits its stages");
-  auto kern = xcorr_tc_kernel<ESIZE, KT, S, FLOAT_OUT, BATCH, SPLIT>;
+  auto kern = xcorr_tc_kernel<ESIZE, KT, S, FLOAT_OUT, BATCH, SPLIT, PACK>;
   static int attr_device = -1;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -553,6 +562,41 @@ cudaError_t launch_variant(const CUtensorMap* tmap, const TcParams& p, int grid,
 }
 
 }  // namespace
+
+// CTAs that share the blocks of one of `items` float tiles: the most of 1, 2, 4, 8 that keep a CTA on an
+// SM of its own and whose clusters all fit the chip at once (a cluster lies within one GPC).
+int tc_float_split(int64_t items, int n_blocks, int num_sms) {
+  static int device = -1, most[4] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  if (device != dev) {
+    constexpr int V = 0;
+    using G = Geometry<2, stage_rows_of(V, 2), stages_of(V)>;
+    auto kern = xcorr_tc_kernel<2, stage_rows_of(V, 2), stages_of(V), true, false, true, false>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmemBytes) != cudaSuccess) return 1;
+    for (int k = 1; k < 4; ++k) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(8 * 512);
+      cfg.blockDim = dim3(kThreads);
+      cfg.dynamicSmemBytes = G::kSmemBytes;
+      cudaLaunchAttribute attr{};
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = 1u << k;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&most[k], kern, &cfg) != cudaSuccess) {
+        most[k] = 0;
+        cudaGetLastError();
+      }
+    }
+    device = dev;
+  }
+  int split = 1;
+  for (int k = 1; k < 4; ++k)
+    if (items << k <= num_sms && items <= most[k] && 1 << k <= n_blocks) split = 1 << k;
+  return split;
+}
 
 int tc_stage_samples(int elem_bytes, int variant) { return stage_rows_of(variant, elem_bytes); }
 
@@ -595,7 +639,13 @@ cudaError_t launch_xcorr_tc(const CUtensorMap* tmap, const TcLaunch& L, cudaStre
   p.exps = L.exps;
   p.exp_windows = L.exp_windows;
   p.ni_pad = L.ni_pad;
-  p.n_pairs = (int64_t)L.n_inputs * (L.n_inputs + 1) / 2;
+  p.pack = L.pack;
+  p.pitch = L.n_inputs / L.pack;
+  p.pitch_inv = 65536 / p.pitch + 1;  // (i < 128, pitch a multiple of 16: exact)
+  p.true_inputs = L.true_inputs;
+  p.true_chans = L.true_chans;
+  const int n_in = L.pack > 1 ? L.true_inputs : L.n_inputs;
+  p.n_pairs = (int64_t)n_in * (n_in + 1) / 2;
   p.accumulate_first = L.accumulate ? 1 : 0;
   p.out = L.out;
   p.status = L.status;
@@ -616,8 +666,12 @@ cudaError_t launch_xcorr_tc(const CUtensorMap* tmap, const TcLaunch& L, cudaStre
   if (!L.float_out) return cudaErrorInvalidValue;
   // Few tile pairs: clusters of 2, 4 or 8 CTAs share the blocks of each while that keeps every CTA on
   // an SM of its own (128 inputs x 64 channels x 1024 samples: 79 -> 54 us).
-  p.split = 1;
-  while (p.split < 8 && items * 2 * p.split <= L.num_sms && 2 * p.split <= p.n_tw * p.n_pairs_k) p.split *= 2;
+  p.split = tc_float_split(items, p.n_tw * p.n_pairs_k, L.num_sms);
+  if (L.pack > 1) {  // (one stage shape each: the tile is what costs)
+    if (nb != 1) return cudaErrorInvalidValue;
+    if (p.split > 1) return launch_variant<2, 0, true, false, true, true>(tmap, p, grid, stream);
+    return launch_variant<2, 0, true, false, false, true>(tmap, p, grid, stream);
+  }
   if (p.split > 1) {
     switch (L.variant) {
       case 0: return launch_variant<2, 0, true, false, true>(tmap, p, grid, stream);

@@ -286,7 +286,7 @@ constexpr int kTileThreads = kTileCols * kTileGroups;
 template <bool ALIGNED>
 __global__ void __launch_bounds__(kTileThreads, 2) unpack_cf32_digits_kernel(
     const float* __restrict__ in, uint16_t* __restrict__ planes, int16_t* __restrict__ exps, int n_time, int n_chan,
-    int c0, int nc, int n_inputs, int ni_pad, int64_t comp_stride, int window, int exp_windows) {
+    int c0, int nc, int n_inputs, int pack, int ni_pad, int64_t comp_stride, int window, int exp_windows) {
   extern __shared__ float4 slice[];  // [window][kTileCols]
   __shared__ uint32_t part[2][kTileGroups][kTileCols];
   __shared__ int win_e[2][kTileCols];
@@ -306,6 +306,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) unpack_cf32_digits_kernel(
     const int cc = static_cast<int>(unit / per_chan), col = static_cast<int>(unit % per_chan) * kUnitCols + q % kUnitCols;
     const bool have = unit < n_units && col < half;
     const int c = c0 + cc, i = 2 * col;
+    const int group = c / pack, at = (c - group * pack) * (ni_pad / pack) + i;  // its plane rows, its place there
     const int t0 = w * window, len = min(n_time, t0 + window) - t0;
     // the slice's rows, all of a thread's copies in flight together
     const float* src = in + (((int64_t)t0 * n_chan + c) * n_inputs + i) * 2;
@@ -343,13 +344,13 @@ __global__ void __launch_bounds__(kTileThreads, 2) unpack_cf32_digits_kernel(
       for (int gg = 0; gg < kTileGroups; ++gg) m = max(m, part[k][gg][q]);
       const int e = window_exponent(m);
       win_e[k][q] = e;
-      if (have) exps[((int64_t)c * exp_windows + w) * ni_pad + i + k] = static_cast<int16_t>(e);
+      if (have) exps[((int64_t)group * exp_windows + w) * ni_pad + at + k] = static_cast<int16_t>(e);
     }
     __syncthreads();
     float s0a, s0b, s1a, s1b;
     window_scale(win_e[0][q], s0a, s0b);
     window_scale(win_e[1][q], s1a, s1b);
-    uint32_t* base = reinterpret_cast<uint32_t*>(planes + (6 * (int64_t)c) * comp_stride + i);
+    uint32_t* base = reinterpret_cast<uint32_t*>(planes + (6 * (int64_t)group) * comp_stride + at);
     const int64_t cs = comp_stride / 2;  // in uint32 units (comp_stride is a multiple of 16)
     if (have) {
       for (int r = g; r < len; r += kTileGroups) {
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) unpack_cf32_digits_kernel(
 
 template <bool ALIGNED>
 cudaError_t launch_cf32_digits(const float* in, uint16_t* planes, int16_t* exps, int n_time, int n_chan, int c0, int nc,
-                               int n_inputs, int ni_pad, int max_time, int window, int exp_windows,
+                               int n_inputs, int pack, int ni_pad, int max_time, int window, int exp_windows,
                                cudaStream_t stream) {
   const size_t smem = (size_t)window * kTileCols * sizeof(float4);
   static int attr_device = -1;
@@ -389,16 +390,16 @@ cudaError_t launch_cf32_digits(const float* in, uint16_t* planes, int16_t* exps,
       (int64_t)((nc + chans - 1) / chans) * ((n_time + window - 1) / window) * (per_chan * chans / 2);
   const unsigned grid = static_cast<unsigned>(slices < 2LL * sms ? slices : 2LL * sms);
   return launch_dependent(unpack_cf32_digits_kernel<ALIGNED>, grid, kTileThreads, smem, stream, in, planes, exps, n_time,
-                          n_chan, c0, nc, n_inputs, ni_pad, (int64_t)max_time * ni_pad, window, exp_windows);
+                          n_chan, c0, nc, n_inputs, pack, ni_pad, (int64_t)max_time * ni_pad, window, exp_windows);
 }
 
 }  // namespace
 
 cudaError_t launch_unpack_cf32_digits(const float* in, uint16_t* planes, int16_t* exps, int n_time, int n_chan,
-                                      int c0, int nc, int n_inputs, int ni_pad, int max_time, int window,
+                                      int c0, int nc, int n_inputs, int pack, int ni_pad, int max_time, int window,
                                       int exp_windows, cudaStream_t stream) {
   return (reinterpret_cast<uintptr_t>(in) % 16 == 0 ? launch_cf32_digits<true> : launch_cf32_digits<false>)(
-      in, planes, exps, n_time, n_chan, c0, nc, n_inputs, ni_pad, max_time, window, exp_windows, stream);
+      in, planes, exps, n_time, n_chan, c0, nc, n_inputs, pack, ni_pad, max_time, window, exp_windows, stream);
 }
 
 }  // namespace xc

@@ -451,3 +451,27 @@ def test_last_wave_split_over_the_idle_sms(torch, variant, n_sta, n_chan, n_time
         got = plan.dump().cpu().numpy()
         plan.sync()
     check("ci4", got, np.concatenate([x, x[:100]]), 2 * n_sta)
+
+
+@pytest.mark.parametrize("n_sta,n_chan,n_time,offset", [(4, 500, 385, 0), (1, 700, 400, 4), (10, 301, 800, 0), (16, 333, 400, 8), (25, 200, 769, 0),
+                                                        (32, 155, 300, 12), (8, 64, 1024, 0)])
+def test_float_channels_side_by_side(torch, n_sta, n_chan, n_time, offset):
+    """Packed tiles: a last group that is not full, single and shared tiles; a store, then an adding
+    execute; a non-finite sample reaches its own channel's visibilities only."""
+    x = draw("cf32", n_time, n_chan, n_sta, seed=n_sta + n_time)
+    buf = placed(torch, x, offset)
+    stream = torch.cuda.current_stream().cuda_stream
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="cf32") as plan:
+        for _ in range(2):
+            xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, n_time, stream)
+        check("cf32", plan.dump().cpu().numpy(), np.concatenate([x, x]), 2 * n_sta)
+        c = n_chan // 2 + 1
+        bad = torch.from_numpy(x).cuda()
+        clean = plan.execute_dump(bad).cpu().numpy()
+        bad[n_time - 1, c, 0, 1, 0] = float("nan")
+        got = plan.execute_dump(bad).cpu().numpy()
+        plan.sync()
+    ii, jj = np.tril_indices(2 * n_sta)
+    hit = np.zeros(got.shape[:2], dtype=bool)
+    hit[c] = (ii == 1) | (jj == 1)
+    assert np.isnan(got[hit]).all() and np.array_equal(got[~hit], clean[~hit])

@@ -72,7 +72,7 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kStashCol = 256;                       // 128 columns of corrected Im after the accumulator
 constexpr uint32_t kAcol0 = 384;                          // then the A stages
 constexpr int kStagingBytes = kBlk * kBlk * 4;            // Re accumulator bits of a whole tile pair
-constexpr int kRowcBytes = kBlk * 8;                      // per-row correction constants
+constexpr int kRowcBytes = 2 * kBlk * 8;                  // per-row correction constants, [item parity][row]
 constexpr int kSumsBytes = 2 * kBlk * 8 + 2 * kBlk * 4;   // columns: [item parity][input] (8P, 8Q); Re, Im code sums
 // Every partial sum of u_a u_b is n 2^-18 with 0 <= n <= 450 T (and |n| <= 225 T for Im).
 // For T <= kMagicSamples, |n| < 2^22 and n + 1.5 2^23 is exact in FP32, so one FFMA
@@ -251,7 +251,9 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
   uint8_t* raw = smem;
   uint8_t* bpl = smem + G::kOffBpl;
   uint32_t* staging = reinterpret_cast<uint32_t*>(smem + G::kOffStaging);  // Re [row][16-byte chunk ^ swz(row)]
-  int2* rowc = reinterpret_cast<int2*>(smem + G::kOffRowc);                 // [row]
+  // [item parity][row]: with eight epilogue warps the one that writes a row's entry is not the only one
+  // that reads it, and the other may still be at the previous item
+  int2* rowc = reinterpret_cast<int2*>(smem + G::kOffRowc);
   int2* sums = reinterpret_cast<int2*>(smem + G::kOffSums);
   int* code_sums = reinterpret_cast<int*>(smem + G::kOffSums + 2 * kBlk * 8);  // [Re, Im][column]
   uint4* dump = reinterpret_cast<uint4*>(smem + G::kOffDump);
@@ -619,8 +621,8 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
         if (lane == 0) mbar_arrive(sempty);
         // Re = n_re - 8 P_a - 8 P_b + 128 T,  Im = -n_im - 8 Q_a + 8 Q_b with P = S_re + S_im, Q = S_im -
         // S_re: the row's part
-        rowc[r_own] = make_int2(t128 - 8 * (row_re + row_im) - (magic ? kMagicBits : 0),
-                                -8 * (row_im - row_re) + (magic ? kMagicBits : 0));
+        rowc[(g & 1) * kBlk + r_own] = make_int2(t128 - 8 * (row_re + row_im) - (magic ? kMagicBits : 0),
+                                                -8 * (row_im - row_re) + (magic ? kMagicBits : 0));
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           s[q] += __shfl_xor_sync(0xFFFFFFFFu, s[q], 8);
@@ -656,7 +658,7 @@ __global__ void __launch_bounds__(Roles<EPI>::kThreads, 1)
         row_out[m] = nullptr;
         firstm[m] = 0;
         lastm[m] = I == J ? rr : kBlk - 1;  // last column of the row in the tile
-        rcm[m] = rowc[rr];
+        rcm[m] = rowc[(g & 1) * kBlk + rr];
         if (packed) {
           const int blk = rr / it.pitch, cr = c * it.pack_g + blk;
           const int i = rr - blk * it.pitch;

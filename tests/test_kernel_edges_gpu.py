@@ -475,3 +475,22 @@ def test_float_channels_side_by_side(torch, n_sta, n_chan, n_time, offset):
     hit = np.zeros(got.shape[:2], dtype=bool)
     hit[c] = (ii == 1) | (jj == 1)
     assert np.isnan(got[hit]).all() and np.array_equal(got[~hit], clean[~hit])
+
+
+@pytest.mark.parametrize("n_sta,n_chan,n_time", [(64, 1500, 1), (72, 700, 40), (100, 500, 128), (136, 120, 300)])
+def test_eight_epilogue_warps_item_after_item(torch, n_sta, n_chan, n_time):
+    """Many short items a CTA whose row corrections differ as far as codes allow (every input at another
+    level, another one in the next channel), storing and adding: a row's correction is read by two
+    warps, of which one may be an item behind."""
+    rng = np.random.default_rng(n_sta)
+    level = rng.integers(0, 256, size=(1, n_chan, n_sta, 2), dtype=np.uint8)
+    x = np.broadcast_to(level, (n_time, n_chan, n_sta, 2)).copy()
+    xd = torch.from_numpy(x).cuda()
+    want = oracle.correlate(oracle.FMT_CI4, x)
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="ci4", engine="tensor") as plan:
+        plan.set_tuning(4, 0, 2, 0)
+        for _ in range(5):
+            for _ in range(3):
+                plan.execute(xd)
+            assert np.array_equal(plan.dump().cpu().numpy().astype(np.int64), 3 * want)
+        plan.sync()

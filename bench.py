@@ -77,7 +77,7 @@ KERNEL_SOURCES = {
     "xcorr_tc_kernel": ("xcorr_tc.cu", "sm103_ptx.cuh", "xcorr_internal.h"),
     "xcorr_tc_raw_pair_kernel": ("xcorr_tc_raw_pair.cu", "pair_common.cuh", "fused_pairing.h", "sm103_ptx.cuh",
                                  "xcorr_internal.h"),
-    "xcorr_tc_pair_kernel": ("pair_common.cuh","xcorr_tc_pair.cu", "unpack_device.cuh", "ci4_decode.cuh", "fused_pairing.h",
+    "xcorr_tc_pair_kernel": ("xcorr_tc_pair.cu", "pair_common.cuh", "ring_order.h", "unpack_device.cuh", "ci4_decode.cuh", "fused_pairing.h",
                              "sm103_ptx.cuh", "xcorr_internal.h"),
 }
 FUSED_TA_VARIANTS = (4, 5, 6, 10)  # tuning stage_variants served by the tensor-memory-A fused kernel

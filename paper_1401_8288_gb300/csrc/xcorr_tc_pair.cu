@@ -72,6 +72,7 @@
 #include <type_traits>
 
 #include "pair_common.cuh"
+#include "ring_order.h"
 #include "unpack_device.cuh"
 #include "xcorr_internal.h"
 
@@ -140,13 +141,10 @@ __device__ __forceinline__ int digit_q(int pk) { return (0x102010 >> (4 * pk)) &
 
 struct P2Params {
   int n_chan, n_inputs, n_time;
-  int nb, n_entries;     // tiles per side; pair entries per channel
-  int n_items;           // entries of the launch
+  int nb;                // tiles per side
+  ring::Order order;
   int n_kt;              // stages along time
-  int chunk, n_chunks;   // samples per ring chunk (a multiple of the stage), chunks along time
-  int batch_chans;       // channel places of a batch in the unpack order
-  int n_batches;
-  int slots;             // ring slots
+  int chunk;             // samples per ring chunk (a multiple of the stage)
   int subs;              // unpack sub-tasks per chunk
   int halves;            // 64-input halves: two per tile
   int64_t slot_bytes;
@@ -168,20 +166,6 @@ struct P2Params {
   int16_t* exps;         // float input: window exponents [C][exp_windows][exp_pitch]
   int exp_windows, exp_pitch;
 };
-
-// Place of (batch, chunk, channel of the batch) in the unpack order.
-__device__ __forceinline__ int place_of(const P2Params& p, int batch, int chunk, int j) {
-  return (batch * p.n_chunks + chunk) * p.batch_chans + j;
-}
-
-// CTAs that read the chunk at place u: two per entry of its channel in its batch.
-__device__ __forceinline__ int readers_of(const P2Params& p, int u, int n_cl) {
-  const int j = u % p.batch_chans, batch = u / (p.batch_chans * p.n_chunks);
-  const int i0 = batch * n_cl, i1 = min(i0 + n_cl, p.n_items);
-  const int c = i0 / p.n_entries + j;
-  const int a = max(i0, c * p.n_entries), b = min(i1, (c + 1) * p.n_entries);
-  return b > a ? 2 * (b - a) : 0;
-}
 
 __device__ __forceinline__ int flag_load(const int* f) {
   int v;
@@ -239,30 +223,31 @@ struct Task {
   int chan, k;         // channel, chunk along time
   const uint8_t* src;  // its first sample, the channel's first input
   int live;            // samples before n_time
-  int done, readers;   // the slot's previous chunk: readers finished (as last seen), readers in all
+  int prev;            // the place that had the slot before, or -1
+  int done, readers;   // its readers: finished (as last seen), in all
 };
 
 // Bring x.u, x.sub to the first sub-task at or after them that has any reader; false at the end.
 template <int FMT>
-__device__ __forceinline__ bool task_seek(const P2Params& p, Task& x, int n_cl, int n_warps, int n_places) {
+__device__ __forceinline__ bool task_seek(const P2Params& p, Task& x, int n_warps, int n_places) {
   for (;; x.sub += n_warps) {
     x.u += x.sub / p.subs;
     x.sub %= p.subs;
     if (x.u >= n_places) return false;
-    if (readers_of(p, x.u, n_cl) > 0) break;
+    if (ring::readers_of(p.order, x.u) > 0) break;
   }
-  const int j = x.u % p.batch_chans, bk = x.u / p.batch_chans;
-  const int batch = bk / p.n_chunks;
-  x.k = bk - batch * p.n_chunks;
-  x.chan = (batch * n_cl) / p.n_entries + j;
+  const int j = x.u % p.order.batch_chans, bk = x.u / p.order.batch_chans;
+  const int batch = bk / p.order.n_chunks;
+  x.k = bk - batch * p.order.n_chunks;
+  x.chan = ring::first_chan(p.order, batch) + j;
   const int t = x.k * p.chunk + (FMT == XCORR_IN_CF32 ? 0 : x.sub / p.col_splits * kRowsPerTask);
   x.src = p.in + ((int64_t)t * p.n_chan + x.chan) * p.row_bytes;
   x.live = p.n_time - t;
   x.done = x.readers = 0;
-  if (x.u >= p.slots) {  // looked up when the sub-task's first copies start, used when they have arrived
-    const int prev = x.u - p.slots;
-    x.readers = readers_of(p, prev, n_cl);
-    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(x.done) : "l"(p.done + prev) : "memory");
+  x.prev = ring::slot_user(p.order, x.u);
+  if (x.prev >= 0) {  // looked up when the sub-task's first copies start, used when they have arrived
+    x.readers = ring::readers_of(p.order, x.prev);
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(x.done) : "l"(p.done + x.prev) : "memory");
   }
   return true;
 }
@@ -338,11 +323,11 @@ __device__ __forceinline__ uint4 fetched(const P2Params& p, const Task& c, int r
 // The unpack warps: raw samples stream through shared memory by asynchronous copies that run three
 // groups ahead (24 KB per SM in flight) across sub-tasks, so that HBM's latency is not waited for.
 template <int FMT, bool VEC>
-__device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, int uw, int lane, int n_cl,
+__device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, int uw, int lane,
                                             volatile int* abort_flag) {
   using G = Geom<FMT>;
   constexpr bool FLOAT = FMT == XCORR_IN_CF32;
-  const int n_places = p.n_batches * p.n_chunks * p.batch_chans;
+  const int n_places = ring::places(p.order);
   const int n_warps = static_cast<int>(gridDim.x) * kUnpackWarps;
   const int n_groups = FLOAT ? 2 * (p.chunk / kFetchRows) : kHalfPerTask * (kRowsPerTask / kFetchRows);
   uint4* buf = reinterpret_cast<uint4*>(fetch) + uw * (kFetchGroups * 128) + lane;
@@ -352,7 +337,7 @@ __device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, i
   // has more groups than are in flight)
   Task f{};
   f.sub = static_cast<int>(blockIdx.x) * kUnpackWarps + uw;
-  bool more = task_seek<FMT>(p, f, n_cl, n_warps, n_places);
+  bool more = task_seek<FMT>(p, f, n_warps, n_places);
   int fg = 0, cg = 0;  // their next groups
   Task c = f;
   bool run = more;
@@ -362,7 +347,7 @@ __device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, i
     if (++fg == n_groups) {
       fg = 0;
       f.sub += n_warps;
-      more = task_seek<FMT>(p, f, n_cl, n_warps, n_places);
+      more = task_seek<FMT>(p, f, n_warps, n_places);
     }
   };
 #pragma unroll
@@ -379,11 +364,11 @@ __device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, i
       if (c.done < c.readers) {  // the slot's previous chunk is still being read
         bool ok = true;
         if (lane == 0)
-          ok = flag_wait(p.done + c.u - p.slots, c.readers, abort_flag, p.status, DEV_TIMEOUT_EMPTY);
+          ok = flag_wait(p.done + c.prev, c.readers, abort_flag, p.status, DEV_TIMEOUT_EMPTY);
         if (!__all_sync(0xFFFFFFFFu, ok)) break;
       }
       asm volatile("fence.proxy.async;" ::: "memory");  // the slot's TMA reads before these writes
-      slot = p.ring + (int64_t)(c.u % p.slots) * p.slot_bytes;
+      slot = p.ring + (int64_t)(c.u % p.order.slots) * p.slot_bytes;
       m0 = m1 = 0u;
     }
     int row, col;
@@ -513,7 +498,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync();  // both CTAs' barriers and tensor memory exist before either touches the other's
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  const int n_items = p.n_items;
+  const int n_items = p.order.n_items, n_entries = p.order.n_entries;
   const int cl = static_cast<int>(blockIdx.x >> 1), n_cl = static_cast<int>(gridDim.x >> 1);
   const int n_tw = (p.n_kt + G::kSpw - 1) / G::kSpw;
   const int n_blocks = n_tw * G::kPairsK;  // drained blocks per item: (window, plane pair)
@@ -532,7 +517,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     int g = 0;
     bool ok = true;
     for (int q = cl; ok && q < n_items; q += n_cl) {
-      const Item it = item_of(p.nb, p.n_entries, q, rank);
+      const Item it = item_of(p.nb, n_entries, q, rank);
       uint2* out_c = static_cast<uint2*>(p.out) + (int64_t)it.chan * p.n_pairs;
       const int row0 = it.R * kBlk + quarter * 32;  // first global row of this warp
       const int col0 = it.S * kBlk + colh * kHalf;  // first global column of this warp
@@ -674,17 +659,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         int pend = -1, pend_n = 0;  // a chunk read but not yet reported, and the stage count at its end
         bool ok = true;
         for (int q = cl, batch = 0; ok && q < n_items; q += n_cl, ++batch) {
-          const Item it = item_of(p.nb, p.n_entries, q, rank);
-          const int j = it.chan - (batch * n_cl) / p.n_entries;
+          const Item it = item_of(p.nb, n_entries, q, rank);
+          const int j = it.chan - ring::first_chan(p.order, batch);
           const uint32_t bytes = (it.has_row ? 4 * G::kPlane : 0) + 2 * G::kPlane;
-          for (int k = 0; ok && k < p.n_chunks; ++k) {
-            const int u = place_of(p, batch, k, j);
+          for (int k = 0; ok && k < p.order.n_chunks; ++k) {
+            const int u = ring::place_of(p.order, batch, k, j);
             if (!flag_wait(p.ready + u, p.subs, abort_flag, p.status, DEV_TIMEOUT_FULL)) {  // it has been unpacked
               ok = false;
               break;
             }
             asm volatile("fence.proxy.async;" ::: "memory");  // generic writes, read by the copies
-            const uint8_t* sl = p.ring + (int64_t)(u % p.slots) * p.slot_bytes;
+            const uint8_t* sl = p.ring + (int64_t)(u % p.order.slots) * p.slot_bytes;
             const int n_st = min(spc, p.n_kt - k * spc);
             for (int pk = 0; ok && pk < G::kPairsK; ++pk) {
               const uint8_t* a = sl + plane_at<FMT>(p, 0, FLOAT_OUT ? digit_p(pk) : 0, 2 * it.R);
@@ -829,9 +814,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (p.vec)
-      unpack_role<FMT, true>(p, smem + G::kOffFetch, warp - kUnpackWarp0, lane, n_cl, abort_flag);
+      unpack_role<FMT, true>(p, smem + G::kOffFetch, warp - kUnpackWarp0, lane, abort_flag);
     else
-      unpack_role<FMT, false>(p, smem + G::kOffFetch, warp - kUnpackWarp0, lane, n_cl, abort_flag);
+      unpack_role<FMT, false>(p, smem + G::kOffFetch, warp - kUnpackWarp0, lane, abort_flag);
   }
 
   tc_fence_before();
@@ -927,10 +912,9 @@ cudaError_t pair_ring_layout(int fmt, int n_inputs, int n_chan, int max_time, si
   const int t_rows = (max_time + rows - 1) / rows * rows;
   r->chunk = t_rows < most_chunk ? t_rows : most_chunk;
   const int64_t chunks = (max_time + r->chunk - 1) / r->chunk;
-  int bc = (r->clusters - 1) / ne + 2;
-  r->batch_chans = bc < n_chan ? bc : n_chan;
-  const int64_t batches = (items + r->clusters - 1) / r->clusters;
-  const int64_t places = batches * chunks * r->batch_chans;
+  const ring::Order one = ring::make_order(n_chan, ne, r->clusters, 1, 1);  // (of one chunk along time)
+  r->batch_chans = one.batch_chans;
+  const int64_t places = chunks * ring::places(one);
   if (places > 0x7FFFFFFF / 4096) return cudaErrorInvalidValue;
   r->places = static_cast<int>(places);
   r->slot_bytes = (size_t)planes * r->chunk * r->halves * kHalf * elem;
@@ -956,14 +940,9 @@ cudaError_t launch_xcorr_tc_pair(const PairLaunch& L, cudaStream_t stream) {
   p.n_inputs = L.n_inputs;
   p.n_time = L.n_time;
   p.nb = (L.n_inputs + kBlk - 1) / kBlk;
-  p.n_entries = pair_entries(p.nb);
-  p.n_items = L.n_chan * p.n_entries;
+  p.order = ring::make_order(L.n_chan, pair_entries(p.nb), r.clusters, (L.n_time + r.chunk - 1) / r.chunk, r.slots);
   p.n_kt = (L.n_time + rows - 1) / rows;
   p.chunk = r.chunk;
-  p.n_chunks = (L.n_time + r.chunk - 1) / r.chunk;
-  p.batch_chans = r.batch_chans;
-  p.n_batches = (p.n_items + r.clusters - 1) / r.clusters;
-  p.slots = r.slots;
   p.halves = r.halves;
   p.slot_bytes = static_cast<int64_t>(r.slot_bytes);
   p.row_bytes = L.n_inputs * in_bytes;
@@ -975,7 +954,7 @@ cudaError_t launch_xcorr_tc_pair(const PairLaunch& L, cudaStream_t stream) {
   p.ready = L.flags;
   p.done = L.flags + r.places;
   p.leavers = L.flags + 2 * r.places;
-  p.n_flags = p.n_batches * p.n_chunks * p.batch_chans;
+  p.n_flags = ring::places(p.order);
   if (p.n_flags > r.places) return cudaErrorInvalidValue;
   p.reuse = p.n_flags > r.slots ? 1 : 0;
   p.vec = (int64_t)L.n_inputs * in_bytes % 16 == 0 && reinterpret_cast<uintptr_t>(L.in) % 16 == 0;

@@ -1,6 +1,6 @@
 // ring_order.h -- the order of the CTA-pair kernel's ring of planes
-// (xcorr_tc_pair.cu): which places there are, who reads them and which one had a
-// slot before.  Plain integer arithmetic for the device and the host, so that
+// (xcorr_tc_pair.cu): which places there are, who reads them, when a reader reports
+// and which place had a slot before.  Plain integer arithmetic for the device and the host, so that
 // every size can be checked without a GPU.
 //
 // An entry is a pair of tile pairs of one channel, an item an entry of the launch
@@ -71,6 +71,29 @@ XC_RING_FN int slot_user(const Order& o, int u) {
   while (v >= 0 && readers_of(o, v) == 0) v -= o.slots;
   return v >= 0 ? v : -1;
 }
+
+// When a CTA reports a chunk as read: once its copies have landed.  They are not waited for while
+// there is work: the chunk is reported when its last stage's buffer comes round again, or at the next
+// chunk's end.  But before the CTA waits for a chunk that is not unpacked yet it reports (and waits for
+// the copies, which land by themselves): that unpack may be waiting for this very slot.
+// So a report waits only for what is in flight, the unpack of a place only for reports of earlier
+// places, and a reader only for the unpack of the place it is at: any ring of one slot or more ends.
+struct Reads {
+  int place = -1;  // read and not reported, or -1
+  int end = 0;     // stages loaded at its end
+  int stages = 0;  // stages loaded
+  XC_RING_FN bool due_before_wait(bool unpacked) const { return place >= 0 && !unpacked; }
+  XC_RING_FN bool due_after_stage(int stage_buffers) {
+    ++stages;
+    return place >= 0 && stages >= end + stage_buffers;
+  }
+  XC_RING_FN bool due_after_chunk() const { return place >= 0; }
+  XC_RING_FN void reported() { place = -1; }
+  XC_RING_FN void chunk_read(int u) {
+    place = u;
+    end = stages;
+  }
+};
 
 }  // namespace ring
 }  // namespace xc

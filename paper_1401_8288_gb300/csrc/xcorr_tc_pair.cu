@@ -44,9 +44,11 @@
 // all clusters walk a batch of consecutive channels together.  The unpack
 // follows that order: (batch, time chunk, channel of the batch).  A chunk's
 // slot is ready when its sub-tasks have added up in ready[u]; it may be
-// refilled once every CTA that reads it has added to done[u].  Both waits are
-// on work earlier in the order, and the launch is cooperative (every CTA is
-// resident), so they always end; like all waits here they are bounded
+// refilled once every CTA that reads it has added to done[u].  An unpack waits
+// for the reports of earlier places only, a reader reports what it has read
+// before it waits for an unpack, and the launch is cooperative (every CTA is
+// resident), so both waits always end, with a ring of any length (ring_order.h;
+// tests/test_ring_order.py plays it); like all waits here they are bounded
 // (sm103_ptx.cuh).  The last CTA to leave clears the flags.
 //
 // Measured (one GB300), against unpack + planes kernel: 512 inputs x 256 channels x 4096 samples, float
@@ -655,8 +657,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int64_t stage_step = plane_at<FMT>(p, 1, 0, 0);
         int s = 0;
         uint32_t ph = 0, filled = 0, fill_parity = 0;  // bit s: the stage was filled, and with which parity
-        int n = 0;                  // stages acquired
-        int pend = -1, pend_n = 0;  // a chunk read but not yet reported, and the stage count at its end
+        ring::Reads reads;  // (kept only while slots are reused)
+        // tell the unpack warps that a chunk is read; landed: its copies are known to have landed
+        auto report = [&](bool landed) {
+          const int ps = (reads.end - 1) % kStages;
+          if (!landed && !mbar_wait(&full[ps], (fill_parity >> ps) & 1u, abort_flag, p.status, DEV_TIMEOUT_FULL))
+            return false;
+          flag_add_relaxed(p.done + reads.place);
+          reads.reported();
+          return true;
+        };
         bool ok = true;
         for (int q = cl, batch = 0; ok && q < n_items; q += n_cl, ++batch) {
           const Item it = item_of(p.nb, n_entries, q, rank);
@@ -664,9 +674,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           const uint32_t bytes = (it.has_row ? 4 * G::kPlane : 0) + 2 * G::kPlane;
           for (int k = 0; ok && k < p.order.n_chunks; ++k) {
             const int u = ring::place_of(p.order, batch, k, j);
-            if (!flag_wait(p.ready + u, p.subs, abort_flag, p.status, DEV_TIMEOUT_FULL)) {  // it has been unpacked
-              ok = false;
-              break;
+            if (flag_load(p.ready + u) < p.subs) {  // it has not been unpacked
+              if ((reads.due_before_wait(false) && !report(false)) ||
+                  !flag_wait(p.ready + u, p.subs, abort_flag, p.status, DEV_TIMEOUT_FULL)) {
+                ok = false;
+                break;
+              }
             }
             asm volatile("fence.proxy.async;" ::: "memory");  // generic writes, read by the copies
             const uint8_t* sl = p.ring + (int64_t)(u % p.order.slots) * p.slot_bytes;
@@ -689,24 +702,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                   s = 0;
                   ph ^= 1u;
                 }
-                ++n;
-                if (pend >= 0 && n >= pend_n + kStages) {  // its last stage's slot has come round
-                  flag_add_relaxed(p.done + pend);
-                  pend = -1;
-                }
+                if (reads.due_after_stage(kStages)) report(true);  // its last stage's buffer has come round
               }
             }
             if (ok && p.reuse) {
-              if (pend >= 0) {  // a chunk shorter than the stage ring: wait for the copies themselves
-                const int ps = (pend_n - 1) % kStages;
-                if (!mbar_wait(&full[ps], (fill_parity >> ps) & 1u, abort_flag, p.status, DEV_TIMEOUT_FULL)) {
-                  ok = false;
-                  break;
-                }
-                flag_add_relaxed(p.done + pend);
+              if (reads.due_after_chunk() && !report(false)) {  // a chunk shorter than the stage ring
+                ok = false;
+                break;
               }
-              pend = u;
-              pend_n = n;
+              reads.chunk_read(u);
             }
           }
         }
@@ -714,7 +718,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         volatile int never = 0;
         for (int k = 0; k < kStages; ++k)
           if (filled & (1u << k)) mbar_wait(&full[k], (fill_parity >> k) & 1u, &never, p.status, DEV_TIMEOUT_DRAIN);
-        if (pend >= 0) flag_add_relaxed(p.done + pend);
+        if (reads.due_after_chunk()) report(true);
       }
     } else if (warp >= kNegWarp0) {
       // -B_re: the real half-tile with the sign bits flipped, at the same swizzled offsets

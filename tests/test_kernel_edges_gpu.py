@@ -494,3 +494,30 @@ def test_eight_epilogue_warps_item_after_item(torch, n_sta, n_chan, n_time):
                 plan.execute(xd)
             assert np.array_equal(plan.dump().cpu().numpy().astype(np.int64), 3 * want)
         plan.sync()
+
+
+def least_budget(n_sta, n_chan, n_time, fmt):
+    """The smallest memory limit that a plan is made with, from the error of one that is too small."""
+    with pytest.raises(RuntimeError, match="plan needs") as err:
+        xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor", hbm_budget_bytes=1)
+    return int(str(err.value).split("plan needs ")[1].split()[0])
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time", [("cf32", 129, 60, 800), ("cf32", 256, 33, 500), ("cf32", 150, 90, 385), ("ci4", 129, 200, 600),
+                                                     ("ci4", 256, 70, 1100)])
+@pytest.mark.parametrize("more", [0, 3])
+def test_pair_ring_kernel_at_its_least_ring(torch, fmt, n_sta, n_chan, n_time, more):
+    """A ring cut to one step of a batch by the memory limit (and to a little more): many batches, each
+    slot refilled again and again; a store, then an adding execute."""
+    budget = least_budget(n_sta, n_chan, n_time, fmt)
+    chunk = 384 * 6 * 2 if fmt == "cf32" else 512 * 2
+    x = draw(fmt, n_time, n_chan, n_sta, seed=n_sta)
+    xd = torch.from_numpy(x).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor",
+                    hbm_budget_bytes=budget + more * chunk * 256 * ((2 * n_sta + 255) // 256)) as plan:
+        plan.set_tuning(0, 0, 1, 1)
+        for _ in range(2):
+            plan.execute(xd)
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check(fmt, got, np.concatenate([x, x]), 2 * n_sta)

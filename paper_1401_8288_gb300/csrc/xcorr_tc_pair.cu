@@ -363,7 +363,8 @@ __device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, i
   float s0a = 0.f, s0b = 0.f, s1a = 0.f, s1b = 0.f;
   while (run) {
     if (cg == 0) {
-      if (c.done < c.readers) {  // the slot's previous chunk is still being read
+      // the slot's previous chunk is still being read (every lane looked for itself, at its own time)
+      if (__any_sync(0xFFFFFFFFu, c.done < c.readers)) {
         bool ok = true;
         if (lane == 0)
           ok = flag_wait(p.done + c.prev, c.readers, abort_flag, p.status, DEV_TIMEOUT_EMPTY);
@@ -447,6 +448,7 @@ __device__ __forceinline__ void unpack_role(const P2Params& p, uint8_t* fetch, i
       asm volatile("fence.proxy.async.global;" ::: "memory");
       __syncwarp();
       if (lane == 0) flag_add(p.ready + c.u);
+      __syncwarp();
       run = f.u < n_places;  // the next sub-task, if there is one: its first copies are in flight
       c = f;
       cg = 0;

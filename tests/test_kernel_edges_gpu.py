@@ -521,3 +521,16 @@ def test_pair_ring_kernel_at_its_least_ring(torch, fmt, n_sta, n_chan, n_time, m
         got = plan.dump().cpu().numpy()
         plan.sync()
     check(fmt, got, np.concatenate([x, x]), 2 * n_sta)
+
+
+def test_pair_ring_kernel_waits_alike_in_every_run(torch):
+    """Unpack warps that find their slot still read, or just read, in every batch: the same bits each
+    time, and a plan that reports no failure."""
+    n_sta, n_chan, n_time = 140, 120, 385
+    x = torch.from_numpy(draw("cf32", n_time, n_chan, n_sta, seed=3)).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="cf32", hbm_budget_bytes=least_budget(n_sta, n_chan, n_time, "cf32")) as plan:
+        first = plan.execute_dump(x)
+        for _ in range(30):
+            assert torch.equal(plan.execute_dump(x), first)
+        plan.sync()
+    check("cf32", first.cpu().numpy(), x.cpu().numpy(), 2 * n_sta)

@@ -79,6 +79,8 @@ __global__ void __launch_bounds__(256) clear_kernel(uint2* __restrict__ out, int
 }  // namespace
 
 cudaError_t launch_clear(void* out, int64_t pairs, cudaStream_t stream) {
+  // (the adding launch behind it takes any output of aligned integers)
+  if (reinterpret_cast<uintptr_t>(out) % sizeof(uint2)) return cudaMemsetAsync(out, 0, pairs * sizeof(uint2), stream);
   int64_t blocks = (pairs + 511) / 512;
   if (blocks > 4096) blocks = 4096;
   return launch_dependent(clear_kernel, static_cast<unsigned>(blocks), 256, 0, stream, static_cast<uint2*>(out), pairs);

@@ -534,3 +534,20 @@ def test_pair_ring_kernel_waits_alike_in_every_run(torch):
             assert torch.equal(plan.execute_dump(x), first)
         plan.sync()
     check("cf32", first.cpu().numpy(), x.cpu().numpy(), 2 * n_sta)
+
+
+@pytest.mark.parametrize("n_sta,n_chan,n_time", [(8, 16, 256), (32, 64, 1024), (29, 5, 700)])
+def test_split_launches_into_an_output_off_its_pairs(torch, n_sta, n_chan, n_time):
+    """Launches whose every tile is split in time clear the output and add 4-byte integers: an output that
+    is aligned to those only is as good as any."""
+    x = draw("ci4", n_time, n_chan, n_sta, seed=n_time)
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="ci4", engine="tensor") as plan:
+        plan.set_tuning(10, 0, 2, 0)
+        n = n_chan * plan.info["n_pairs"] * 2
+        buf = torch.full((n + 2,), -9, dtype=torch.int32, device="cuda")
+        for _ in range(2):
+            plan.execute_dump(torch.from_numpy(x).cuda(), buf[1:n + 1])
+        plan.sync()
+    got = buf.cpu().numpy()
+    assert got[0] == -9 and got[-1] == -9
+    check("ci4", got[1:-1].reshape(n_chan, -1, 2), x, 2 * n_sta)

@@ -110,8 +110,8 @@ typedef struct xcorr_plan_s *xcorr_plan;
 /* Launch shape of the tensor-core path (xcorr_plan_set_tuning, xcorr_autotune). */
 typedef struct {
     int stage_variant;  /* shared-memory ring, 0 .. 10: planes path of up to 128 inputs 0 = 3 x 64 KB,
-                           1 (and 3 .. 10) = 4 x 48 KB, 2 = 6 x 32 KB stages (more inputs, and
-                           int8: launches on CTA pairs with one shape); fused path see `unfused` */
+                           1 (and 3 .. 10) = 4 x 48 KB, 2 = 6 x 32 KB stages (more inputs, and int8
+                           decoded on chip: launches on CTA pairs with one shape); fused path see `unfused` */
     int groups;         /* channel groups whose unpack overlaps the X kernel; 0 = automatic (<= 8) */
     int x_streams;      /* 1 or 2 streams the groups' X launches alternate over                 */
     int unfused;        /* 4-bit input: 0 = unpack on chip inside the X kernel where possible

@@ -128,6 +128,36 @@ bool raw_ci8_applies(xcorr_plan plan, const void* d_in) {
   return plan->cfg.fmt == XCORR_IN_CI8 && plan->engine == XCORR_ENGINE_TENSOR && xc::raw_pair_takes(plan->n_inputs, d_in);
 }
 
+// Whether int8 input is decoded on chip (xcorr_tc_raw_pair.cu) or goes through planes in memory
+// (xcorr_unpack.cu and xcorr_tc.cu), by the time of an execute: a set-up, rounds of the persistent kernel
+// (so many us, and so many a sample), the MB that the unpack or the padding copy moves, and the MB of
+// visibilities.  On chip a CTA pair takes an entry of a channel, and with one tile its second CTA has no
+// rows; from planes every SM takes a tile and a step is shorter, but the planes are written and read.
+// The figures are least squares over 1500 sizes (2 to 1024 inputs, 1 to 512 channels, 32 to 4096 samples;
+// within 17 % of the times of all but 4 % of them); the margin of 5 % goes to the planes, whose time varies
+// less.  us, planes / on chip: 16 inputs x 152 channels x 4096 samples 58 / 103, 64 x 512 x 1024 90 / 97, 128 x
+// 64 x 1024 29 / 23, 128 x 4 x 4096 51 / 58, 136 x 48 x 256 17 / 21, 256 x 152 x 4096 310 / 214, 62 x 304 x 1024
+// 110 / 68.
+bool ci8_from_planes(int n_inputs, int n_chan, int n_time, int num_sms, bool aligned) {
+  const int nb = (n_inputs + 127) / 128;
+  const double t = n_time, mb = 1e-6 * n_chan * t, out = 4e-6 * n_chan * n_inputs * (n_inputs + 1.0);
+  const int64_t tiles = (int64_t)n_chan * nb * (nb + 1) / 2, entries = (int64_t)n_chan * xc::raw_pair_items(nb);
+  const double rt = static_cast<double>((tiles + num_sms - 1) / num_sms);
+  const double re = static_cast<double>((entries + num_sms / 2 - 1) / (num_sms / 2));
+  const int padded = (n_inputs + 15) / 16 * 16;
+  const double planes = aligned ? 7.9 + rt * (3.3 + 0.0087 * t) + 0.183 * 6 * padded * mb + 0.10 * out
+                                : 7.7 + rt * (3.8 + 0.0092 * t) + 0.632 * 6 * n_inputs * mb + 0.13 * out;  // by elements
+  const double chip = aligned ? 8.7 + re * (2.3 + 0.0106 * t) + 0.19 * out
+                              : 9.8 + re * (2.3 + 0.0106 * t) + 0.116 * 4 * n_inputs * mb + 0.27 * out;  // with the copy
+  return planes < 1.05 * chip;
+}
+
+// An execute of a plan that has the planes still takes the faster route for its own samples and address.
+bool staged_execute(xcorr_plan plan, const void* d_in, int n_time) {
+  return plan->staged_ci8 && ci8_from_planes(plan->n_inputs, plan->cfg.n_channels, n_time, plan->num_sms,
+                                             xc::raw_pair_takes(plan->n_inputs, d_in));
+}
+
 // Input that would be decoded on chip but for its rows' or its address's alignment is copied piece by
 // piece to padded rows in the plan's planes memory and correlated from there (xcorr_repitch.cu).
 // A piece: `nc` channels x `nt` samples.
@@ -216,6 +246,9 @@ cudaError_t unpack_group(xcorr_plan plan, const void* d_in, int n_time, int c0, 
     case XCORR_IN_CI4:
       return xc::launch_unpack_ci4_e4m3_channels(static_cast<const uint8_t*>(d_in), static_cast<uint8_t*>(plan->planes),
                                                  n_time, C, c0, nc, N, plan->ni_pad, T, plan->num_sms, s);
+    case XCORR_IN_CI8:
+      return xc::launch_unpack_ci8_bf16(static_cast<const int8_t*>(d_in), static_cast<uint16_t*>(plan->planes), n_time,
+                                        C, c0, nc, N, plan->ni_pad, T, plan->num_sms, s);
     default:
       return xc::launch_unpack_cf32_digits(static_cast<const float*>(d_in), static_cast<uint16_t*>(plan->planes),
                                            plan->exps, n_time, C, c0, nc, N, plan->pack, plan->ni_pad, T, plan->window_samples,
@@ -250,6 +283,7 @@ int host_groups(int C, size_t bytes, int* edge) {
 xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* target, bool target_fresh,
                          cudaStream_t s) {
   const int C = plan->cfg.n_channels, N = plan->n_inputs;
+  const bool staged_ci8 = staged_execute(plan, d_in, n_time);
   cudaError_t e;
   cudaEvent_t* ev = nullptr;
   if (plan->prof_cap) {
@@ -266,7 +300,7 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     if (e != cudaSuccess) return cuda_fail(e, "fused X kernel launch");
     if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
     if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
-  } else if (raw_ci8_applies(plan, d_in)) {
+  } else if (!staged_ci8 && raw_ci8_applies(plan, d_in)) {
     // int8 input decoded on chip: one launch on the caller's stream
     if (ev && ((e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventRecord(ev[2], s)) != cudaSuccess))
       return cuda_fail(e, "profile event");
@@ -275,7 +309,7 @@ xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* ta
     if (e != cudaSuccess) return cuda_fail(e, "CTA-pair X kernel launch");
     if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return cuda_fail(e, "profile event");
     if (ev) plan->prof_ngroups[plan->prof_count % plan->prof_cap] = 1;
-  } else if (const Pieces pieces = repitch_pieces(plan, n_time); pieces.pitch) {
+  } else if (const Pieces pieces = staged_ci8 ? Pieces{} : repitch_pieces(plan, n_time); pieces.pitch) {
     // the same kernels over padded rows, piece by piece on the caller's stream
     if (ev && ((e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventRecord(ev[2], s)) != cudaSuccess))
       return cuda_fail(e, "profile event");
@@ -499,12 +533,13 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   ni_pad *= pack;
   // two or more 128-input tiles run on CTA pairs from a small ring of planes; smaller problems stage
   // all their planes
-  // (int8 never needs planes)
-  const bool decoded_ci8 = engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CI8;
-  const bool pair = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles;
-  size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && !pair ? (size_t)plane_chans * ppc *
-                                                                     (size_t)c.max_time_per_exec * ni_pad * elem_bytes
-                                                               : 0;
+  const size_t all_planes = (size_t)plane_chans * ppc * (size_t)c.max_time_per_exec * ni_pad * elem_bytes;
+  const bool staged_ci8 = engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CI8 &&
+                          ci8_from_planes(n_inputs, c.n_channels, c.max_time_per_exec, prop.multiProcessorCount, n_inputs % 8 == 0) &&
+                          (!c.hbm_budget_bytes || acc_bytes + all_planes + 256 <= c.hbm_budget_bytes);
+  const bool decoded_ci8 = engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CI8 && !staged_ci8;
+  const bool pair = engine == XCORR_ENGINE_TENSOR && c.fmt != XCORR_IN_CI8 && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles;
+  size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && !pair ? all_planes : 0;
   const int exp_windows = (c.max_time_per_exec + xc::kTcWindowBF16 - 1) / xc::kTcWindowBF16;
   // (+ 256: the drain reads a tile's 128 column exponents past the last row's ni_pad)
   const size_t exps_bytes = (engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CF32)
@@ -549,6 +584,7 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   plan->n_inputs = n_inputs;
   plan->ni_pad = ni_pad;
   plan->pack = pack;
+  plan->staged_ci8 = staged_ci8;
   plan->n_pairs = n_pairs;
   plan->engine = engine;
   plan->max_integration = max_int;
@@ -856,8 +892,8 @@ xcorr_status xcorr_plan_query(xcorr_plan plan, xcorr_plan_info* info) {
   const bool fused = plan->engine == XCORR_ENGINE_TENSOR && plan->cfg.fmt == XCORR_IN_CI4 && !plan->tune_unfused &&
                      plan->n_inputs % 16 == 0;
   // (int8: a 16-byte aligned input, nullptr standing for one)
-  const bool one_launch = plan->pair || raw_ci8_applies(plan, nullptr);
-  const Pieces pieces = fused || raw_ci8_applies(plan, nullptr) ? Pieces{} : repitch_pieces(plan, plan->cfg.max_time_per_exec);
+  const bool raw = !plan->staged_ci8 && raw_ci8_applies(plan, nullptr), one_launch = plan->pair || raw;
+  const Pieces pieces = fused || raw || plan->staged_ci8 ? Pieces{} : repitch_pieces(plan, plan->cfg.max_time_per_exec);
   info->kernels_per_execute = fused ? xc::fused_launches(plan->cfg.max_time_per_exec)
                               : pieces.pitch ? pieces.count * (1 + (plan->cfg.fmt == XCORR_IN_CI4 ? xc::fused_launches(pieces.nt) : 1))
                               : one_launch                          ? 1
@@ -923,7 +959,7 @@ xcorr_status xcorr_autotune(xcorr_plan plan, const void* d_in, int n_time, void*
         if (uf == 0 && (gi > 0 || xs > 1)) continue;      // the fused kernel is one launch
         if (uf == 0 && padded_ci4 && padded_shape(v) != v - 4 && v != xc::kSmallFusedVariant) continue;
         // the CTA-pair kernels have one shape each
-        if (uf == 1 && (plan->pair || plan->cfg.fmt == XCORR_IN_CI8) && (v > 0 || gi > 0)) continue;
+        if (uf == 1 && (plan->pair || (plan->cfg.fmt == XCORR_IN_CI8 && !plan->staged_ci8)) && (v > 0 || gi > 0)) continue;
         plan->tune_variant = v;
         plan->tune_groups = group_choices[gi];
         plan->tune_x_streams = xs;

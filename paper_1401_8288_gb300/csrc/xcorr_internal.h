@@ -86,6 +86,7 @@ struct xcorr_plan_s {
   int num_sms = 0;
   int n_inputs = 0;  // N_i
   int ni_pad = 0;    // plane row pitch (inputs), multiple of 16: of pack channels side by side
+  bool staged_ci8 = false;  // int8 input: the plan has planes of all channels (else everything is decoded on chip)
   int pack = 1;      // float input of at most 64 inputs: channels that share a plane row and a tile
   int64_t n_pairs = 0;
   int engine = 0;
@@ -348,6 +349,10 @@ cudaError_t launch_xcorr_tc_raw_pair(const int8_t* in, int row_chans, int n_time
 cudaError_t launch_repitch(const void* in, const void* end, void* out, int row_bytes, int row_chans, int n_chan,
                            int n_time, int num_sms, cudaStream_t stream);
 
+// int8 (re, im) samples -> two BF16 planes [c][2][t][ni_pad] (exact).
+cudaError_t launch_unpack_ci8_bf16(const int8_t* in, uint16_t* planes, int n_time, int n_chan, int c0,
+                                   int nc, int n_inputs, int ni_pad, int max_time, int num_sms,
+                                   cudaStream_t stream);
 // float (re, im) samples -> six BF16 planes [c][6][t][ni_pad] of integer digits
 // (re digits 0-2, im digits 0-2) and one exponent per (channel, window, input).
 cudaError_t launch_unpack_cf32_digits(const float* in, uint16_t* planes, int16_t* exps, int n_time, int n_chan,

@@ -663,7 +663,13 @@ cudaError_t launch_xcorr_tc(const CUtensorMap* tmap, const TcLaunch& L, cudaStre
       default: return launch_variant<1, 2, false>(tmap, p, grid, stream);
     }
   }
-  if (!L.float_out) return cudaErrorInvalidValue;
+  if (!L.float_out) {
+    switch (L.variant) {
+      case 0: return launch_variant<2, 0, false>(tmap, p, grid, stream);
+      case 1: return launch_variant<2, 1, false>(tmap, p, grid, stream);
+      default: return launch_variant<2, 2, false>(tmap, p, grid, stream);
+    }
+  }
   // Few tile pairs: clusters of 2, 4 or 8 CTAs share the blocks of each while that keeps every CTA on
   // an SM of its own (128 inputs x 64 channels x 1024 samples: 79 -> 54 us).
   p.split = tc_float_split(items, p.n_tw * p.n_pairs_k, L.num_sms);

@@ -16,9 +16,10 @@
 // measured 415-420.  Planes from L2 (xcorr_tc_pair.cu) stop at 12 KB per step and
 // SM and have to be written first: 480.  One GB300, against unpack + planes kernel
 // (us): 512 inputs x 256 channels x 4096 samples 870 (1310), 256 x 256 x 1024 116
-// (159), 128 x 300 x 1024 66 (87), 128 x 64 x 1024 23 (34), 16 x 64 x 1024 21 (26):
-// faster at every size tried, also where one tile leaves half of each pair's rows
-// idle, since there is no unpack launch and no plane in HBM.
+// (159), 128 x 300 x 1024 66 (83), 128 x 64 x 1024 23 (29): no unpack launch, no plane
+// in memory.  With one tile half of every pair's rows are idle and only half as
+// many channels run side by side, so few inputs on many channels go through planes
+// (64 x 152 x 4096 105 here, 97 so; ci8_from_planes in xcorr_api.cu has the rule).
 //
 // Layout.  Everything is cut into half-tiles of 64 inputs, 4 KB of raw samples a
 // stage of 32 samples.  TMA lands a raw half-tile with the 128-byte swizzle of

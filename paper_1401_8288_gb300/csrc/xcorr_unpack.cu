@@ -8,7 +8,7 @@
 // X kernel multiplies the true integers.  The planes stay input-contiguous:
 // the X kernel reads them as MN-major operands, so the tensor memory access
 // itself performs the transpose of the corner turn and this kernel is a pure
-// element-wise decode with 128-bit loads and stores.
+// element-wise decode with 128-bit loads and stores.  int8 and float input: below.
 #include <cudaTypedefs.h>
 
 #include <cstring>
@@ -263,6 +263,91 @@ bool encode_raw_ci4_packed_tmap(CUtensorMap* map, const void* in, int n_inputs, 
   }
   raw_memo_put(*map, in, n_inputs, n_chan, row_chans, n_time, box_t, 128, 1);
   return true;
+}
+
+// ------------------------------------------------------ int8 input --
+namespace {
+
+__device__ __forceinline__ uint32_t bf16_bits(float f) {
+  return static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(f)));
+}
+
+// Eight int8 samples (16 bytes: re, im interleaved) -> eight BF16 real parts
+// and eight imaginary parts, exact (|v| <= 128 needs 8 significant bits).
+// Idx as for unpack_ci4_e4m3_vec.
+template <typename Idx>
+__global__ void __launch_bounds__(256) unpack_ci8_bf16_vec(const int8_t* __restrict__ in,
+                                                           uint16_t* __restrict__ planes, int64_t n_rows,
+                                                           int n_chan, int c0, int nc, int q_per_row,
+                                                           int ni_pad, int64_t comp_stride) {
+  const Idx total = static_cast<Idx>(n_rows * q_per_row);
+  for (Idx q = blockIdx.x * static_cast<Idx>(blockDim.x) + threadIdx.x; q < total;
+       q += static_cast<Idx>(gridDim.x) * blockDim.x) {
+    const Idx row = q / static_cast<Idx>(q_per_row);
+    const int k = static_cast<int>(q - row * q_per_row);
+    const int64_t t = static_cast<int64_t>(row / static_cast<Idx>(nc));
+    const int c = c0 + static_cast<int>(row - static_cast<Idx>(t) * nc);
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(in + ((t * n_chan + c) * q_per_row + k) * 16));
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t re[4], im[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {  // word h holds samples 2h, 2h + 1: re0 im0 re1 im1
+      const float r0 = static_cast<float>(static_cast<int8_t>(w[h] & 0xFF));
+      const float i0 = static_cast<float>(static_cast<int8_t>((w[h] >> 8) & 0xFF));
+      const float r1 = static_cast<float>(static_cast<int8_t>((w[h] >> 16) & 0xFF));
+      const float i1 = static_cast<float>(static_cast<int8_t>(w[h] >> 24));
+      re[h] = bf16_bits(r0) | (bf16_bits(r1) << 16);
+      im[h] = bf16_bits(i0) | (bf16_bits(i1) << 16);
+    }
+    uint16_t* dst = planes + (2 * (int64_t)c) * comp_stride + t * ni_pad + 8 * (int64_t)k;
+    *reinterpret_cast<uint4*>(dst) = make_uint4(re[0], re[1], re[2], re[3]);
+    *reinterpret_cast<uint4*>(dst + comp_stride) = make_uint4(im[0], im[1], im[2], im[3]);
+  }
+}
+
+__global__ void __launch_bounds__(256) unpack_ci8_bf16_elem(const int8_t* __restrict__ in,
+                                                            uint16_t* __restrict__ planes, int64_t n_rows,
+                                                            int n_chan, int c0, int nc, int n_inputs,
+                                                            int ni_pad, int64_t comp_stride) {
+  const int64_t total = n_rows * n_inputs;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total;
+       q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = q / n_inputs;
+    const int i = static_cast<int>(q - row * n_inputs);
+    const int64_t t = row / nc;
+    const int c = c0 + static_cast<int>(row - t * nc);
+    const int64_t s = (t * n_chan + c) * n_inputs + i;
+    uint16_t* dst = planes + (2 * (int64_t)c) * comp_stride + t * ni_pad + i;
+    dst[0] = static_cast<uint16_t>(bf16_bits(static_cast<float>(in[2 * s])));
+    dst[comp_stride] = static_cast<uint16_t>(bf16_bits(static_cast<float>(in[2 * s + 1])));
+  }
+}
+
+int64_t grid_for(int64_t work, int num_sms) {
+  int64_t blocks = (work + 255) / 256;
+  const int64_t cap = (int64_t)num_sms * 16;
+  if (blocks > cap) blocks = cap;
+  return blocks < 1 ? 1 : blocks;
+}
+
+}  // namespace
+
+cudaError_t launch_unpack_ci8_bf16(const int8_t* in, uint16_t* planes, int n_time, int n_chan, int c0, int nc,
+                                   int n_inputs, int ni_pad, int max_time, int num_sms, cudaStream_t stream) {
+  const int64_t n_rows = (int64_t)n_time * nc;
+  const int64_t comp_stride = (int64_t)max_time * ni_pad;
+  const bool vec = (n_inputs % 8 == 0) && (reinterpret_cast<uintptr_t>(in) % 16 == 0);
+  const int64_t work = n_rows * (n_inputs / 8), blocks = grid_for(work, num_sms);
+  if (vec && work + blocks * 256 < (INT64_C(1) << 32))
+    unpack_ci8_bf16_vec<uint32_t><<<(unsigned)blocks, 256, 0, stream>>>(in, planes, n_rows, n_chan, c0, nc,
+                                                                       n_inputs / 8, ni_pad, comp_stride);
+  else if (vec)
+    unpack_ci8_bf16_vec<int64_t><<<(unsigned)blocks, 256, 0, stream>>>(in, planes, n_rows, n_chan, c0, nc,
+                                                                      n_inputs / 8, ni_pad, comp_stride);
+  else
+    unpack_ci8_bf16_elem<<<(unsigned)grid_for(n_rows * n_inputs, num_sms), 256, 0, stream>>>(
+        in, planes, n_rows, n_chan, c0, nc, n_inputs, ni_pad, comp_stride);
+  return cudaGetLastError();
 }
 
 // ----------------------------------------------------- float input --

@@ -551,3 +551,42 @@ def test_split_launches_into_an_output_off_its_pairs(torch, n_sta, n_chan, n_tim
     got = buf.cpu().numpy()
     assert got[0] == -9 and got[-1] == -9
     check("ci4", got[1:-1].reshape(n_chan, -1, 2), x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("n_sta,n_chan,n_time,planes", [(8, 152, 4096, True), (9, 78, 1014, True), (4, 395, 2567, True), (32, 512, 1024, True),
+                                                        (64, 4, 4096, True), (68, 48, 256, True), (64, 64, 1024, False),
+                                                        (128, 152, 1024, False), (31, 304, 1024, False)])
+def test_int8_route(torch, n_sta, n_chan, n_time, planes):
+    """int8 plans decode on chip or go through planes, whichever is faster at their size: an unpack and
+    an X launch a group, or one launch (two where rows are padded)."""
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="ci8", engine="tensor") as plan:
+        info = plan.query()
+    assert info["kernels_per_execute"] == (2 * info["tuning"]["groups"] if planes else 1 if n_sta % 4 == 0 else 2)
+
+
+@pytest.mark.parametrize("n_sta,n_chan,n_time,offset", [(1, 152, 257, 0), (5, 100, 400, 2), (8, 160, 383, 0), (8, 160, 384, 1), (12, 305, 129, 0),
+                                                        (32, 153, 769, 0), (33, 80, 385, 16), (64, 3, 1500, 0), (65, 48, 200, 0), (66, 49, 33, 8)])
+def test_int8_through_planes(torch, n_sta, n_chan, n_time, offset):
+    """Windows, stages and 16-byte units that do not end evenly, all-(-128) samples among them; a store,
+    an adding execute of a few samples (by whichever route), then a graph's replay and host memory."""
+    x = draw("ci8", n_time, n_chan, n_sta, seed=n_sta + n_time)
+    x[:, n_chan // 2] = -128
+    buf = placed(torch, x, offset)
+    stream = torch.cuda.current_stream().cuda_stream
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="ci8", engine="tensor") as plan:
+        for variant, groups in ((0, 0), (1, 3), (2, 8)):
+            plan.set_tuning(variant, groups, 2, 0)
+            xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, n_time, stream)
+            xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, 30, stream)
+            check("ci8", plan.dump().cpu().numpy(), np.concatenate([x, x[:30]]), 2 * n_sta)
+        out = torch.empty((n_chan, plan.info["n_pairs"], 2), dtype=torch.int32, device="cuda")
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            xcorr.xcorr_execute_dump(plan.handle, buf.data_ptr() + offset, n_time, out.data_ptr(), True,
+                                     xcorr.XCORR_DUMP_RESET, torch.cuda.current_stream().cuda_stream)
+        out.fill_(7)
+        graph.replay()
+        check("ci8", out.cpu().numpy(), x, 2 * n_sta)
+        host = plan.execute_dump_host(torch.from_numpy(x).pin_memory())
+        plan.sync()
+        check("ci8", host.numpy(), x, 2 * n_sta)

@@ -606,9 +606,9 @@ def our_arm(args) -> int:
     fused_ta = fused and tuning["stage_variant"] in FUSED_TA_VARIANTS
     fused_pair = fused and tuning["stage_variant"] in FUSED_PAIR_VARIANTS
     x_kernel = (("xcorr_tc_fused_pair_kernel" if fused_pair else "xcorr_tc_fused_ta_kernel" if fused_ta
-                 else "xcorr_tc_fused_kernel") if fused else "xcorr_tc_raw_pair_kernel" if fmt == "ci8"
-                else "xcorr_tc_pair_kernel" if n_sta > 64 else "xcorr_tc_kernel")
-    one_launch = fused or fmt == "ci8" or n_sta > 64  # else unpack + X per channel group
+                 else "xcorr_tc_fused_kernel") if fused else "xcorr_tc_kernel" if launches_per_step > 1
+                else "xcorr_tc_raw_pair_kernel" if fmt == "ci8" else "xcorr_tc_pair_kernel")
+    one_launch = fused or launches_per_step == 1  # else unpack + X per channel group
     x_launches = launches_per_step if one_launch else launches_per_step // 2
     out_dtype = torch.float32 if fmt == "cf32" else torch.int32
     out = torch.empty((n_chan, n_pairs, 2), dtype=out_dtype, device=dev)

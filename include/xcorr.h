@@ -109,9 +109,9 @@ typedef struct xcorr_plan_s *xcorr_plan;
 
 /* Launch shape of the tensor-core path (xcorr_plan_set_tuning, xcorr_autotune). */
 typedef struct {
-    int stage_variant;  /* shared-memory ring, 0 .. 10: planes path of up to 128 inputs 0 = 3 x 64 KB,
-                           1 (and 3 .. 10) = 4 x 48 KB, 2 = 6 x 32 KB stages (more inputs, and int8
-                           decoded on chip: launches on CTA pairs with one shape); fused path see `unfused` */
+    int stage_variant;  /* shared-memory ring, 0 .. 10: planes path 0 = 3 x 64 KB, 1 (and 3 .. 10) =
+                           4 x 48 KB, 2 = 6 x 32 KB stages (the ring of planes, and int8 decoded on
+                           chip: launches on CTA pairs with one shape); fused path see `unfused` */
     int groups;         /* channel groups whose unpack overlaps the X kernel; 0 = automatic (<= 8) */
     int x_streams;      /* 1 or 2 streams the groups' X launches alternate over                 */
     int unfused;        /* 4-bit input: 0 = unpack on chip inside the X kernel where possible
@@ -131,8 +131,8 @@ typedef struct {
                            side in one 128-row tile; and when a launch has fewer tiles
                            than SMs, each tile's stages split over several CTAs whose
                            sums are added atomically into the (cleared) output;
-                           1 = always through E4M3 planes (in HBM up to 128 inputs; a ring of
-                           them that stays in L2 beyond)                                    */
+                           1 = always through E4M3 planes (of all channels, or where they would
+                           take too much memory or time a ring of them, beyond 128 inputs)  */
 } xcorr_tuning;
 
 /* Opaque to the caller except through these fields (xcorr_plan_query). */

@@ -152,6 +152,33 @@ bool ci8_from_planes(int n_inputs, int n_chan, int n_time, int num_sms, bool ali
   return planes < 1.05 * chip;
 }
 
+// Whether two or more tiles a side of float input, or of 4-bit input that is not decoded on chip, go
+// through planes in memory rather than through the ring (xcorr_tc_pair.cu), by the same kind of model.  The
+// ring's single launch starts on clusters one at a time and unpacks on the CTAs that it runs, so it wins
+// where the rounds are long and many: float, us, planes / ring (1800 sizes; the route so chosen costs 30 % less
+// than the ring alone on average): 256 inputs x 16 channels x 256 samples 27 / 44, 256 x 16 x 1024 64 / 106, 512 x 64
+// x 1024 439 / 414, 192 x 64 x 4096 670 / 591, 130 x 100 x 10000 2530 / 2010, 512 x 256 x 4096 7200 / 5800.
+// 4-bit: where rows are whole 16-byte units the planes take less time at 158 of 170 sizes (256 x 200 x 1024
+// 64 / 124); off them they are unpacked byte by byte (338 x 200 x 4096 1226 / 506, 130 x 32 x 1024 33 / 36).
+bool planes_beat_ring(int fmt, int n_inputs, int n_chan, int n_time, int num_sms) {
+  const int nb = (n_inputs + 127) / 128;
+  const double t = n_time, mb = 1e-6 * n_chan * t, out = 4e-6 * n_chan * n_inputs * (n_inputs + 1.0);
+  const int64_t tiles = (int64_t)n_chan * nb * (nb + 1) / 2, entries = (int64_t)n_chan * xc::raw_pair_items(nb);
+  const double rt = static_cast<double>((tiles + num_sms - 1) / num_sms);
+  const double re = static_cast<double>((entries + num_sms / 2 - 1) / (num_sms / 2));
+  if (fmt == XCORR_IN_CI4) {
+    if (n_inputs % 16 == 0) return true;
+    return 7.6 + rt * (4.6 + 0.0056 * t) + 1.196 * 3 * n_inputs * mb + 0.064 * out < 17.8 + re * (3.9 + 0.014 * t) + 0.033 * out;
+  }
+  const int blocks = 6 * ((n_time + xc::kTcWindowBF16 - 1) / xc::kTcWindowBF16);  // drained one by one, shared by a cluster
+  const int split = xc::tc_float_split(tiles, blocks, num_sms);
+  const double steps = 6 * t * ((blocks + split - 1) / split) / blocks;
+  const int units = (n_inputs + 15) / 16;  // of the unpack, which takes longer over an odd number of them
+  const double planes = 11 + rt * (6.2 + 0.0091 * steps) + (units % 2 ? 0.394 : 0.194) * 20 * 16 * units * mb + 0.006 * out;
+  const double ring = 20 + re * (3.1 + 0.01165 * 6 * t) + 0.054 * 12 * 128 * nb * mb + 0.27 * out;
+  return 1.03 * planes < ring;
+}
+
 // An execute of a plan that has the planes still takes the faster route for its own samples and address.
 bool staged_execute(xcorr_plan plan, const void* d_in, int n_time) {
   return plan->staged_ci8 && ci8_from_planes(plan->n_inputs, plan->cfg.n_channels, n_time, plan->num_sms,
@@ -531,20 +558,25 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   }
   const int plane_chans = (c.n_channels + pack - 1) / pack;
   ni_pad *= pack;
-  // two or more 128-input tiles run on CTA pairs from a small ring of planes; smaller problems stage
-  // all their planes
-  const size_t all_planes = (size_t)plane_chans * ppc * (size_t)c.max_time_per_exec * ni_pad * elem_bytes;
-  const bool staged_ci8 = engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CI8 &&
-                          ci8_from_planes(n_inputs, c.n_channels, c.max_time_per_exec, prop.multiProcessorCount, n_inputs % 8 == 0) &&
-                          (!c.hbm_budget_bytes || acc_bytes + all_planes + 256 <= c.hbm_budget_bytes);
-  const bool decoded_ci8 = engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CI8 && !staged_ci8;
-  const bool pair = engine == XCORR_ENGINE_TENSOR && c.fmt != XCORR_IN_CI8 && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles;
-  size_t planes_bytes = engine == XCORR_ENGINE_TENSOR && !decoded_ci8 && !pair ? all_planes : 0;
   const int exp_windows = (c.max_time_per_exec + xc::kTcWindowBF16 - 1) / xc::kTcWindowBF16;
   // (+ 256: the drain reads a tile's 128 column exponents past the last row's ni_pad)
   const size_t exps_bytes = (engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CF32)
                                 ? (size_t)plane_chans * exp_windows * ni_pad * 2 + 256
                                 : 0;
+  const size_t all_planes = (size_t)plane_chans * ppc * (size_t)c.max_time_per_exec * ni_pad * elem_bytes;
+  // Where the operands come from.  int8: decoded on chip, or planes of all channels.  Two or more 128-input
+  // tiles a side of the others: a small ring of planes, or all of them; one tile: all of them.  (4-bit
+  // input that is decoded on chip never touches its planes: they take no more memory than padded rows
+  // may.)  All planes take at most the caller's limit, or a quarter of the memory where there is none.
+  const bool tensor = engine == XCORR_ENGINE_TENSOR;
+  const bool planes_fit = acc_bytes + all_planes + exps_bytes + 256 <= (c.hbm_budget_bytes ? c.hbm_budget_bytes : prop.totalGlobalMem / 4);
+  const bool staged_ci8 = tensor && c.fmt == XCORR_IN_CI8 && planes_fit &&
+                          ci8_from_planes(n_inputs, c.n_channels, c.max_time_per_exec, prop.multiProcessorCount, n_inputs % 8 == 0);
+  const bool decoded_ci8 = tensor && c.fmt == XCORR_IN_CI8 && !staged_ci8;
+  const bool pair = tensor && c.fmt != XCORR_IN_CI8 && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles &&
+                    !(planes_fit && (c.fmt == XCORR_IN_CF32 || all_planes <= kPieceBytes) &&
+                      planes_beat_ring(c.fmt, n_inputs, c.n_channels, c.max_time_per_exec, prop.multiProcessorCount));
+  size_t planes_bytes = tensor && !decoded_ci8 && !pair ? all_planes : 0;
   xc::PairRing ring;
   const size_t other = acc_bytes + exps_bytes + 256;
   const size_t room = c.hbm_budget_bytes > other ? c.hbm_budget_bytes - other : 1;

@@ -7,7 +7,8 @@
 // Sec. 1, Sec. 2.1, Eq. 1; the unpack and corner turn of Sec. 2.4): 4-bit
 // samples as E4M3 planes, float as six BF16 planes of integer digits with one
 // exponent per (channel, 384-sample window, input).
-// For problems of two or more 128-input tiles.
+// For problems of two or more 128-input tiles that keep every cluster at work for
+// long (planes_beat_ring in xcorr_api.cu has the rule).
 //
 // Why one launch.  Unpacking to planes in HBM writes 2 (4-bit) or 12 (float)
 // bytes per sample that the X kernel reads back: as much time as the
@@ -56,10 +57,10 @@
 // 256 channels x 2048, float, 1.22 ms (1.40), 250 x 300 x 2048, 4-bit, 355 us (670).
 // A step takes 272 cycles with the MMAs alone, 307-318 from a ring that nobody refills (about 40
 // bytes per cycle and SM from L2, the rate every form of these loads stopped at), 450-470 beside the
-// unpack, which alone would take 250-330.  The rule: two or more tiles.  With one tile half of every
+// unpack, which alone would take 250-330.  With one tile half of every
 // pair's rows are idle, and the planes kernel wins once there are channels for every SM (128 inputs x
 // 300 channels x 4096, float: 1.11 ms against 1.29 here).  4-bit input comes here when planes are asked
-// for, or under a memory limit too tight for padded rows: otherwise it stays with the fused kernel (492
+// for and all of them would be too much, or under a memory limit too tight for padded rows: otherwise it stays with the fused kernel (492
 // us against about 600 here at 512 inputs x 512 channels x 2048 samples: its L2 traffic is the raw
 // bytes), over padded rows where its own are not aligned (70 against 119 us at 338 x 97 x 1500).  int8
 // input goes to xcorr_tc_raw_pair.cu (0.87 ms against 1.00 with BF16 planes here).

@@ -590,3 +590,33 @@ def test_int8_through_planes(torch, n_sta, n_chan, n_time, offset):
         host = plan.execute_dump_host(torch.from_numpy(x).pin_memory())
         plan.sync()
         check("ci8", host.numpy(), x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time,ring", [("cf32", 128, 16, 256, False), ("cf32", 128, 16, 1024, False), ("cf32", 65, 8, 4096, False),
+                                                          ("cf32", 256, 64, 2048, True), ("cf32", 256, 256, 1024, True), ("ci4", 128, 100, 1024, False),
+                                                          ("ci4", 169, 97, 1500, True), ("ci4", 65, 16, 256, False)])
+def test_route_of_two_or_more_tiles(torch, fmt, n_sta, n_chan, n_time, ring):
+    """The ring's one launch, or an unpack and an X launch a group through all planes."""
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor") as plan:
+        plan.set_tuning(0, 0, 2, 1)
+        info = plan.query()
+    assert info["kernels_per_execute"] == (1 if ring else 2 * info["tuning"]["groups"])
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time,offset", [("cf32", 65, 90, 800, 0), ("cf32", 75, 100, 1100, 4), ("cf32", 169, 60, 900, 0),
+                                                            ("cf32", 331, 30, 800, 8), ("cf32", 200, 70, 1153, 0), ("ci4", 65, 200, 1100, 0),
+                                                            ("ci4", 169, 120, 1600, 3), ("ci4", 136, 160, 1300, 0), ("ci4", 260, 80, 1031, 8)])
+def test_ring_where_all_planes_do_not_fit(torch, fmt, n_sta, n_chan, n_time, offset):
+    """The ring under a limit that all planes pass: odd tile counts, inputs that end inside a tile, rows
+    and addresses off 16 bytes, a last chunk that is not full; a store, then a shorter adding execute."""
+    x = draw(fmt, n_time, n_chan, n_sta, seed=n_sta)
+    buf = placed(torch, x, offset)
+    stream = torch.cuda.current_stream().cuda_stream
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor", hbm_budget_bytes=least_budget(n_sta, n_chan, n_time, fmt) + (1 << 20)) as plan:
+        plan.set_tuning(0, 0, 2, 1)
+        assert plan.query()["kernels_per_execute"] == 1
+        xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, n_time, stream)
+        xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, n_time - 77, stream)
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check(fmt, got, np.concatenate([x, x[:n_time - 77]]), 2 * n_sta)

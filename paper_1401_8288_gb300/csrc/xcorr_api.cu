@@ -573,7 +573,7 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   const bool staged_ci8 = tensor && c.fmt == XCORR_IN_CI8 && planes_fit &&
                           ci8_from_planes(n_inputs, c.n_channels, c.max_time_per_exec, prop.multiProcessorCount, n_inputs % 8 == 0);
   const bool decoded_ci8 = tensor && c.fmt == XCORR_IN_CI8 && !staged_ci8;
-  const bool pair = tensor && c.fmt != XCORR_IN_CI8 && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles &&
+  bool pair = tensor && c.fmt != XCORR_IN_CI8 && (n_inputs + 127) / 128 >= xc::kTcPairMinTiles &&
                     !(planes_fit && (c.fmt == XCORR_IN_CF32 || all_planes <= kPieceBytes) &&
                       planes_beat_ring(c.fmt, n_inputs, c.n_channels, c.max_time_per_exec, prop.multiProcessorCount));
   size_t planes_bytes = tensor && !decoded_ci8 && !pair ? all_planes : 0;
@@ -594,9 +594,10 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   }
   if (pair) {
     e = xc::pair_ring_layout(c.fmt, n_inputs, c.n_channels, c.max_time_per_exec, c.hbm_budget_bytes ? room : 0, &ring);
-    if (e != cudaSuccess) return cuda_fail(e, "ring layout");
-    planes_bytes = ring.bytes;
-    if (c.fmt == XCORR_IN_CI4 && row_bytes % 16 != 0) {
+    if (e != cudaSuccess && e != cudaErrorNotSupported) return cuda_fail(e, "ring layout");
+    if (e == cudaErrorNotSupported) pair = false, ring = xc::PairRing{};
+    planes_bytes = pair ? ring.bytes : all_planes;
+    if (pair && c.fmt == XCORR_IN_CI4 && row_bytes % 16 != 0) {
       const size_t left = room > ring.flag_bytes ? room - ring.flag_bytes : 0;
       if (c.hbm_budget_bytes && piece > left) piece = left;
       if (piece > planes_bytes) planes_bytes = piece;

@@ -239,7 +239,8 @@ cudaError_t launch_xcorr_tc_batch(const void* subs, const uint4* items, int n_it
                                   int num_sms, cudaStream_t stream);
 cudaError_t launch_xcorr_tc(const CUtensorMap* tmap, const TcLaunch& launch, cudaStream_t stream);
 
-// The ring for executes of up to max_time samples, within most_bytes (0: no limit) where possible.
+// The ring for executes of up to max_time samples, within most_bytes (0: no limit) where possible;
+// cudaErrorNotSupported for more places than a launch can count.
 cudaError_t pair_ring_layout(int fmt, int n_inputs, int n_chan, int max_time, size_t most_bytes, PairRing* ring);
 struct PairLaunch {
   int fmt = 0;

@@ -103,6 +103,7 @@ constexpr int kFetchRows = 16;     // samples per group: 4 copies of 16 bytes pe
 constexpr int kFetchSlots = kUnpackWarps * 32 * 4 * kFetchGroups;
 constexpr int kFetchBytes = kFetchSlots * 16 + kFetchSlots / 8 * 4;
 constexpr int kBarrierBytes = 512;
+constexpr int64_t kRingPlaces = int64_t(1) << 24;   // of a launch: 134 MB of flags, far inside an int
 constexpr int kSinkSlots = kNegWarps + kEpiWarps;  // one per signalling warp of the odd CTA
 
 // FMT: XCORR_IN_CI4 / CF32
@@ -913,7 +914,7 @@ cudaError_t pair_ring_layout(int fmt, int n_inputs, int n_chan, int max_time, si
   const int most_chunk = fmt == XCORR_IN_CI4 ? Geom<XCORR_IN_CI4>::kMaxChunk : Geom<XCORR_IN_CF32>::kMaxChunk;
   const int nb = (n_inputs + kBlk - 1) / kBlk, ne = pair_entries(nb);
   const int64_t items = (int64_t)n_chan * ne;
-  if (items > 0x7FFFFFFF / 2) return cudaErrorInvalidValue;
+  if (items > 0x7FFFFFFF / 2) return cudaErrorNotSupported;
   r->clusters = static_cast<int>(items < n_cl ? items : n_cl);
   r->halves = 2 * nb;
   const int t_rows = (max_time + rows - 1) / rows * rows;
@@ -922,7 +923,7 @@ cudaError_t pair_ring_layout(int fmt, int n_inputs, int n_chan, int max_time, si
   const ring::Order one = ring::make_order(n_chan, ne, r->clusters, 1, 1);  // (of one chunk along time)
   r->batch_chans = one.batch_chans;
   const int64_t places = chunks * ring::places(one);
-  if (places > 0x7FFFFFFF / 4096) return cudaErrorInvalidValue;
+  if (places > kRingPlaces) return cudaErrorNotSupported;
   r->places = static_cast<int>(places);
   r->slot_bytes = (size_t)planes * r->chunk * r->halves * kHalf * elem;
   // at least three batch-wide steps of chunks, and as many as fit kRingBytes (L2 holds them)

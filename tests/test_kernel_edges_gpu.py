@@ -620,3 +620,23 @@ def test_ring_where_all_planes_do_not_fit(torch, fmt, n_sta, n_chan, n_time, off
         got = plan.dump().cpu().numpy()
         plan.sync()
     check(fmt, got, np.concatenate([x, x[:n_time - 77]]), 2 * n_sta)
+
+
+@pytest.mark.parametrize("n_sta,n_chan,max_time", [(72, 16, 16777215), (128, 1024, 300000)])
+def test_plans_of_very_long_executes(torch, n_sta, n_chan, max_time):
+    """4-bit plans whose longest execute has more ring places than short ones ever need."""
+    n_time = 700
+    x = draw("ci4", n_time, n_chan, n_sta, seed=n_sta)
+    xd = torch.from_numpy(x).cuda()
+    with xcorr.Plan(n_sta, n_chan, max_time, fmt="ci4") as plan:
+        for unfused in (0, 1):
+            plan.set_tuning(4, 0, 2, unfused)
+            plan.execute(xd)
+            plan.execute(xd[:65].contiguous())
+            got = plan.dump().cpu().numpy()
+            plan.sync()
+            if unfused == 0:
+                check("ci4", got, np.concatenate([x, x[:65]]), 2 * n_sta)
+                first = got
+            else:
+                assert np.array_equal(got, first)

@@ -559,9 +559,8 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
   const int plane_chans = (c.n_channels + pack - 1) / pack;
   ni_pad *= pack;
   const int exp_windows = (c.max_time_per_exec + xc::kTcWindowBF16 - 1) / xc::kTcWindowBF16;
-  // (+ 256: the drain reads a tile's 128 column exponents past the last row's ni_pad)
   const size_t exps_bytes = (engine == XCORR_ENGINE_TENSOR && c.fmt == XCORR_IN_CF32)
-                                ? (size_t)plane_chans * exp_windows * ni_pad * 2 + 256
+                                ? (size_t)plane_chans * exp_windows * ni_pad * 2
                                 : 0;
   const size_t all_planes = (size_t)plane_chans * ppc * (size_t)c.max_time_per_exec * ni_pad * elem_bytes;
   // Where the operands come from.  int8: decoded on chip, or planes of all channels.  Two or more 128-input

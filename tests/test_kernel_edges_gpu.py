@@ -640,3 +640,18 @@ def test_plans_of_very_long_executes(torch, n_sta, n_chan, max_time):
                 first = got
             else:
                 assert np.array_equal(got, first)
+
+
+@pytest.mark.parametrize("n_sta,n_chan,n_time", [(64, 5, 400), (50, 3, 385), (8, 9, 768), (65, 4, 300)])
+def test_float_plan_takes_its_planes_and_no_more(torch, n_sta, n_chan, n_time):
+    """The limit that planes of all channels (twelve bytes a sample of rows of a multiple of 16), one
+    exponent a window and input, the accumulator and the status words need."""
+    pad = (2 * n_sta + 15) // 16 * 16
+    windows = (n_time + 383) // 384
+    need = n_chan * (n_sta * (2 * n_sta + 1) * 8 + 12 * n_time * pad + 2 * windows * pad) + 256
+    x = draw("cf32", n_time, n_chan, n_sta, seed=n_sta)
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="cf32", hbm_budget_bytes=need) as plan:
+        assert plan.query()["device_bytes"] <= need
+        got = plan.execute_dump(torch.from_numpy(x).cuda()).cpu().numpy()
+        plan.sync()
+    check("cf32", got, x, 2 * n_sta)

@@ -592,9 +592,18 @@ xcorr_status xcorr_plan_create(xcorr_plan* out, const xcorr_config* cfg) {
     planes_bytes = piece > least ? piece : least;
   }
   if (pair) {
-    e = xc::pair_ring_layout(c.fmt, n_inputs, c.n_channels, c.max_time_per_exec, c.hbm_budget_bytes ? room : 0, &ring);
+    e = xc::pair_ring_layout(c.fmt, n_inputs, c.n_channels, c.max_time_per_exec, 0, &ring);
     if (e != cudaSuccess && e != cudaErrorNotSupported) return cuda_fail(e, "ring layout");
-    if (e == cudaErrorNotSupported) pair = false, ring = xc::PairRing{};
+    // Under a limit the ring is cut short only where all planes do not fit either: they take less than a
+    // ring of whole tiles and chunks where samples or channels are few.
+    const bool over = e == cudaSuccess && c.hbm_budget_bytes && ring.bytes + ring.flag_bytes > room;
+    if (e == cudaErrorNotSupported || (over && planes_fit)) {
+      pair = false;
+      ring = xc::PairRing{};
+    } else if (over) {
+      e = xc::pair_ring_layout(c.fmt, n_inputs, c.n_channels, c.max_time_per_exec, room, &ring);
+      if (e != cudaSuccess) return cuda_fail(e, "ring layout");
+    }
     planes_bytes = pair ? ring.bytes : all_planes;
     if (pair && c.fmt == XCORR_IN_CI4 && row_bytes % 16 != 0) {
       const size_t left = room > ring.flag_bytes ? room - ring.flag_bytes : 0;

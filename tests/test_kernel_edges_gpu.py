@@ -655,3 +655,24 @@ def test_float_plan_takes_its_planes_and_no_more(torch, n_sta, n_chan, n_time):
         got = plan.execute_dump(torch.from_numpy(x).cuda()).cpu().numpy()
         plan.sync()
     check("cf32", got, x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time", [("ci4", 169, 24, 513), ("ci4", 65, 1, 100), ("ci4", 99, 40, 700), ("ci4", 136, 3, 130), ("cf32", 65, 1, 100),
+                                                     ("cf32", 256, 48, 2048), ("ci8", 65, 3, 100), ("ci8", 201, 9, 1000)])
+def test_plan_at_the_limit_of_all_its_planes(torch, fmt, n_sta, n_chan, n_time):
+    """Whatever the route, a plan is made where planes of all channels, the accumulator, the exponents
+    and the status words fit, and it stays within that."""
+    pad = (2 * n_sta + 15) // 16 * 16
+    bytes_per = {"ci4": 2, "ci8": 4, "cf32": 12}[fmt]
+    need = n_chan * (n_sta * (2 * n_sta + 1) * 8 + bytes_per * n_time * pad) + 256
+    if fmt == "cf32":
+        need += n_chan * 2 * pad * ((n_time + 383) // 384)
+    x = draw(fmt, n_time, n_chan, n_sta, seed=n_sta)
+    xd = torch.from_numpy(x).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor", hbm_budget_bytes=need) as plan:
+        assert plan.query()["device_bytes"] <= need
+        for unfused in (0, 1):
+            plan.set_tuning(4, 0, 2, unfused)
+            got = plan.execute_dump(xd).cpu().numpy()
+            plan.sync()
+            check(fmt, got, x, 2 * n_sta)

@@ -4,7 +4,10 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <array>
 #include <cstdint>
+#include <map>
+#include <mutex>
 #include <string>
 
 #include "xcorr.h"
@@ -147,6 +150,32 @@ struct xcorr_plan_s {
 };
 
 namespace xc {
+
+// N numbers of each device, made on first use by one thread while others wait (every plan has its own
+// host thread; two of them may make or run their first plans at once, on the same device or on two).
+template <int N>
+class PerDevice {
+ public:
+  // make(out): fills out for the current device.
+  template <typename Make>
+  cudaError_t get(std::array<int, N>* out, Make make) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu_);
+    const auto it = made_.find(dev);
+    if (it != made_.end()) {
+      *out = it->second;
+      return cudaSuccess;
+    }
+    if ((e = make(*out)) == cudaSuccess) made_[dev] = *out;
+    return e;
+  }
+
+ private:
+  std::mutex mu_;
+  std::map<int, std::array<int, N>> made_;
+};
 
 // Launch a kernel that calls pdl_wait so that its start overlaps the tail of the stream's previous
 // kernel (about 2 us per call on small problems: the launch latency, barrier and tensor-memory setup).

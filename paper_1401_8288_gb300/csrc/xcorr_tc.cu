@@ -566,14 +566,14 @@ cudaError_t launch_variant(const CUtensorMap* tmap, const TcParams& p, int grid,
 // CTAs that share the blocks of one of `items` float tiles: the most of 1, 2, 4, 8 that keep a CTA on an
 // SM of its own and whose clusters all fit the chip at once (a cluster lies within one GPC).
 int tc_float_split(int64_t items, int n_blocks, int num_sms) {
-  static int device = -1, most[4] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-  if (device != dev) {
+  static PerDevice<4> fitting;  // clusters of 1 << k CTAs that run at the same time
+  std::array<int, 4> most{};
+  const cudaError_t e = fitting.get(&most, [](std::array<int, 4>& m) {
     constexpr int V = 0;
     using G = Geometry<2, stage_rows_of(V, 2), stages_of(V)>;
     auto kern = xcorr_tc_kernel<2, stage_rows_of(V, 2), stages_of(V), true, false, true, false>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmemBytes) != cudaSuccess) return 1;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmemBytes);
+    if (e != cudaSuccess) return e;
     for (int k = 1; k < 4; ++k) {
       cudaLaunchConfig_t cfg{};
       cfg.gridDim = dim3(8 * 512);
@@ -585,13 +585,14 @@ int tc_float_split(int64_t items, int n_blocks, int num_sms) {
       attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&most[k], kern, &cfg) != cudaSuccess) {
-        most[k] = 0;
+      if (cudaOccupancyMaxActiveClusters(&m[k], kern, &cfg) != cudaSuccess) {
+        m[k] = 0;
         cudaGetLastError();
       }
     }
-    device = dev;
-  }
+    return cudaSuccess;
+  });
+  if (e != cudaSuccess) return 1;
   int split = 1;
   for (int k = 1; k < 4; ++k)
     if (items << k <= num_sms && items <= most[k] && 1 << k <= n_blocks) split = 1 << k;

@@ -856,25 +856,21 @@ template <int FMT, bool ADD>
 cudaError_t pair_clusters(int* n) {
   using G = Geom<FMT>;
   auto kern = xcorr_tc_pair_kernel<FMT, ADD>;
-  static int attr_device = -1, max_clusters = 0;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (attr_device != dev) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmem);
+  static PerDevice<1> most;
+  std::array<int, 1> clusters{};
+  const cudaError_t e = most.get(&clusters, [kern](std::array<int, 1>& m) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmem);
     if (e != cudaSuccess) return e;
     // pairs of SMs that can hold one CTA each at the same time
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * 1024);
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = G::kSmem;
-    e = cudaOccupancyMaxActiveClusters(&max_clusters, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (max_clusters < 1) return cudaErrorLaunchOutOfResources;
-    attr_device = dev;
-  }
-  *n = max_clusters;
-  return cudaSuccess;
+    e = cudaOccupancyMaxActiveClusters(&m[0], kern, &cfg);
+    return e == cudaSuccess && m[0] < 1 ? cudaErrorLaunchOutOfResources : e;
+  });
+  *n = clusters[0];
+  return e;
 }
 
 template <int FMT, bool ADD>

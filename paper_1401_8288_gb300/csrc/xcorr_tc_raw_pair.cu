@@ -417,24 +417,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 template <bool ADD>
 cudaError_t launch_raw_pair(const CUtensorMap& map, const RParams& p, int num_sms, cudaStream_t stream) {
   auto kern = xcorr_tc_raw_pair_kernel<ADD>;
-  static int attr_device = -1, max_clusters = 0;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (attr_device != dev) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  static PerDevice<1> most;
+  std::array<int, 1> clusters{};
+  const cudaError_t e = most.get(&clusters, [kern](std::array<int, 1>& m) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (e != cudaSuccess) return e;
     // pairs of SMs that can hold one CTA each at the same time
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * 1024);
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmem;
-    e = cudaOccupancyMaxActiveClusters(&max_clusters, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (max_clusters < 1) return cudaErrorLaunchOutOfResources;
-    attr_device = dev;
-  }
-  int n_cl = max_clusters < num_sms / 2 ? max_clusters : num_sms / 2;
+    e = cudaOccupancyMaxActiveClusters(&m[0], kern, &cfg);
+    return e == cudaSuccess && m[0] < 1 ? cudaErrorLaunchOutOfResources : e;
+  });
+  if (e != cudaSuccess) return e;
+  int n_cl = clusters[0] < num_sms / 2 ? clusters[0] : num_sms / 2;
   if (n_cl < 1) n_cl = 1;
   if (p.n_items < n_cl) n_cl = p.n_items;
   return launch_dependent(kern, 2 * n_cl, kThreads, kSmem, stream, map, p);

@@ -1,6 +1,10 @@
 """Kernels and dispatch branches at the sizes where they can go wrong (tile and stage edges,
 remainders, the ends of their ranges), bit for bit against the oracle."""
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -8,6 +12,7 @@ import oracle
 from paper_1401_8288_gb300 import synth, xcorr
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -676,3 +681,48 @@ def test_plan_at_the_limit_of_all_its_planes(torch, fmt, n_sta, n_chan, n_time):
             got = plan.execute_dump(xd).cpu().numpy()
             plan.sync()
             check(fmt, got, x, 2 * n_sta)
+
+
+FIRST_PLANS = r"""
+import threading
+import numpy as np, torch
+import oracle
+from paper_1401_8288_gb300 import synth, xcorr
+xcorr.load()
+torch.zeros(1, device="cuda")
+sizes = [("cf32", 20, 9, 800), ("cf32", 64, 12, 400), ("ci8", 64, 20, 300), ("ci8", 130, 9, 200), ("cf32", 130, 8, 500), ("cf32", 8, 40, 900)]
+makers = {"ci8": (synth.uniform_ci8, oracle.FMT_CI8), "cf32": (synth.gaussian_cf32, oracle.FMT_CF32)}
+xs = [makers[f][0](t, c, s, seed=k) for k, (f, s, c, t) in enumerate(sizes)]
+xd = [torch.from_numpy(x).cuda() for x in xs]
+torch.cuda.synchronize()
+got, meet = [None] * len(sizes), threading.Barrier(len(sizes))
+def work(k):
+    f, s, c, t = sizes[k]
+    stream = torch.cuda.Stream()
+    meet.wait()
+    with torch.cuda.stream(stream):
+        plan = xcorr.Plan(s, c, t, fmt=f, engine="tensor")
+        out = plan.execute_dump(xd[k])
+        plan.sync()
+        got[k] = out.cpu().numpy()
+threads = [threading.Thread(target=work, args=(k,)) for k in range(len(sizes))]
+[t.start() for t in threads]
+[t.join() for t in threads]
+for k, (f, s, c, t) in enumerate(sizes):
+    want = oracle.correlate(makers[f][1], xs[k])
+    if f == "ci8":
+        assert np.array_equal(got[k].astype(np.int64), want), sizes[k]
+    else:
+        i = np.arange(2 * s)
+        autos = want[:, i * (i + 1) // 2 + i, 0]
+        ii, jj = np.tril_indices(2 * s)
+        err = np.abs((got[k][..., 0] - want[..., 0]) + 1j * (got[k][..., 1] - want[..., 1]))
+        assert (err <= 1e-6 * np.sqrt(autos[:, ii] * autos[:, jj])).all(), sizes[k]
+print("alike")
+"""
+
+
+def test_first_plans_of_several_threads(torch):
+    """The first plans of a process, made and run by threads that start together."""
+    r = subprocess.run([sys.executable, "-c", FIRST_PLANS], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip().endswith("alike"), r.stdout + r.stderr

@@ -609,7 +609,8 @@ def our_arm(args) -> int:
                  else "xcorr_tc_fused_kernel") if fused else "xcorr_tc_kernel" if launches_per_step > 1
                 else "xcorr_tc_raw_pair_kernel" if fmt == "ci8" else "xcorr_tc_pair_kernel")
     one_launch = fused or launches_per_step == 1  # else unpack + X per channel group
-    x_launches = launches_per_step if one_launch else launches_per_step // 2
+    # (a fused execute may clear the output by a kernel of its own; one X launch per 37,248 samples)
+    x_launches = -(-n_time // 37248) if fused else launches_per_step if one_launch else launches_per_step // 2
     out_dtype = torch.float32 if fmt == "cf32" else torch.int32
     out = torch.empty((n_chan, n_pairs, 2), dtype=out_dtype, device=dev)
 

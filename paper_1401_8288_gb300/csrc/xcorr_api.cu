@@ -191,7 +191,6 @@ bool staged_execute(xcorr_plan plan, const void* d_in, int n_time) {
 struct Pieces {
   int pitch = 0;  // inputs from one row to the next; 0: does not apply
   int nc = 0, nt = 0;
-  int count = 0;
 };
 // At most a GB at a time.  A piece that stays in the L2 saves less than it costs in waves of the X
 // kernel that are not full and in launches (510 inputs x 400 channels x 2048 4-bit samples with pieces
@@ -219,13 +218,11 @@ Pieces repitch_pieces(xcorr_plan plan, int n_time) {
       const int whole = static_cast<int>(static_cast<int64_t>(r.nc) * per_chan / wave * wave / per_chan);
       if (whole > 0) r.nc = whole;
     }
-    r.count = (C + r.nc - 1) / r.nc;
     r.nt = n_time;
   } else {  // a long integration: one channel, whole stages of samples at a time
     r.nc = 1;
     r.nt = static_cast<int>(rows / 128 * 128);
     if (r.nt == 0) return r;  // (4-bit under a tight memory limit: the ring of planes)
-    r.count = C * ((n_time + r.nt - 1) / r.nt);
   }
   r.pitch = static_cast<int>(fmt == XCORR_IN_CI4 ? row : row / 2);
   return r;
@@ -264,6 +261,22 @@ cudaError_t run_repitched(xcorr_plan plan, const Pieces& r, const void* d_in, in
     }
   }
   return cudaSuccess;
+}
+
+// The kernels that run_repitched launches for a storing execute of the plan's channels.
+int repitched_launches(xcorr_plan plan, const Pieces& r, int n_time) {
+  const int C = plan->cfg.n_channels, shape = padded_shape(plan->tune_variant);
+  int n = 0;
+  for (int t0 = 0; t0 < n_time; t0 += r.nt) {
+    const int nt = n_time - t0 < r.nt ? n_time - t0 : r.nt;
+    for (int c0 = 0; c0 < C; c0 += r.nc) {
+      const int nc = C - c0 < r.nc ? C - c0 : r.nc;
+      n += 1 + (plan->cfg.fmt != XCORR_IN_CI4 ? 1
+                : t0 > 0 ? (nt + xc::kFusedWindowCI4 - 1) / xc::kFusedWindowCI4
+                         : xc::fused_ta_launches(shape, nt, nc, plan->n_inputs, r.pitch, plan->num_sms));
+    }
+  }
+  return n;
 }
 
 // Unpack channels [c0, c0 + nc) of the input into the plan's planes.
@@ -935,8 +948,9 @@ xcorr_status xcorr_plan_query(xcorr_plan plan, xcorr_plan_info* info) {
   // (int8: a 16-byte aligned input, nullptr standing for one)
   const bool raw = !plan->staged_ci8 && raw_ci8_applies(plan, nullptr), one_launch = plan->pair || raw;
   const Pieces pieces = fused || raw || plan->staged_ci8 ? Pieces{} : repitch_pieces(plan, plan->cfg.max_time_per_exec);
-  info->kernels_per_execute = fused ? xc::fused_launches(plan->cfg.max_time_per_exec)
-                              : pieces.pitch ? pieces.count * (1 + (plan->cfg.fmt == XCORR_IN_CI4 ? xc::fused_launches(pieces.nt) : 1))
+  info->kernels_per_execute = fused ? xc::fused_launches(plan->tune_variant, plan->cfg.max_time_per_exec, plan->cfg.n_channels,
+                                                         plan->n_inputs, plan->num_sms)
+                              : pieces.pitch ? repitched_launches(plan, pieces, plan->cfg.max_time_per_exec)
                               : one_launch                          ? 1
                               : plan->engine == XCORR_ENGINE_TENSOR ? 2 * tensor_groups(plan)
                                                                      : 1;

@@ -337,7 +337,9 @@ bool encode_raw_ci4_packed_tmap(CUtensorMap* map, const void* in, int n_inputs, 
 // The fused 4-bit X kernel (unpack on chip, offset-binary operands): one
 // launch per kFusedWindowCI4 samples; n_inputs % 16 == 0, `in` 16-byte aligned.
 int fused_stage_samples(int variant);
-int fused_launches(int n_time);
+// Kernel launches of a storing call, the clearing of an output that split tiles add into among them.
+int fused_launches(int variant, int n_time, int n_chan, int n_inputs, int num_sms);
+int fused_ta_launches(int variant, int n_time, int n_chan, int n_inputs, int pitch, int num_sms);
 // `in` points at the first of n_chan channels; time rows hold row_chans channels.
 // Variants 0-3 decode both operands into shared memory; 4-6 run the kernel
 // with the A operand in tensor memory (its variants 0-2); 7-9 run the CTA-pair

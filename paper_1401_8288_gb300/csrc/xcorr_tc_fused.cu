@@ -486,7 +486,11 @@ int fused_stage_samples(int variant) {
   return variant == 0 ? 128 : variant == 2 ? 64 : 96;
 }
 
-int fused_launches(int n_time) { return n_time <= 0 ? 0 : (n_time + kFusedWindowCI4 - 1) / kFusedWindowCI4; }
+int fused_launches(int variant, int n_time, int n_chan, int n_inputs, int num_sms) {
+  if (variant == 10 || (variant >= 4 && variant < 7))
+    return fused_ta_launches(variant == 10 ? 3 : variant - 4, n_time, n_chan, n_inputs, n_inputs, num_sms);
+  return (n_time + kFusedWindowCI4 - 1) / kFusedWindowCI4;
+}
 
 cudaError_t launch_xcorr_tc_fused_ci4(const uint8_t* in, int row_chans, int variant, int n_time, int n_chan,
                                       int n_inputs, int2* out, bool accumulate, int* status, int num_sms,

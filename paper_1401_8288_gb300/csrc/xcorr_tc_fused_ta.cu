@@ -832,6 +832,28 @@ void split_tail(int tiles, int num_sms, TParams& p) {
   p.n_split = (p.n_kt + kt - 1) / kt;
 }
 
+// One launch over `len` samples: how its tiles are cut into items.
+void cut_items(TParams& p, int len, int kt, bool small, int n_chan, int pitch, bool accumulate, int num_sms) {
+  p.n_kt = (len + kt - 1) / kt;
+  p.accumulate = accumulate ? 1 : 0;
+  int pack_g = 1, tiles = n_chan * p.n_tile_pairs;
+  p.n_split = 1;
+  p.split_kt = p.n_kt;
+  if (small) small_layout(n_chan, pitch, p.n_kt, num_sms, pack_g, tiles, p.n_split, p.split_kt);
+  p.tail_first = 0;
+  if (kt == 128 && pack_g == 1 && p.n_split == 1 && !accumulate) split_tail(tiles, num_sms, p);
+  p.atomic_out = p.n_split > 1 ? 1 : 0;
+  p.n_items = p.tail_first + (tiles - p.tail_first) * p.n_split;
+}
+
+int fused_ta_launches(int variant, int n_time, int n_chan, int n_inputs, int pitch, int num_sms) {
+  const int kt = fused_ta_stage_samples(variant), nb = (n_inputs + kBlk - 1) / kBlk;
+  TParams p{};
+  p.n_tile_pairs = nb * (nb + 1) / 2;
+  cut_items(p, n_time < kFusedWindowCI4 ? n_time : kFusedWindowCI4, kt, variant == 3, n_chan, pitch, false, num_sms);
+  return (n_time + kFusedWindowCI4 - 1) / kFusedWindowCI4 + (p.atomic_out ? 1 : 0);  // (the first may clear the output)
+}
+
 cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int variant, int n_time, int n_chan,
                                          int n_inputs, int pitch, int2* out, bool accumulate, int* status,
                                          int num_sms, cudaStream_t stream) {
@@ -867,16 +889,7 @@ cudaError_t launch_xcorr_tc_fused_ta_ci4(const uint8_t* in, int row_chans, int v
   for (int t0 = 0; t0 < n_time; t0 += kFusedWindowCI4) {
     const int len = n_time - t0 < kFusedWindowCI4 ? n_time - t0 : kFusedWindowCI4;
     p.t0 = t0;
-    p.n_kt = (len + kt - 1) / kt;
-    p.accumulate = (accumulate || t0 > 0) ? 1 : 0;
-    int tiles = n_chan * p.n_tile_pairs;
-    p.n_split = 1;
-    p.split_kt = p.n_kt;
-    if (small) small_layout(n_chan, pitch, p.n_kt, num_sms, pack_g, tiles, p.n_split, p.split_kt);
-    p.tail_first = 0;
-    if (kt == 128 && pack_g == 1 && p.n_split == 1 && !p.accumulate) split_tail(tiles, num_sms, p);
-    p.atomic_out = p.n_split > 1 ? 1 : 0;
-    p.n_items = p.tail_first + (tiles - p.tail_first) * p.n_split;
+    cut_items(p, len, kt, small, n_chan, pitch, accumulate || t0 > 0, num_sms);
     if (p.atomic_out && !p.accumulate) {  // the split items add into a cleared output (the whole tiles of their channels overwrite theirs)
       const int c0 = pack_g > 1 ? 0 : p.tail_first / p.n_tile_pairs;
       cudaError_t e = launch_clear(out + c0 * p.n_pairs, (n_chan - c0) * p.n_pairs, stream);

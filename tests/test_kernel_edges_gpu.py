@@ -726,3 +726,44 @@ def test_first_plans_of_several_threads(torch):
     """The first plans of a process, made and run by threads that start together."""
     r = subprocess.run([sys.executable, "-c", FIRST_PLANS], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip().endswith("alike"), r.stdout + r.stderr
+
+
+def kernels_of(torch, call):
+    """Kernel nodes of a captured call."""
+    import ctypes
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    rt = ctypes.CDLL("libcudart.so.13")
+    n = ctypes.c_size_t()
+    raw = ctypes.c_void_p(graph.raw_cuda_graph())
+    assert rt.cudaGraphGetNodes(raw, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert rt.cudaGraphGetNodes(raw, nodes, ctypes.byref(n)) == 0
+    kinds = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append(kind.value)
+    return kinds.count(0)  # cudaGraphNodeTypeKernel
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time,variant", [
+    ("ci4", 8, 16, 256, 10), ("ci4", 32, 64, 1024, 10), ("ci4", 64, 40, 3300, 4), ("ci4", 64, 153, 2700, 4), ("ci4", 64, 153, 2700, 0),
+    ("ci4", 128, 16, 700, 7), ("ci4", 29, 5, 700, 10), ("ci4", 70, 20, 4100, 4), ("ci4", 16, 3, 40000, 10), ("ci4", 20, 3, 40000, 4),
+    ("ci8", 64, 20, 300, 0), ("ci8", 33, 200, 300, 0), ("ci8", 70, 20, 1024, 0), ("cf32", 64, 20, 800, 0), ("cf32", 130, 100, 300, 0),
+    ("cf32", 256, 64, 2048, 0)])
+def test_kernels_per_execute(torch, fmt, n_sta, n_chan, n_time, variant):
+    """The count that the plan gives is what a storing execute launches."""
+    x = torch.zeros((n_time * n_chan * n_sta * 2 * {"ci4": 1, "ci8": 2, "cf32": 8}[fmt],), dtype=torch.uint8, device="cuda")
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor") as plan:
+        plan.set_tuning(variant, 0, 2, 0)
+        out = torch.empty((n_chan, plan.info["n_pairs"], 2), dtype=torch.float32 if fmt == "cf32" else torch.int32, device="cuda")
+
+        def call():
+            xcorr.xcorr_execute_dump(plan.handle, x.data_ptr(), n_time, out.data_ptr(), True, xcorr.XCORR_DUMP_RESET,
+                                     torch.cuda.current_stream().cuda_stream)
+
+        call()
+        plan.sync()
+        assert kernels_of(torch, call) == plan.query()["kernels_per_execute"]

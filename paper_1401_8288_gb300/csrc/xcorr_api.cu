@@ -1014,7 +1014,8 @@ xcorr_status xcorr_autotune(xcorr_plan plan, const void* d_in, int n_time, void*
         if (uf == 0 && (gi > 0 || xs > 1)) continue;      // the fused kernel is one launch
         if (uf == 0 && padded_ci4 && padded_shape(v) != v - 4 && v != xc::kSmallFusedVariant) continue;
         // the CTA-pair kernels have one shape each
-        if (uf == 1 && (plan->pair || (plan->cfg.fmt == XCORR_IN_CI8 && !plan->staged_ci8)) && (v > 0 || gi > 0)) continue;
+        if (uf == 1 && (plan->pair || (plan->cfg.fmt == XCORR_IN_CI8 && !staged_execute(plan, d_in, n_time))) && (v > 0 || gi > 0)) continue;
+        if (uf == 1 && plan->pack > 1 && v > 0) continue;  // nor have packed channels another
         plan->tune_variant = v;
         plan->tune_groups = group_choices[gi];
         plan->tune_x_streams = xs;

@@ -767,3 +767,16 @@ def test_kernels_per_execute(torch, fmt, n_sta, n_chan, n_time, variant):
         call()
         plan.sync()
         assert kernels_of(torch, call) == plan.query()["kernels_per_execute"]
+
+
+@pytest.mark.parametrize("n_sta,n_chan,n_time", [(4, 60, 400), (16, 200, 800), (32, 300, 385)])
+def test_autotune_of_packed_float_channels(torch, n_sta, n_chan, n_time):
+    """Packed channels have one launch shape: the tuner does not choose among names for it."""
+    x = torch.from_numpy(draw("cf32", n_time, n_chan, n_sta, seed=1)).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="cf32") as plan:
+        for _ in range(4):
+            plan.set_tuning(2, 0, 2, 0)
+            shape, ms = plan.autotune(x)
+            assert shape["stage_variant"] == 0 and ms > 0
+        check("cf32", plan.execute_dump(x).cpu().numpy(), x.cpu().numpy(), 2 * n_sta)
+        plan.sync()

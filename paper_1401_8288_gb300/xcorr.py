@@ -708,19 +708,23 @@ class Plan:
                       self._stream(stream))
 
     def dump(self, out=None, reset: bool = True, wide: bool = False, stream=None):
-        torch = self._torch
-        shape = (self.n_channels, self.info["n_pairs"], 2)
         new = out is None
-        if new:  # (every entry is written)
-            out = torch.empty(shape, dtype=self._out_dtype(wide), device="cuda")
+        if new:
+            out = self._new_output(wide)
         if new and wide:
-            self.samples = _dump_wide_new(self.handle, out.data_ptr(), XCORR_DUMP_RESET if reset else 0,
-                                          self._stream(stream))
-            return out
+            return self._dump_wide_into(out, reset, stream)
         flags = (XCORR_DUMP_RESET if reset else 0) | (XCORR_DUMP_ADD_WIDE if wide else 0)
         self.samples = xcorr_dump(self.handle, out.data_ptr(), out.is_cuda, flags,
                                   self._stream(stream))
         return out
+
+    def _new_output(self, wide: bool):
+        """(Not cleared: every entry is written.)"""
+        return self._torch.empty((self.n_channels, self.info["n_pairs"], 2), dtype=self._out_dtype(wide), device="cuda")
+
+    def _dump_wide_into(self, new, reset: bool, stream):
+        self.samples = _dump_wide_new(self.handle, new.data_ptr(), XCORR_DUMP_RESET if reset else 0, self._stream(stream))
+        return new
 
     def accum_load(self, src, n_samples: int, stream=None):
         """Resume an integration from a dump taken with reset=False: src is that dump (a host or
@@ -733,14 +737,14 @@ class Plan:
 
     def execute_dump(self, x, out=None, reset: bool = True, wide: bool = False, stream=None):
         """execute(x) then dump(...), fused into one pass when x is the whole integration."""
-        torch = self._torch
         if not x.is_cuda or not x.is_contiguous():
             raise ValueError("input must be a contiguous CUDA tensor")
-        if out is None and wide:  # (the two calls that a wide xcorr_execute_dump is)
+        new = out is None
+        if new:  # (before anything is integrated: without memory for it the call changes nothing)
+            out = self._new_output(wide)
+        if new and wide:  # (the two calls that a wide xcorr_execute_dump is)
             self.execute(x, stream=stream)
-            return self.dump(reset=reset, wide=True, stream=stream)
-        if out is None:
-            out = torch.empty((self.n_channels, self.info["n_pairs"], 2), dtype=self._out_dtype(wide), device="cuda")
+            return self._dump_wide_into(out, reset, stream)
         flags = (XCORR_DUMP_RESET if reset else 0) | (XCORR_DUMP_ADD_WIDE if wide else 0)
         self.samples = xcorr_execute_dump(self.handle, x.data_ptr(), x.shape[0], out.data_ptr(),
                                           out.is_cuda, flags, self._stream(stream))

@@ -780,3 +780,19 @@ def test_autotune_of_packed_float_channels(torch, n_sta, n_chan, n_time):
             assert shape["stage_variant"] == 0 and ms > 0
         check("cf32", plan.execute_dump(x).cpu().numpy(), x.cpu().numpy(), 2 * n_sta)
         plan.sync()
+
+
+@pytest.mark.parametrize("wide", [False, True])
+def test_execute_dump_without_memory_for_the_output(torch, wide, monkeypatch):
+    """A call that cannot make its output has not integrated the samples."""
+    n_sta, n_chan, n_time = 8, 3, 100
+    x = torch.from_numpy(draw("ci4", n_time, n_chan, n_sta, seed=1)).cuda()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt="ci4") as plan:
+        with monkeypatch.context() as m:
+            m.setattr(plan._torch, "empty", lambda *a, **k: (_ for _ in ()).throw(torch.OutOfMemoryError("no memory")))
+            with pytest.raises(torch.OutOfMemoryError):
+                plan.execute_dump(x, wide=wide)
+        assert plan.query()["samples_integrated"] == 0
+        got = plan.execute_dump(x, wide=wide).cpu().numpy()
+        plan.sync()
+    check("ci4", got, x.cpu().numpy(), 2 * n_sta)

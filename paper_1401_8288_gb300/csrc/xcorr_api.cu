@@ -882,6 +882,11 @@ xcorr_status xcorr_execute_dump_host(xcorr_plan plan, const void* h_in, int n_ti
     int edge[xc::kMaxGroups + 1];  // group g: channels edge[g] .. edge[g + 1] - 1
     const int G = n_groups > 0 ? even_groups(C, n_groups, edge)
                                : host_groups(C, row_bytes * n_time + out_chan_bytes * C, edge);
+    // timed as other executes: no unpack, a launch (or a piece's two) per group
+    cudaEvent_t* ev = plan->prof_cap && !fused ? plan->prof_events + xc::kProfileEvents * (plan->prof_count % plan->prof_cap) : nullptr;
+    if (ev && ((e = cudaEventRecord(ev[0], s)) != cudaSuccess || (e = cudaEventRecord(ev[1], s)) != cudaSuccess))
+      return cuda_fail(e, "profile event");
+    int timed = 0;
     if ((e = cudaEventRecord(plan->ev_fork, s)) != cudaSuccess) return cuda_fail(e, "fork event");
     for (cudaStream_t t : {plan->s_unpack, plan->s_x[0], plan->s_x[1], plan->s_down})
       if ((e = cudaStreamWaitEvent(t, plan->ev_fork, 0)) != cudaSuccess) return cuda_fail(e, "fork wait");
@@ -896,17 +901,24 @@ xcorr_status xcorr_execute_dump_host(xcorr_plan plan, const void* h_in, int n_ti
           (e = cudaEventRecord(plan->ev_up[g], plan->s_unpack)) != cudaSuccess ||
           (e = cudaStreamWaitEvent(sx, plan->ev_up[g], 0)) != cudaSuccess)
         return cuda_fail(e, "group input copy");
+      if (ev && (e = cudaEventRecord(ev[2 + 2 * timed], sx)) != cudaSuccess) return cuda_fail(e, "profile event");
       e = fused ? xc::launch_xcorr_tc_fused_ci4(stage + off, C, plan->tune_variant, n_time, c1 - c0, N, out_g, false,
                                                 plan->status, plan->num_sms, sx)
           : raw ? xc::launch_xcorr_tc_raw_pair(reinterpret_cast<const int8_t*>(stage + off), C, n_time, c1 - c0, N, N, out_g,
                                                false, plan->status, plan->num_sms, sx)
                 : run_repitched(plan, pieces, stage + off, c1 - c0, n_time, out_g, true, sx);
       if (e != cudaSuccess) return cuda_fail(e, "X kernel launch");
+      if (ev && (e = cudaEventRecord(ev[3 + 2 * timed], sx)) != cudaSuccess) return cuda_fail(e, "profile event");
+      ++timed;
       if ((e = cudaEventRecord(plan->ev_group_done[g], sx)) != cudaSuccess ||
           (e = cudaStreamWaitEvent(plan->s_down, plan->ev_group_done[g], 0)) != cudaSuccess ||
           (e = cudaMemcpyAsync(static_cast<uint8_t*>(h_out) + out_chan_bytes * c0, out_g, out_chan_bytes * (c1 - c0),
                                cudaMemcpyDeviceToHost, plan->s_down)) != cudaSuccess)
         return cuda_fail(e, "group output copy");
+    }
+    if (ev) {
+      plan->prof_ngroups[plan->prof_count % plan->prof_cap] = timed;
+      ++plan->prof_count;
     }
     // join: every group's copy-out is on s_down, after its X launch and its input copy
     if ((e = cudaEventRecord(plan->ev_down, plan->s_down)) != cudaSuccess ||

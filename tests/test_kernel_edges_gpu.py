@@ -796,3 +796,18 @@ def test_execute_dump_without_memory_for_the_output(torch, wide, monkeypatch):
         got = plan.execute_dump(x, wide=wide).cpu().numpy()
         plan.sync()
     check("ci4", got, x.cpu().numpy(), 2 * n_sta)
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time,n_groups", [("ci8", 64, 20, 300, 0), ("ci8", 70, 20, 300, 3), ("ci4", 37, 20, 300, 8), ("cf32", 20, 5, 100, 0)])
+def test_host_executes_are_timed(torch, fmt, n_sta, n_chan, n_time, n_groups):
+    """Host-to-host executes of int8, float and padded rows leave their durations, each once."""
+    x = torch.from_numpy(draw(fmt, n_time, n_chan, n_sta, seed=1)).pin_memory()
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor") as plan:
+        xcorr.xcorr_profile_enable(plan.handle, 4)
+        for k in range(3):
+            plan.execute_dump_host(x, n_groups=n_groups)
+            plan.execute_dump(x.cuda())
+        plan.sync()
+        read = xcorr.xcorr_profile_read(plan.handle, 4)
+        xcorr.xcorr_profile_enable(plan.handle, 0)
+    assert len(read) == 4 and all(0 <= unpack < 10 and 0 < span < 10 for unpack, span in read)

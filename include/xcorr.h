@@ -234,7 +234,8 @@ xcorr_status xcorr_execute_dump(xcorr_plan plan, const void *d_in, int n_time, v
 /*
  * One whole integration from host memory to host memory, with the copies
  * overlapped with the X-stage: the channels are cut into n_groups groups (0 =
- * the library's choice, by the bytes that move); each group's input columns go up (a 2-D
+ * the library's choice, by the bytes that move, which is also the most for int8
+ * and padded rows; one group where either side is not pinned); each group's input columns go up (a 2-D
  * copy of its channels of every sample), are correlated, and its triangle
  * comes back while later groups are still being copied or correlated.  The
  * result equals copying the input to the device, xcorr_execute_dump with
@@ -243,7 +244,7 @@ xcorr_status xcorr_execute_dump(xcorr_plan plan, const void *d_in, int n_time, v
  * pinned (cudaHostAlloc / cudaHostRegister), or the copies do not overlap.  The
  * plan must hold no integration (nothing executed since the last reset) and
  * still holds none afterwards.  Input that is not decoded on chip (float, 4-bit
- * through planes, the CUDA-core engine) runs as one piece:
+ * and int8 through planes, the CUDA-core engine) runs as one piece:
  * the copy up, the X-stage and the copy down, in order.  The first call
  * allocates a device copy of one input (max_time_per_exec samples), kept
  * until xcorr_destroy.  Stream-ordered on `stream`.

@@ -318,6 +318,21 @@ int host_groups(int C, size_t bytes, int* edge) {
   return 4;
 }
 
+// Host memory that is not pinned.
+bool pageable(const void* p) {
+  cudaPointerAttributes a{};
+  return cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeUnregistered;
+}
+
+// The most groups of an int8 host execute.  However few its channels, a group's launch takes the time of one
+// channel's samples (0.0106 us each; padded rows share their memory, so one group after the other; else two
+// at a time): together no more than the way up at 200 GB/s.  (18 inputs x 64 channels x 14,563 samples: one
+// group 388 us, two 486, four 780.)
+int ci8_host_groups(size_t bytes, int n_time, bool two_streams) {
+  const double n = (two_streams ? 2 : 1) * (5e-6 * bytes) / (0.0106 * n_time);
+  return n < 1 ? 1 : n > xc::kMaxGroups ? xc::kMaxGroups : static_cast<int>(n);
+}
+
 // Correlate n_time samples into target (the plan's accumulator, or the
 // caller's buffer for a fused dump).  target_fresh: store instead of add.
 xcorr_status run_execute(xcorr_plan plan, const void* d_in, int n_time, void* target, bool target_fresh,
@@ -866,8 +881,9 @@ xcorr_status xcorr_execute_dump_host(xcorr_plan plan, const void* h_in, int n_ti
       }
   uint8_t* stage = static_cast<uint8_t*>(plan->host_stage);
   const size_t out_chan_bytes = static_cast<size_t>(plan->n_pairs) * 8;
-  const bool fused = plan->engine == XCORR_ENGINE_TENSOR && fused_applies(plan, stage), raw = raw_ci8_applies(plan, stage);
-  const Pieces pieces = fused || raw ? Pieces{} : repitch_pieces(plan, n_time);
+  const bool staged = staged_execute(plan, stage, n_time);
+  const bool fused = plan->engine == XCORR_ENGINE_TENSOR && fused_applies(plan, stage), raw = !staged && raw_ci8_applies(plan, stage);
+  const Pieces pieces = fused || raw || staged ? Pieces{} : repitch_pieces(plan, n_time);
   if (!fused && !raw && !pieces.pitch) {
     // one piece: up, X-stage, down, in order on the caller's stream
     if ((e = cudaMemcpyAsync(stage, h_in, row_bytes * n_time, cudaMemcpyHostToDevice, s)) != cudaSuccess)
@@ -880,8 +896,14 @@ xcorr_status xcorr_execute_dump_host(xcorr_plan plan, const void* h_in, int n_ti
     // launch can start on the SMs the previous one's tail leaves idle) and comes
     // down on s_down while later groups are still moving
     int edge[xc::kMaxGroups + 1];  // group g: channels edge[g] .. edge[g + 1] - 1
-    const int G = n_groups > 0 ? even_groups(C, n_groups, edge)
-                               : host_groups(C, row_bytes * n_time + out_chan_bytes * C, edge);
+    int G = host_groups(C, row_bytes * n_time + out_chan_bytes * C, edge);
+    int most = fused ? xc::kMaxGroups : G;  // (padded rows and int8: more groups than the library's choice only add launches)
+    if (plan->cfg.fmt == XCORR_IN_CI8) {
+      const int m = ci8_host_groups(row_bytes * n_time, n_time, raw);
+      if (m < most) most = m;
+    }
+    if (pageable(h_in) || pageable(h_out)) most = 1;  // (its copies overlap nothing, and narrow columns of it take longer)
+    if (n_groups > 0 || G > most) G = even_groups(C, n_groups > 0 && n_groups < most ? n_groups : most, edge);
     // timed as other executes: no unpack, a launch (or a piece's two) per group
     cudaEvent_t* ev = plan->prof_cap && !fused ? plan->prof_events + xc::kProfileEvents * (plan->prof_count % plan->prof_cap) : nullptr;
     if (ev && ((e = cudaEventRecord(ev[0], s)) != cudaSuccess || (e = cudaEventRecord(ev[1], s)) != cudaSuccess))
@@ -896,8 +918,10 @@ xcorr_status xcorr_execute_dump_host(xcorr_plan plan, const void* h_in, int n_ti
       const size_t off = chan_bytes * c0, width = chan_bytes * (c1 - c0);
       cudaStream_t sx = plan->s_x[pieces.pitch ? 0 : g & 1];  // (padded rows: one piece of memory)
       int2* out_g = static_cast<int2*>(plan->acc) + static_cast<int64_t>(c0) * plan->n_pairs;
-      if ((e = cudaMemcpy2DAsync(stage + off, row_bytes, static_cast<const uint8_t*>(h_in) + off, row_bytes, width,
-                                 n_time, cudaMemcpyHostToDevice, plan->s_unpack)) != cudaSuccess ||
+      // (all channels: one run of bytes, which the copy engines take faster than as rows)
+      if ((e = width == row_bytes ? cudaMemcpyAsync(stage, h_in, row_bytes * n_time, cudaMemcpyHostToDevice, plan->s_unpack)
+                                  : cudaMemcpy2DAsync(stage + off, row_bytes, static_cast<const uint8_t*>(h_in) + off, row_bytes,
+                                                      width, n_time, cudaMemcpyHostToDevice, plan->s_unpack)) != cudaSuccess ||
           (e = cudaEventRecord(plan->ev_up[g], plan->s_unpack)) != cudaSuccess ||
           (e = cudaStreamWaitEvent(sx, plan->ev_up[g], 0)) != cudaSuccess)
         return cuda_fail(e, "group input copy");

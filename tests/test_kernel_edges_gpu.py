@@ -811,3 +811,19 @@ def test_host_executes_are_timed(torch, fmt, n_sta, n_chan, n_time, n_groups):
         read = xcorr.xcorr_profile_read(plan.handle, 4)
         xcorr.xcorr_profile_enable(plan.handle, 0)
     assert len(read) == 4 and all(0 <= unpack < 10 and 0 < span < 10 for unpack, span in read)
+
+
+@pytest.mark.parametrize("n_groups", [0, 1, 5])
+@pytest.mark.parametrize("pinned", [(True, True), (False, False), (True, False), (False, True)])
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time", [("ci4", 64, 40, 4000), ("ci4", 37, 70, 700), ("ci8", 64, 40, 1000), ("ci8", 9, 64, 5000), ("ci8", 8, 64, 4096),
+                                                     ("cf32", 20, 9, 100)])
+def test_host_memory_that_is_not_pinned(torch, fmt, n_sta, n_chan, n_time, pinned, n_groups):
+    """Pageable memory on either side; int8 whose chains allow few groups, and through planes in one piece."""
+    x = draw(fmt, n_time, n_chan, n_sta, seed=n_time)
+    xt = torch.from_numpy(x)
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor") as plan:
+        shape, dtype = (n_chan, plan.info["n_pairs"], 2), torch.float32 if fmt == "cf32" else torch.int32
+        out = torch.full(shape, 3, dtype=dtype, pin_memory=pinned[1])
+        plan.execute_dump_host(xt.pin_memory() if pinned[0] else xt, out, n_groups=n_groups)
+        plan.sync()
+    check(fmt, out.numpy(), x, 2 * n_sta)

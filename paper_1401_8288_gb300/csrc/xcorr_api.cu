@@ -196,6 +196,9 @@ struct Pieces {
 // kernel that are not full and in launches (510 inputs x 400 channels x 2048 4-bit samples with pieces
 // of 64 / 96 / 256 MB / 1 GB: 605 / 556 / 522 / 510 us; 510 x 300 x 2048 int8: 807 / 771 / 740 / 725).
 constexpr size_t kPieceBytes = size_t(1) << 30;
+// (338 inputs x 20 channels x 1,500,000 4-bit samples in pieces of all samples of one channel or two 96 ms, of a
+// wave's channels 13; 512 x 97 x 100,000 at an odd address 49 and 7.6; int8 512 x 40 x 40,000 at one 19 and 2.4.)
+constexpr size_t kPieceSamples = 1024;
 constexpr size_t kOddAddressPieceBytes = size_t(64) << 20;  // kept by plans that need it at odd addresses only
 size_t padded_row_bytes(int fmt, int n_inputs) {
   return static_cast<size_t>((n_inputs * (fmt == XCORR_IN_CI4 ? 1 : 2) + 15) / 16) * 16;
@@ -209,20 +212,26 @@ Pieces repitch_pieces(xcorr_plan plan, int n_time) {
   const size_t row = padded_row_bytes(fmt, plan->n_inputs);
   const size_t room = plan->planes_bytes < kPieceBytes ? plan->planes_bytes : kPieceBytes;
   const size_t rows = room / row;  // of one channel and sample each
-  if (rows >= static_cast<size_t>(n_time)) {
-    r.nc = rows / n_time < static_cast<size_t>(C) ? static_cast<int>(rows / n_time) : C;
-    if (r.nc < C) {  // several pieces: whole waves of the X kernel where a piece holds one
-      const int nb = (plan->n_inputs + 127) / 128;
-      const int per_chan = fmt == XCORR_IN_CI4 ? nb * (nb + 1) / 2 : xc::raw_pair_items(nb);
-      const int wave = fmt == XCORR_IN_CI4 ? plan->num_sms : plan->num_sms / 2;
-      const int whole = static_cast<int>(static_cast<int64_t>(r.nc) * per_chan / wave * wave / per_chan);
-      if (whole > 0) r.nc = whole;
-    }
-    r.nt = n_time;
-  } else {  // a long integration: one channel, whole stages of samples at a time
-    r.nc = 1;
-    r.nt = static_cast<int>(rows / 128 * 128);
-    if (r.nt == 0) return r;  // (4-bit under a tight memory limit: the ring of planes)
+  const int nb = (plan->n_inputs + 127) / 128;
+  const int per_chan = fmt == XCORR_IN_CI4 ? nb * (nb + 1) / 2 : xc::raw_pair_items(nb);
+  const int wave = fmt == XCORR_IN_CI4 ? plan->num_sms : plan->num_sms / 2;
+  const int full = wave / per_chan < 1 ? 1 : wave / per_chan < C ? wave / per_chan : C;  // channels of a full wave
+  r.nt = n_time;
+  if (rows / full < static_cast<size_t>(n_time)) {
+    // A long integration: stages of samples at a time rather than channels that leave SMs idle.  Every
+    // piece of them after the first adds into the visibilities, so a piece has kPieceSamples of them
+    // where the memory holds so many (4-bit: the fused kernel's own blocks, which add anyway).
+    const size_t fits = rows / full, block = fits >= xc::kFusedWindowCI4 && fmt == XCORR_IN_CI4 ? xc::kFusedWindowCI4 : 128;
+    size_t nt = fits < kPieceSamples ? kPieceSamples : fits;
+    if (nt > rows) nt = rows;
+    nt = nt / block * block;
+    if (nt == 0 && rows < static_cast<size_t>(n_time)) return r;  // (4-bit under a tight memory limit: the ring of planes)
+    if (nt > 0 && nt < static_cast<size_t>(n_time)) r.nt = static_cast<int>(nt);
+  }
+  r.nc = rows / r.nt < static_cast<size_t>(C) ? static_cast<int>(rows / r.nt) : C;
+  if (r.nc < C) {  // several pieces: whole waves of the X kernel where a piece holds one
+    const int whole = static_cast<int>(static_cast<int64_t>(r.nc) * per_chan / wave * wave / per_chan);
+    if (whole > 0) r.nc = whole;
   }
   r.pitch = static_cast<int>(fmt == XCORR_IN_CI4 ? row : row / 2);
   return r;

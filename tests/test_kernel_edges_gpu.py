@@ -827,3 +827,24 @@ def test_host_memory_that_is_not_pinned(torch, fmt, n_sta, n_chan, n_time, pinne
         plan.execute_dump_host(xt.pin_memory() if pinned[0] else xt, out, n_groups=n_groups)
         plan.sync()
     check(fmt, out.numpy(), x, 2 * n_sta)
+
+
+@pytest.mark.parametrize("fmt,n_sta,n_chan,n_time,offset,rows,least", [
+    ("ci8", 19, 90, 2500, 0, 76 * 256, 30), ("ci8", 21, 90, 2500, 0, 76 * 1100, 10), ("ci8", 64, 40, 1500, 2, 40 * 1100, 4), ("ci8", 20, 2, 300, 3, 128, 12),
+    ("ci8", 131, 30, 1400, 0, 25 * 1030, 8), ("ci4", 65, 3, 80000, 0, 3 * 40000, 6), ("ci4", 65, 60, 2600, 0, 50 * 1600, 6), ("ci4", 72, 40, 2600, 5, 40 * 1850, 4)])
+def test_long_padded_rows_in_pieces_of_samples(torch, fmt, n_sta, n_chan, n_time, offset, rows, least):
+    """Memory for fewer samples of a wave's channels than there are: pieces along time that add into the
+    first, whole stages or the fused kernel's blocks, with short last ones in both directions."""
+    row = (2 * n_sta * (1 if fmt == "ci4" else 2) + 15) // 16 * 16
+    budget = n_chan * n_sta * (2 * n_sta + 1) * 8 + 256 + 8192 + rows * row
+    x = draw(fmt, n_time, n_chan, n_sta, seed=rows)
+    buf = placed(torch, x, offset)
+    stream = torch.cuda.current_stream().cuda_stream
+    with xcorr.Plan(n_sta, n_chan, n_time, fmt=fmt, engine="tensor", hbm_budget_bytes=budget) as plan:
+        if offset == 0:
+            assert plan.query()["kernels_per_execute"] >= least
+        for _ in range(2):
+            xcorr.xcorr_execute(plan.handle, buf.data_ptr() + offset, n_time, stream)
+        got = plan.dump().cpu().numpy()
+        plan.sync()
+    check(fmt, got, np.concatenate([x, x]), 2 * n_sta)

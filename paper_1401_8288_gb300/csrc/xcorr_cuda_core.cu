@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256) xcorr_cc_kernel(const CcParams p) {
 
   uint32_t nr[4], ni[4];
   int buf = 0;
-  pdl_release();  // 16 inputs x 16 channels x 256 samples, call after call: 8.9 -> 8.3 us
+  pdl_release();  // (16 int8 inputs x 16 channels x 256 samples, call after call: 15.4 -> 13.5 us; 11.5 from a graph either way)
   pdl_wait();
   if (loads) {
     load_group<FMT>(p, c, t_begin + 4 * t4, t_end, base, aligned, nr, ni);
@@ -236,7 +236,6 @@ cudaError_t launch_xcorr_cuda_core(int fmt, const void* in, int n_time, int n_ch
   if (fmt == XCORR_IN_CI4)
     return launch_dependent(xcorr_cc_kernel<XCORR_IN_CI4>, (unsigned)blocks, 256, 0, stream, p);
   return launch_dependent(xcorr_cc_kernel<XCORR_IN_CI8>, (unsigned)blocks, 256, 0, stream, p);
-  return cudaGetLastError();
 }
 
 }  // namespace xc

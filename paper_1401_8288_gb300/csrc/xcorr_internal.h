@@ -70,7 +70,7 @@ constexpr int kProfileEvents = 2 + 2 * kMaxGroups;  // per timed execute
 // The whole tensor path in one launch on CTA pairs (xcorr_tc_pair.cu), for two or more 128-input
 // tiles: samples unpacked once into a ring of operand planes, correlated from it.
 constexpr int kTcPairMinTiles = 2;
-constexpr size_t kRingBytes = size_t(48) << 20;  // of the 129 MB L2
+constexpr size_t kRingBytes = size_t(48) << 20;  // (more where three steps of a batch are more)
 struct PairRing {
   int clusters = 0;      // CTA pairs of a launch
   int halves = 0;        // 64-input halves of a plane: two per tile

@@ -8,18 +8,19 @@
 //
 // The operands are planes of tensor-core numbers, [channel][plane][t][input]:
 //   * 4-bit samples: two E4M3 planes (re, im); every code in [-8, 7] is exact;
+//   * int8 samples: two BF16 planes, exact;
 //   * float samples: six BF16 planes of integer digits.  Per input and time
 //     window of W samples each component is quantised against the window's
 //     largest magnitude 2^E to a 23-bit integer M = d0 2^16 + d1 2^8 + d2
 //     with balanced digits |d_p| <= 128 (exact BF16 values); a product of two
 //     components is the sum of the digit products d_p d_q 2^(-8(p+q)) with
 //     p + q <= 2 (the dropped ones are below 2^-23 of the largest product).
-// The K axis runs over (time window, plane pair, stage): for 4-bit input a
-// single pair (the re/im planes against themselves), for float input
+// The K axis runs over (time window, plane pair, stage): for 4-bit and int8 input
+// a single pair (the re/im planes against themselves), for float input
 // the six digit pairs (p, q).  Each (window, pair) block is accumulated in
 // FP32 tensor memory and drained on its own: every partial sum of a block is
-// an integer of magnitude below 2^24 (at most 128 or 2 * 2^14 per sample for
-// 4-bit and digit products), so it is exact -- which matters
+// an integer of magnitude below 2^24 (at most 128 per sample for 4-bit, 2 * 2^14 for
+// int8 and digit products), so it is exact -- which matters
 // because the tensor core truncates each accumulation toward zero -- and the
 // drain converts it exactly to int32, or scales it by 2^(E_i + E_j - 12 -
 // 8(p + q)) and adds it (rounded to nearest) into a float accumulator.

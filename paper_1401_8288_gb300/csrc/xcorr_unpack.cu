@@ -353,13 +353,14 @@ cudaError_t launch_unpack_ci8_bf16(const int8_t* in, uint16_t* planes, int n_tim
 // ----------------------------------------------------- float input --
 namespace {
 
-// Float input read once: a CTA stages one (window, 16 columns) slice in shared memory -- a column is a
-// pair of neighbouring inputs of one channel, 16 bytes a sample; the slice is two units of 8 columns,
-// whose digits fill whole 32-byte sectors of the planes' rows (columns that ran on through the
-// channels of an input count that is no multiple of 16 took 494 us with the X kernel for 122 x 300 x
-// 1024, now 345; kernels that read the input twice, 595) -- by asynchronous copies, takes each input's window maximum from it, then writes the digits from it.  Two CTAs of 256
+// Float input read once: a CTA stages one (window, 16 columns) slice in shared memory by asynchronous
+// copies, takes each input's window maximum from it, then writes the digits from it.  Two CTAs of 256
 // threads share an SM, so one loads while the other converts.  Thread (column q, time group g) handles
 // samples g, g + 16, ...; a warp covers two time rows of 16 columns, conflict-free.
+// A column is a pair of neighbouring inputs of one channel, 16 bytes a sample.  A slice is two units of
+// 8 columns, whose digits fill whole 32-byte sectors of the planes' rows.  (122 inputs x 300 channels x
+// 1024 samples, with the X kernel: 345 us so; 494 with columns that run on through the channels; 595 with
+// kernels that read the input twice.)
 //
 // Bound by memory: 8 bytes read and 12 written per sample (128 inputs x 64 channels x 1024 samples: 40
 // us with conversion instructions for the digits, which run at an eighth of the ALU's rate, now 28).

@@ -275,17 +275,15 @@ cudaError_t run_repitched(xcorr_plan plan, const Pieces& r, const void* d_in, in
 // The kernels that run_repitched launches for a storing execute of the plan's channels.
 int repitched_launches(xcorr_plan plan, const Pieces& r, int n_time) {
   const int C = plan->cfg.n_channels, shape = padded_shape(plan->tune_variant);
-  int n = 0;
-  for (int t0 = 0; t0 < n_time; t0 += r.nt) {
-    const int nt = n_time - t0 < r.nt ? n_time - t0 : r.nt;
-    for (int c0 = 0; c0 < C; c0 += r.nc) {
-      const int nc = C - c0 < r.nc ? C - c0 : r.nc;
-      n += 1 + (plan->cfg.fmt != XCORR_IN_CI4 ? 1
-                : t0 > 0 ? (nt + xc::kFusedWindowCI4 - 1) / xc::kFusedWindowCI4
-                         : xc::fused_ta_launches(shape, nt, nc, plan->n_inputs, r.pitch, plan->num_sms));
-    }
-  }
-  return n;
+  const auto piece = [&](int nt, int nc, bool first) {
+    return 1 + (plan->cfg.fmt != XCORR_IN_CI4 ? 1
+                : first ? xc::fused_ta_launches(shape, nt, nc, plan->n_inputs, r.pitch, plan->num_sms)
+                        : (nt + xc::kFusedWindowCI4 - 1) / xc::kFusedWindowCI4);
+  };
+  const auto pieces = [&](int nt, bool first) {
+    return nt == 0 ? 0 : C / r.nc * piece(nt, r.nc, first) + (C % r.nc ? piece(nt, C % r.nc, first) : 0);
+  };
+  return pieces(r.nt, true) + (n_time / r.nt - 1) * pieces(r.nt, false) + pieces(n_time % r.nt, false);
 }
 
 // Unpack channels [c0, c0 + nc) of the input into the plan's planes.

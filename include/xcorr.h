@@ -145,7 +145,7 @@ typedef struct {
     int64_t max_integration;  /* most samples one integration may hold exactly in int32 */
     size_t device_bytes;      /* device memory the plan owns                             */
     size_t output_bytes;      /* bytes of one dump in the plan's own element type        */
-    int kernels_per_execute;  /* kernel launches of one full-size execute (unpack + X)   */
+    int kernels_per_execute;  /* kernel launches of one full-size storing execute       */
     xcorr_tuning tuning;      /* current launch shape (groups resolved)                  */
 } xcorr_plan_info;
 
